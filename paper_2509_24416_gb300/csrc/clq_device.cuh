@@ -87,12 +87,11 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // Wait for the phase of `bar` with the given parity to complete.  Gives up
 // after `limit_ns`, or as soon as *abort (shared memory) becomes non-zero;
 // on running out it records CLQ_ERR_TIMEOUT and raises *abort.  Returns
-// true when the phase completed.
-static __device__ __noinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity,
-                                               volatile int32_t* abort,
-                                               int32_t* status,
-                                               uint64_t limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
+// true when the phase completed.  The check that usually succeeds is inline;
+// only a wait that has to last calls the loop.
+static __device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity,
+                                                   volatile int32_t* abort, int32_t* status,
+                                                   uint64_t limit_ns) {
   const uint64_t t0 = global_timer_ns();
   while (true) {
 #pragma unroll 1
@@ -105,6 +104,29 @@ static __device__ __noinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t pa
       return false;
     }
   }
+}
+
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity,
+                                                  volatile int32_t* abort, int32_t* status,
+                                                  uint64_t limit_ns) {
+  if (mbar_try_wait(bar, parity)) return true;
+  return mbar_wait_slow(bar, parity, abort, status, limit_ns);
+}
+
+// True in one lane of a converged warp.  A branch on it tells the compiler
+// that a single thread goes on: the TMA and tcgen05 instructions inside then
+// take their operands from uniform registers directly, where a branch on
+// `lane == 0` costs a serialization per instruction (measured in the GEMM's
+// main loop alone, 128 x 256 tiles of four 48 KB stages: 793 clocks a K step
+// with lane == 0, 599 with this; the E4M3 MMAs of a step take 542).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
 }
 
 // ------------------------------------------------------------------ TMA ---

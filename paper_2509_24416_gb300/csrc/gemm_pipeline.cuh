@@ -206,19 +206,21 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
   const int tiles = ((g.M + BM - 1) / BM) * tiles_n;
 
   if (warp == WARP_TMA) {
-    if (lane == 0) {
+    if (elect_one()) {
       prefetch_tensor_map(maps.A);
       prefetch_tensor_map(maps.B);
       if (PA == 2) prefetch_tensor_map(maps.A2);
       if (PB == 2) prefetch_tensor_map(maps.B2);
       if (maps.Y != nullptr) prefetch_tensor_map(maps.Y);
-      int it = 0;  // K steps issued so far (all tiles)
+      int it = 0;  // K steps issued so far (all tiles), stage it % S
+      int s = 0;
+      uint32_t phase = 1;  // of mma_done[s]: the first pass over the ring waits for nothing
       int ready_m = -1;
       bool ok = true;
       for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
         const int mb = t / tiles_n;
         const int m0 = mb * BM;
-        const int n0 = (t % tiles_n) * BNT;
+        const int n0 = (t - mb * tiles_n) * BNT;
         if (ready != nullptr && mb != ready_m) {
           if (!wait_rows_ready(ready, mb, static_cast<uint32_t>(min(BM, g.M - m0)), abort,
                                g.status)) {
@@ -228,27 +230,28 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
           ready_m = mb;
         }
         for (int kb = 0; kb < nk; ++kb, ++it) {
-          const int s = it % S;
-          if (!mbar_wait_bounded(&bars->mma_done[s], ((it / S) & 1) ^ 1, abort, g.status,
-                                 kWaitLimitNs)) {
+          if (!mbar_wait_bounded(&bars->mma_done[s], phase, abort, g.status, kWaitLimitNs)) {
             ok = false;
             break;
           }
-          mbar_arrive_expect_tx(&bars->tma_full[s], TX);
+          uint64_t* full = &bars->tma_full[s];
+          mbar_arrive_expect_tx(full, TX);
           if (APACK)
-            tma_load_2d(smem + C::OFF_PA + s * A_P, maps.A, kb * BKP, m0, &bars->tma_full[s]);
+            tma_load_2d(smem + C::OFF_PA + s * A_P, maps.A, kb * BKP, m0, full);
           else
-            tma_load_2d(smem + C::OFF_UA + s * C::AU, maps.A, kb * BK, m0, &bars->tma_full[s]);
+            tma_load_2d(smem + C::OFF_UA + s * C::AU, maps.A, kb * BK, m0, full);
           if (PA == 2)
-            tma_load_2d(smem + C::OFF_UA + s * C::AU + A_U, maps.A2, kb * BK, m0,
-                        &bars->tma_full[s]);
+            tma_load_2d(smem + C::OFF_UA + s * C::AU + A_U, maps.A2, kb * BK, m0, full);
           if (BPACK)
-            tma_load_2d(smem + C::OFF_PB + s * C::BP, maps.B, kb * BKP, n0, &bars->tma_full[s]);
+            tma_load_2d(smem + C::OFF_PB + s * C::BP, maps.B, kb * BKP, n0, full);
           else
-            tma_load_2d(smem + C::OFF_UB + s * C::BU, maps.B, kb * BK, n0, &bars->tma_full[s]);
+            tma_load_2d(smem + C::OFF_UB + s * C::BU, maps.B, kb * BK, n0, full);
           if (PB == 2)
-            tma_load_2d(smem + C::OFF_UB + s * C::BU + BNT * BK, maps.B2, kb * BK, n0,
-                        &bars->tma_full[s]);
+            tma_load_2d(smem + C::OFF_UB + s * C::BU + BNT * BK, maps.B2, kb * BK, n0, full);
+          if (++s == S) {
+            s = 0;
+            phase ^= 1;
+          }
         }
       }
       // On an abort, the copies already in flight must land before exit.
@@ -257,11 +260,17 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
           mbar_wait_bounded(&bars->tma_full[j % S], (j / S) & 1, nullptr, nullptr, 10000000ull);
       }
     }
+    __syncwarp();
   } else if (warp == WARP_MMA) {
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t idesc = F6 ? idesc_f8f6f4_f32(BM, BNT, kFmtE2M3, kFmtE2M3)
                                     : idesc_e4m3_f32(BM, BNT);
-      int it = 0, tc = 0;
+      // Operand descriptors of stage 0; a stage, plane or K slice further adds
+      // its bytes / 16 to the start-address field.
+      const uint64_t adesc = sw128_desc(smem_addr(smem + C::OFF_UA));
+      const uint64_t bdesc = sw128_desc(smem_addr(smem + C::OFF_UB));
+      int s = 0, tc = 0;
+      uint32_t phase = 0;  // of the stage's ready barrier
       bool ok = true;
       for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tc) {
         const int buf = SEP ? 0 : (tc & 1);
@@ -273,16 +282,15 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
         }
         tc_fence_after();
         const uint32_t d = tmem + buf * BNT;
-        for (int kb = 0; kb < nk; ++kb, ++it) {
-          const int s = it % S;
+        for (int kb = 0; kb < nk; ++kb) {
           uint64_t* ready_bar = C::UNPACK ? &bars->unpacked[s] : &bars->tma_full[s];
-          if (!mbar_wait_bounded(ready_bar, (it / S) & 1, abort, g.status, kWaitLimitNs)) {
+          if (!mbar_wait_bounded(ready_bar, phase, abort, g.status, kWaitLimitNs)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t a0 = smem_addr(smem + C::OFF_UA + s * C::AU);
-          const uint32_t b0 = smem_addr(smem + C::OFF_UB + s * C::BU);
+          const uint64_t a0 = adesc + static_cast<uint32_t>(s * (C::AU / 16));
+          const uint64_t b0 = bdesc + static_cast<uint32_t>(s * (C::BU / 16));
 #pragma unroll
           for (int pa = 0; pa < PA; ++pa)
 #pragma unroll
@@ -294,10 +302,14 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
                 const int acc_i = SEP ? (pa + pb) : 0;
                 const bool first = SEP ? ((kb | k) == 0 && !(pa == 1 && pb == 0))
                                        : (kb | pa | pb | k) == 0;
-                mma_e4m3(d + acc_i * BNT, sw128_desc(a0 + pa * A_U + k * 32),
-                         sw128_desc(b0 + pb * BNT * BK + k * 32), idesc, first ? 0u : 1u);
+                mma_e4m3(d + acc_i * BNT, a0 + (pa * A_U + k * 32) / 16,
+                         b0 + (pb * BNT * BK + k * 32) / 16, idesc, first ? 0u : 1u);
               }
           mma_commit(&bars->mma_done[s]);
+          if (++s == S) {
+            s = 0;
+            phase ^= 1;
+          }
         }
         if (ok) mma_commit(&bars->acc_full[buf]);
       }
@@ -305,6 +317,7 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
       mma_commit(&bars->drained);
       mbar_wait_bounded(&bars->drained, 0, nullptr, nullptr, 10000000ull);
     }
+    __syncwarp();
   } else if (warp < 4 || (C::EPI_WARPS == 8 && warp >= 6 && warp < 10)) {
     // ---- epilogue ----
     const int quarter = warp & 3;

@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(128, 1)
   __shared__ int32_t abort;
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStreamStages; ++s) {
       mbar_init(&full[s], 1);
@@ -155,40 +155,51 @@ __global__ void __launch_bounds__(128, 1)
   const int nk = K / 128, mt = rows / 128, nt = rows / 256;
   constexpr uint32_t TX = F6 ? (kStreamA + kStreamB) / 4 * 3 : kStreamA + kStreamB;
   const int steps = tiles * nk;
-  if (warp == 0 && lane == 0) {
+  if (warp == 0 && elect_one()) {
     prefetch_tensor_map(&mapA);
     prefetch_tensor_map(&mapB);
+    int s = 0, kb = 0, t = static_cast<int>(blockIdx.x);
+    uint32_t phase = 1;
     for (int it = 0; it < steps; ++it) {
-      const int s = it % kStreamStages;
-      const int t = static_cast<int>(blockIdx.x) + (it / nk) * static_cast<int>(gridDim.x);
-      const int kb = it % nk;
-      if (!mbar_wait_bounded(&empty[s], ((it / kStreamStages) & 1) ^ 1, &abort, status,
-                             kWaitLimitNs))
-        break;
+      if (!mbar_wait_bounded(&empty[s], phase, &abort, status, kWaitLimitNs)) break;
       mbar_arrive_expect_tx(&full[s], TX);
       uint8_t* st = smem + s * (kStreamA + kStreamB);
       tma_load_2d(st, &mapA, kb * 128, (t % mt) * 128, &full[s]);
       tma_load_2d(st + kStreamA, &mapB, kb * 128, ((t / mt) % nt) * 256, &full[s]);
+      if (++s == kStreamStages) {
+        s = 0;
+        phase ^= 1;
+      }
+      if (++kb == nk) {
+        kb = 0;
+        t += static_cast<int>(gridDim.x);
+      }
     }
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1 && elect_one()) {
     constexpr uint32_t idesc = F6 ? idesc_f8f6f4_f32(128, 256, kFmtE2M3, kFmtE2M3)
                                   : idesc_e4m3_f32(128, 256);
+    const uint64_t adesc = sw128_desc(smem_addr(smem));
+    const uint64_t bdesc = sw128_desc(smem_addr(smem) + kStreamA);
+    const uint32_t d = MMA ? slot : 0u;
+    int s = 0;
+    uint32_t phase = 0;
     bool ok = true;
     for (int it = 0; it < steps && ok; ++it) {
-      const int s = it % kStreamStages;
-      ok = mbar_wait_bounded(&full[s], (it / kStreamStages) & 1, &abort, status, kWaitLimitNs);
+      ok = mbar_wait_bounded(&full[s], phase, &abort, status, kWaitLimitNs);
       if (!ok) break;
       if (MMA) {
         tc_fence_after();
-        const uint32_t a0 = smem_addr(smem + s * (kStreamA + kStreamB));
-        const uint32_t b0 = a0 + kStreamA;
+        const uint32_t off = static_cast<uint32_t>(s * ((kStreamA + kStreamB) / 16));
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          mma_e4m3(slot, sw128_desc(a0 + 32 * k), sw128_desc(b0 + 32 * k), idesc,
-                   (it | k) != 0 ? 1u : 0u);
+          mma_e4m3(d, adesc + off + 2 * k, bdesc + off + 2 * k, idesc, (it | k) != 0 ? 1u : 0u);
         mma_commit(&empty[s]);
       } else {
         mbar_arrive(&empty[s]);
+      }
+      if (++s == kStreamStages) {
+        s = 0;
+        phase ^= 1;
       }
     }
     if (MMA) {
