@@ -60,9 +60,9 @@ struct GemmArgs {
 // ([rows][K/2]), CLQ_CODES_E4M3 ([rows][K]) or, for 8-bit codes,
 // CLQ_CODES_E4M3_SPLIT ([rows][2][K]; A split with B E4M3 or split); TMA maps
 // are built here.
-// Output-channel tile width (192 or 256) of the E4M3 x E4M3 GEMM for an
-// M x N product on `sms` SMs.
-int gemm_tile_n(int M, int N, int sms);
+// Output-channel tile width (192 or 256) of the product of 4-bit
+// execution-layout operands, tiles of `rows` rows dealt to `units` CTAs or pairs.
+int gemm_tile_n(int M, int N, int rows, int units);
 cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, int w_codes,
                              const GemmArgs& g, int out_dtype, cudaStream_t st);
 
@@ -123,7 +123,7 @@ bool encode_tma_2d_strided(CUtensorMap* map, CUtensorMapDataType dt, uint32_t es
                            CUtensorMapSwizzle swz);
 bool encode_tma_2d_u8(CUtensorMap* map, const void* base, uint64_t inner_bytes,
                       uint64_t rows, uint32_t box_inner, uint32_t box_rows);
-// 2-byte output tile map for the epilogue stores (box 32 columns x 128 rows).
+// 2-byte output tile map for the epilogue stores (box 32 columns x 32 rows).
 bool encode_tma_out_tile(CUtensorMap* map, void* Y, int M, int N);
 int sm_count();  // cached per device
 // TMA map of a code array (rows x K) in layout `codes`, box_rows rows; for
@@ -172,6 +172,27 @@ template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int threads, size_t smem,
                        cudaStream_t st, Args&&... args) {
   return launch_ex(kernel, grid, threads, smem, st, true, std::forward<Args>(args)...);
+}
+
+// launch_pdl as clusters of `cluster` CTAs.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_cluster_pdl(void (*kernel)(KArgs...), int grid, int cluster, int threads,
+                               size_t smem, cudaStream_t st, Args&&... args) {
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned>(cluster);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(grid));
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
 }  // namespace clq

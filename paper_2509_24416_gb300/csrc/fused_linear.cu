@@ -43,6 +43,10 @@ using namespace gemm;
 // rotate-quant warps 6-15.
 constexpr int FT = 512;
 
+// Epilogue warps of the sequential form (unpack warps leave room for four).
+template <bool BPACK>
+constexpr int kSeqEpiWarps = BPACK ? 4 : 8;
+
 // Adds the rows [row0, row0 + rows) to the ready counters of the 128-token
 // blocks they fall in (a tile of rows may straddle two blocks); RELEASE: each
 // add is a release at GPU scope, else relaxed (the caller fences first).
@@ -95,7 +99,7 @@ constexpr int kTeamFirst = (WARP_MMA + 1) * 32;  // 192
 constexpr int kTeamThreads = FT - kTeamFirst;     // 320
 constexpr int kTeamCompute = kTeamThreads - 32;   // 288
 constexpr uint32_t kTeamBarrier = 2;  // 0: CTA, 1: GEMM epilogue, 2-3: team
-constexpr int kConcStride = 19 * 1024;
+constexpr int kConcStride = 18 * 1024;
 constexpr int kConcStages = 3;
 constexpr int kConcGemmStages = 3;
 
@@ -117,7 +121,8 @@ __global__ void __launch_bounds__(FT, 1)
   __shared__ Barriers bars;
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  setup<false, BPACK, BNT>(&bars);
+  constexpr int EW = kSeqEpiWarps<BPACK>;
+  setup<false, BPACK, BNT, 1, 1, EW>(&bars);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -128,11 +133,11 @@ __global__ void __launch_bounds__(FT, 1)
   __syncthreads();
 
   const Maps maps{&mapA, &mapB, use_tma_store ? &mapY : nullptr};
-  pipeline<T, false, BPACK, BNT, false, 1, 1, false, 0, MAX_STAGES, F6>(maps, g, smem, &bars,
-                                                                        tmem, ready);
+  pipeline<T, false, BPACK, BNT, 1, 1, false, EW, MAX_STAGES, F6>(maps, g, smem, &bars, tmem,
+                                                                  ready);
   tc_fence_before();
   __syncthreads();
-  teardown(tmem, Cfg<false, BPACK, BNT>::TMEM);
+  teardown(tmem, Cfg<false, BPACK, BNT, 1, 1, EW>::TMEM);
 }
 
 template <typename T, int BNT, bool F6>
@@ -162,7 +167,7 @@ __global__ void __launch_bounds__(FT, 1)
         rq, smem + Conc<BNT>::RQ_OFF, tile_counter, PublishRows{ready, team}, team);
   } else {
     const Maps maps{&mapA, &mapB, use_tma_store ? &mapY : nullptr, nullptr, nullptr};
-    pipeline<T, false, false, BNT, false, 1, 1, false, 4, kConcGemmStages, F6>(maps, g, smem,
+    pipeline<T, false, false, BNT, 1, 1, false, 4, kConcGemmStages, F6>(maps, g, smem,
                                                                               &bars, tmem, ready);
   }
   tc_fence_before();
@@ -213,7 +218,7 @@ FusedWorkspace fused_workspace_layout(int M, int K) {
 namespace {
 
 // Concurrent form (E4M3 weights): rows per tile as the 288 compute threads
-// and a 19 KB stage allow (8 at K = 1152, 2 at K = 4608).
+// and a 18 KB stage allow (8 at K = 1152, 2 at K = 4608).
 cudaError_t launch_concurrent(const RotateQuantArgs& rq_in, const uint8_t* W, int w_codes,
                               const GemmArgs& g, int logb, int dtype, uint32_t* ready, int sms,
                               cudaStream_t st) {
@@ -226,7 +231,7 @@ cudaError_t launch_concurrent(const RotateQuantArgs& rq_in, const uint8_t* W, in
   const int R = std::min(kTeamCompute / segs, kConcStride / (2 * rq.K));
   if (R < 1) return cudaErrorInvalidValue;
   rq.rows_per_tile = R;
-  const int bn = gemm_tile_n(g.M, g.N, sms);
+  const int bn = gemm_tile_n(g.M, g.N, BM, sms);
   const size_t gemm_off = bn == 192 ? Conc<192>::RQ_OFF : Conc<256>::RQ_OFF;
   const size_t smem = gemm_off + rq::smem_bytes(R, kConcStride, kConcStages) + 1024;
   if (smem > 227u * 1024u - 2048u) return cudaErrorInvalidValue;
@@ -271,7 +276,8 @@ cudaError_t launch_fused_linear(const RotateQuantArgs& rq_in, const uint8_t* W, 
   if (!bpack && rq_in.K <= kConcStride / 2 && rq_in.K / 32 <= kTeamCompute)
     return launch_concurrent(rq_in, W, w_codes, g, logb, dtype, ready, sms, st);
   const int bn = BN;
-  const size_t gemm_bytes = bpack ? Cfg<false, true>::BYTES : Cfg<false, false>::BYTES;
+  const size_t gemm_bytes = bpack ? Cfg<false, true, BN, 1, 1, kSeqEpiWarps<true>>::BYTES
+                                  : Cfg<false, false, BN, 1, 1, kSeqEpiWarps<false>>::BYTES;
   const size_t limit = 227u * 1024u - 2048u;  // dynamic + static shared memory
   // Rotate-quant phase: as many rows per tile as 512 threads cover and one
   // raw stage holds.

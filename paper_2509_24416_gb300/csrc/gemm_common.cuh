@@ -18,10 +18,8 @@ constexpr int A_P = BM * BKP;     // 8 KB packed A stage
 constexpr int B_P = BN * BKP;     // 16 KB packed B stage
 constexpr int EPI_COLS = 32;      // output columns per epilogue store
 constexpr int EPI_ROWS = 32;      // rows per store: one warp's TMEM lanes
-constexpr int EPI_BYTES = EPI_ROWS * EPI_COLS * 2;  // 2 KB staging buffer
-constexpr int EPI_TOTAL = 8 * EPI_BYTES;            // 4 warps x 2 or 8 warps x 1
+constexpr int EPI_BYTES = EPI_ROWS * EPI_COLS * 2;  // 2 KB staging buffer, one a warp
 constexpr int TMEM_COLS = 512;    // two 128 x 256 fp32 accumulators
-constexpr uint32_t kEpiBarrier = 1;  // named barrier id of the epilogue warps
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;
@@ -31,10 +29,6 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t c) {
 
 __device__ __forceinline__ uint32_t pack2(uint16_t lo, uint16_t hi) {
   return static_cast<uint32_t>(lo) | (static_cast<uint32_t>(hi) << 16);
-}
-
-__device__ __forceinline__ void named_bar_sync(uint32_t id, uint32_t threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
 // Eight 4-bit two's-complement codes (code j in nibble j) -> eight E4M3
@@ -80,19 +74,26 @@ __device__ __forceinline__ void unpack_rows(const uint8_t* __restrict__ src,
   }
 }
 
-// 32 lanes x 32 bit, 32 consecutive columns per thread.
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
+// 16 TMEM lanes x 32 columns, one matrix fragment per 8 columns: thread t gets,
+// of column group g, columns 8 g + 2 (t % 4) and + 1 of lane t / 4 in r[4 g],
+// r[4 g + 1] and of lane t / 4 + 8 in r[4 g + 2], r[4 g + 3].
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
         "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-        "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]),
-        "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]),
-        "=r"(r[31])
+        "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
+}
+
+// Four 8 x 8 matrices of 16-bit values to shared memory: lane l gives the
+// address of row l % 8 of matrix l / 8, register m the pair at row l / 4,
+// columns 2 (l % 4) and + 1 of matrix m.
+__device__ __forceinline__ void stmatrix4(uint32_t addr, const uint32_t (&o)[4]) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr),
+               "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3])
+               : "memory");
 }
 
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void* smem_src,
@@ -119,169 +120,157 @@ __device__ __forceinline__ void bulk_wait_all() {
 
 // Wait for this thread's outstanding tcgen05.ld and make every register of
 // r depend on that wait, so that no use of r is scheduled before it.
-__device__ __forceinline__ void tmem_ld_wait_tie(uint32_t (&r)[32]) {
+__device__ __forceinline__ void tmem_ld_wait_tie(uint32_t (&r)[16]) {
   tmem_ld_wait();
 #pragma unroll
-  for (int i = 0; i < 32; ++i) asm volatile("" : "+r"(r[i]));
+  for (int i = 0; i < 16; ++i) asm volatile("" : "+r"(r[i]));
 }
 
-// One 32-row x 32-column block of the epilogue (the block at tile column c):
-// y = acc * s_x[row] * s_w[col] / b + bias[col], rounded to OutT, where
-// col_scale / col_bias hold s_w / b and bias for the tile's columns.  With a
-// TMA map for Y the block goes through one of the warp's NBUF 64-byte-swizzled
-// staging buffers and one bulk tensor store issued by lane 0; otherwise (N not
-// a multiple of 8) each lane stores its row directly.
-// ASYM (asymmetric activation codes, centered): s_x[row] is the row's step
-// delta, zm the value of code 0, col_zw holds sum_k q_w[col][k] * s_w / b,
-// and y = acc * delta * s_w / b + zm * col_zw + bias.
-template <typename OutT, int NBUF, bool ASYM = false>
-__device__ __forceinline__ void epilogue_block(const uint32_t (&r)[32], int c, int quarter,
-                                               int lane, int m0, int n0, int M, int N,
-                                               float sx, const float* col_scale,
-                                               const float* col_bias, float zm,
-                                               const float* col_zw, uint8_t* staging,
-                                               const CUtensorMap* mapY, void* Y,
-                                               int32_t* acc_dbg, int& store_count) {
-  const int row = m0 + quarter * 32 + lane;
-  uint32_t o[16];
-  const float2 sx2 = make_float2(sx, sx);
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const float4 cs = *reinterpret_cast<const float4*>(col_scale + c + 4 * j);
-    float4 cb = *reinterpret_cast<const float4*>(col_bias + c + 4 * j);
-    if constexpr (ASYM) {
-      const float4 cz = *reinterpret_cast<const float4*>(col_zw + c + 4 * j);
-      const float2 zm2 = make_float2(zm, zm);
-      const float2 b0 = __ffma2_rn(zm2, make_float2(cz.x, cz.y), make_float2(cb.x, cb.y));
-      const float2 b1 = __ffma2_rn(zm2, make_float2(cz.z, cz.w), make_float2(cb.z, cb.w));
-      cb = make_float4(b0.x, b0.y, b1.x, b1.y);
-    }
-    const float2 a0 = make_float2(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1]));
-    const float2 a1 = make_float2(__uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3]));
-    const float2 y0 =
-        __ffma2_rn(a0, __fmul2_rn(sx2, make_float2(cs.x, cs.y)), make_float2(cb.x, cb.y));
-    const float2 y1 =
-        __ffma2_rn(a1, __fmul2_rn(sx2, make_float2(cs.z, cs.w)), make_float2(cb.z, cb.w));
-    o[2 * j] = Num<OutT>::pack2(y0.x, y0.y);
-    o[2 * j + 1] = Num<OutT>::pack2(y1.x, y1.y);
-  }
-  if (acc_dbg != nullptr && row < M) {
-    int32_t* arow = acc_dbg + static_cast<size_t>(row) * N + n0 + c;
-#pragma unroll
-    for (int j = 0; j < 32; ++j)
-      if (n0 + c + j < N) arow[j] = __float2int_rn(__uint_as_float(r[j]));
-  }
-  if (mapY != nullptr) {
-    uint8_t* sb = staging + (NBUF > 1 ? (store_count & 1) * EPI_BYTES : 0);
-    // The store that last used sb has finished reading it.
-    if (lane == 0) bulk_wait_read<NBUF - 1>();
-    __syncwarp();
-    uint8_t* srow = sb + lane * 64;
-    const int sw = (lane >> 1) & 3;
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      *reinterpret_cast<uint4*>(srow + ((q ^ sw) << 4)) =
-          make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
-    fence_proxy_async_smem();
-    __syncwarp();
-    if (lane == 0) {
-      tma_store_2d(mapY, sb, n0 + c, m0 + quarter * 32);
-      bulk_commit();
-    }
-    ++store_count;
-  } else if (row < M) {
-    uint16_t* yrow = static_cast<uint16_t*>(Y) + static_cast<size_t>(row) * N + n0 + c;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      if (n0 + c + 2 * j < N) yrow[2 * j] = static_cast<uint16_t>(o[j] & 0xFFFFu);
-      if (n0 + c + 2 * j + 1 < N) yrow[2 * j + 1] = static_cast<uint16_t>(o[j] >> 16);
-    }
+// Byte offset of 16-byte chunk q (8 columns) of row r in a staging buffer: the
+// tensor map's 64-byte swizzle, which also spreads the rows over the banks.
+__device__ __forceinline__ int staged_chunk(int r, int q) {
+  return r * 64 + ((q ^ ((r >> 1) & 3)) << 4);
+}
+
+// A staged block (rows row0 .. row0 + 31, columns col0 .. col0 + 31) straight to
+// Y when N % 8 != 0 rules the tensor store out: half a warp takes consecutive
+// column pairs of one row, four-byte aligned whatever N's parity.
+__device__ __forceinline__ void store_block_direct(const uint8_t* staging, int lane, int row0,
+                                                   int M, int col0, int N, uint16_t* Y) {
+  const int ncol = min(EPI_COLS, N - col0);
+  const int rows = min(EPI_ROWS, M - row0);
+  auto elem = [&](int r, int j) {
+    return *reinterpret_cast<const uint16_t*>(staging + staged_chunk(r, j >> 3) + (j & 7) * 2);
+  };
+#pragma unroll 4
+  for (int r = lane >> 4; r < rows; r += 2) {
+    const size_t e0 = static_cast<size_t>(row0 + r) * N + col0;
+    uint16_t* y = Y + e0;
+    const int j = 2 * (lane & 15) + static_cast<int>(e0 & 1);  // y + j is four-byte aligned
+    if (j + 1 < ncol)
+      *reinterpret_cast<uint32_t*>(y + j) = pack2(elem(r, j), elem(r, j + 1));
+    else if (j < ncol)
+      y[j] = elem(r, j);
+    if ((e0 & 1) && (lane & 15) == 0) y[0] = elem(r, 0);
   }
 }
 
-// One warp's share of a tile's epilogue: TMEM lanes 32 * quarter .. + 31
-// (the warp's rows) and tile columns [col0, col0 + NCOL).  With PREFETCH the
-// TMEM load of the next 32 columns is issued before the current block is
-// processed, so its latency hides behind the arithmetic and the store (32
-// more registers a thread).  `store_count` counts this warp's stores (it
-// selects the staging buffer).
+// One warp's share of a tile's epilogue: TMEM lanes 32 * quarter .. + 31 (the
+// warp's rows) and tile columns [col0, col0 + NCOL) in blocks of 32 columns:
+// TMEM -> registers -> y = acc * s_x[row] * s_w[col] / b + bias[col], rounded to
+// OutT -> the warp's swizzled staging buffer -> one bulk tensor store a block (or
+// direct stores, mapY null).  `col` is the warp's column data (s_w / b, bias,
+// zero-point sums; NCOL floats each); sx[k] belongs to row 8 k + lane / 4 of the
+// 32.  ASYM (asymmetric activation codes, centered): sx is the row's step delta,
+// zm the value of code 0, and y = acc * delta * s_w / b + zm * sum_k q_w * s_w /
+// b + bias.  Once the last block is in registers, `release()` hands the
+// accumulator back, so that the MMAs of the tile after next need not wait for
+// the stores.
+//
+// What it costs is shared-memory time, which the MMAs' operands and the copies
+// that bring them want too.  So the accumulators are read as matrix fragments:
+// a thread's two columns of a group serve four rows, and 32 columns take 8
+// eight-byte loads of column data a warp where one row a lane took 16
+// sixteen-byte ones; the packed pairs leave by stmatrix.
 //
 // SEP3 > 0: the accumulator is the sum of three TMEM accumulators SEP3
 // columns apart, each an exact integer in fp32 (the W8A8 plane products); they
 // are added as int32 and the block goes on with that (exact) sum.
-template <typename OutT, int NCOL, int NBUF, bool PREFETCH, bool ASYM = false, int SEP3 = 0>
-__device__ __forceinline__ void epilogue_part(uint32_t tmem_acc, int quarter, int col0,
-                                              int lane, int m0, int n0, int M, int N, float sx,
-                                              const float* col_scale, const float* col_bias,
-                                              float zm, const float* col_zw,
-                                              uint8_t* staging, const CUtensorMap* mapY,
-                                              void* Y, int32_t* acc_dbg, int& store_count) {
+template <typename OutT, int NCOL, bool ASYM, int SEP3, typename Release>
+__device__ __forceinline__ void epilogue_part(uint32_t tmem_acc, int quarter, int col0, int lane,
+                                              int m0, int n0, int M, int N, const float (&sx)[4],
+                                              const float* col, const float (&zm)[4],
+                                              uint8_t* staging, const CUtensorMap* mapY, void* Y,
+                                              int32_t* acc_dbg, Release release) {
   static_assert(NCOL % EPI_COLS == 0, "column share must be whole 32-column blocks");
   const uint32_t lane_base = tmem_acc + (static_cast<uint32_t>(quarter * 32) << 16);
-  if (n0 + col0 >= N) return;
-  if constexpr (SEP3 > 0) {
-    const int row = m0 + quarter * 32 + lane;
-#pragma unroll 1
-    for (int c = col0; c < col0 + NCOL && n0 + c < N; c += EPI_COLS) {
-      uint32_t r[32], r1[32];
-      tmem_ld32(lane_base + c, r);
-      tmem_ld32(lane_base + SEP3 + c, r1);
-      tmem_ld_wait_tie(r);
-      tmem_ld_wait_tie(r1);
-      int32_t isum[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j)
-        isum[j] = __float2int_rn(__uint_as_float(r[j])) + __float2int_rn(__uint_as_float(r1[j]));
-      tmem_ld32(lane_base + 2 * SEP3 + c, r1);
-      tmem_ld_wait_tie(r1);
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        isum[j] += __float2int_rn(__uint_as_float(r1[j]));
-        r[j] = __float_as_uint(static_cast<float>(isum[j]));
-      }
-      if (acc_dbg != nullptr && row < M) {
-        int32_t* arow = acc_dbg + static_cast<size_t>(row) * N + n0 + c;
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (n0 + c + j < N) arow[j] = isum[j];
-      }
-      epilogue_block<OutT, NBUF, ASYM>(r, c, quarter, lane, m0, n0, M, N, sx, col_scale,
-                                       col_bias, zm, col_zw, staging, mapY, Y, nullptr,
-                                       store_count);
-    }
+  const int row0 = m0 + quarter * EPI_ROWS;
+  // blocks that hold rows and columns of Y (warp-uniform)
+  const int nblk =
+      row0 < M ? max(0, min(NCOL / EPI_COLS, (N - n0 - col0 + EPI_COLS - 1) / EPI_COLS)) : 0;
+  if (nblk == 0) {
+    release();
     return;
   }
-  if (!PREFETCH) {
+  const uint32_t stage_addr = smem_addr(staging);
 #pragma unroll 1
-    for (int c = col0; c < col0 + NCOL && n0 + c < N; c += EPI_COLS) {
-      uint32_t r[32];
-      tmem_ld32(lane_base + c, r);
-      tmem_ld_wait_tie(r);
-      epilogue_block<OutT, NBUF, ASYM>(r, c, quarter, lane, m0, n0, M, N, sx, col_scale,
-                                       col_bias, zm, col_zw, staging, mapY, Y, acc_dbg,
-                                       store_count);
+  for (int i = 0; i < nblk; ++i) {
+    const int c = col0 + i * EPI_COLS;  // tile column
+    uint32_t r[2][16];                  // rows 0 .. 15 and 16 .. 31
+    tmem_ld_frag(lane_base + c, r[0]);
+    tmem_ld_frag(lane_base + (16u << 16) + c, r[1]);
+    const float* cc = col + i * EPI_COLS + 2 * (lane & 3);
+    float2 cs[4], cb[4], cz[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      cs[g] = *reinterpret_cast<const float2*>(cc + 8 * g);
+      cb[g] = *reinterpret_cast<const float2*>(cc + NCOL + 8 * g);
+      if (ASYM) cz[g] = *reinterpret_cast<const float2*>(cc + 2 * NCOL + 8 * g);
     }
-    return;
-  }
-  uint32_t ra[32], rb[32];
-  tmem_ld32(lane_base + col0, ra);
-#pragma unroll 1
-  for (int c = col0; c < col0 + NCOL; c += 2 * EPI_COLS) {
-    // ra holds block c (issued earlier); warp-uniform conditions throughout.
-    tmem_ld_wait_tie(ra);
-    const bool more1 = c + EPI_COLS < col0 + NCOL && n0 + c + EPI_COLS < N;
-    if (more1) tmem_ld32(lane_base + c + EPI_COLS, rb);
-    epilogue_block<OutT, NBUF, ASYM>(ra, c, quarter, lane, m0, n0, M, N, sx, col_scale,
-                                     col_bias, zm, col_zw, staging, mapY, Y, acc_dbg,
-                                     store_count);
-    if (!more1) break;
-    tmem_ld_wait_tie(rb);
-    const bool more2 = c + 2 * EPI_COLS < col0 + NCOL && n0 + c + 2 * EPI_COLS < N;
-    if (more2) tmem_ld32(lane_base + c + 2 * EPI_COLS, ra);
-    epilogue_block<OutT, NBUF, ASYM>(rb, c + EPI_COLS, quarter, lane, m0, n0, M, N, sx,
-                                     col_scale, col_bias, zm, col_zw, staging, mapY, Y,
-                                     acc_dbg, store_count);
-    if (!more2) break;
+    tmem_ld_wait_tie(r[0]);
+    tmem_ld_wait_tie(r[1]);
+    if constexpr (SEP3 > 0) {
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        uint32_t r1[16], r2[16];
+        const uint32_t at = lane_base + (static_cast<uint32_t>(half * 16) << 16) + c;
+        tmem_ld_frag(at + SEP3, r1);
+        tmem_ld_frag(at + 2 * SEP3, r2);
+        tmem_ld_wait_tie(r1);
+        tmem_ld_wait_tie(r2);
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+          r[half][j] = static_cast<uint32_t>(__float2int_rn(__uint_as_float(r[half][j])) +
+                                             __float2int_rn(__uint_as_float(r1[j])) +
+                                             __float2int_rn(__uint_as_float(r2[j])));
+      }
+    }
+    if (i == nblk - 1) release();
+    if (acc_dbg != nullptr) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int row = row0 + 8 * k + (lane >> 2);
+          const int cn = n0 + c + 8 * (j >> 1) + 2 * (lane & 3) + (j & 1);
+          const uint32_t v = r[k >> 1][4 * (j >> 1) + 2 * (k & 1) + (j & 1)];
+          if (row < M && cn < N)
+            acc_dbg[static_cast<size_t>(row) * N + cn] =
+                SEP3 > 0 ? static_cast<int32_t>(v) : __float2int_rn(__uint_as_float(v));
+        }
+    }
+    // The store that last used the staging buffer has finished reading it.
+    if (mapY != nullptr && elect_one()) bulk_wait_read<0>();
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {  // rows 8 k + lane / 4
+      const float2 sx2 = make_float2(sx[k], sx[k]);
+      uint32_t o[4];
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        const uint32_t v0 = r[k >> 1][4 * g + 2 * (k & 1)];
+        const uint32_t v1 = r[k >> 1][4 * g + 2 * (k & 1) + 1];
+        const float2 acc = SEP3 > 0 ? make_float2(static_cast<float>(static_cast<int32_t>(v0)),
+                                                  static_cast<float>(static_cast<int32_t>(v1)))
+                                    : make_float2(__uint_as_float(v0), __uint_as_float(v1));
+        const float2 bias = ASYM ? __ffma2_rn(make_float2(zm[k], zm[k]), cz[g], cb[g]) : cb[g];
+        const float2 y = __ffma2_rn(acc, __fmul2_rn(sx2, cs[g]), bias);
+        o[g] = Num<OutT>::pack2(y.x, y.y);
+      }
+      stmatrix4(stage_addr + staged_chunk(8 * k + (lane & 7), lane >> 3), o);
+    }
+    if (mapY != nullptr) {
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (elect_one()) {
+        tma_store_2d(mapY, staging, n0 + c, row0);
+        bulk_commit();
+      }
+    } else {
+      __syncwarp();
+      store_block_direct(staging, lane, row0, M, n0 + c, N, static_cast<uint16_t*>(Y));
+      __syncwarp();
+    }
   }
 }
 

@@ -15,24 +15,36 @@
 // accumulators (SEP below) that are each exact and are added as integers.
 // E2M3 operands (F6) take the same MMA with 6-bit formats.
 //
-// Persistent: one CTA per SM walks 128 (M) x 256 (N) tiles in a static
+// Persistent: one CTA per SM walks 128 (M) x 256 (N) tiles, or a pair of CTAs
+// (CG 2, one cluster, tcgen05 cta_group::2) walks 256 x 256 tiles, in a static
 // round-robin order, K step 128 codes.  Each operand arrives either as E4M3
 // bytes, which TMA writes straight into the MMA operand buffer with the
 // 128-byte swizzle, or as packed nibbles (APACK / BPACK), which TMA stages and
-// unpack warps expand into that layout.  Warp roles:
+// unpack warps expand into that layout.  Each CTA of a pair loads its own 128
+// rows of A and half of B's rows, all copies of a stage completing on the
+// leader's barrier; the leader issues the MMAs, which read both CTAs' shared
+// memory, and their completion signals the barriers of both.  Warp roles:
 //   warp 4       TMA producer;
 //   warps 6-13   unpack (only when an operand is packed; 448 threads);
-//   warp 5       one lane issues tcgen05.mma (4 x K=32 per stage) and commits
-//                stage and tile completion;
-//   warps 0-3    epilogue (and warps 6-9 too when no operand is packed; 320
-//                threads then, so 168 registers a thread): warp w drains accumulator
-//                rows 32 * (w % 4) .. + 31 (the TMEM lanes its SM sub-
-//                partition may read), all 256 columns with four warps, one
-//                half each with eight: TMEM -> registers -> scale, bias,
+//   warp 5       one lane (of the leader) issues tcgen05.mma (4 x K=32 per
+//                stage) and commits stage and tile completion;
+//   warps 0-3, 6-9 epilogue (warps 0-3 alone when an operand is packed or the
+//                caller asks for four): warp w drains accumulator rows 32 * (w %
+//                4) .. + 31 (the TMEM lanes its SM sub-partition may read), half
+//                the columns each with eight: TMEM -> registers -> scale, bias,
 //                round -> swizzled staging -> TMA tensor store.  Two TMEM
 //                accumulators let the epilogue of tile i overlap the MMAs of
 //                tile i + 1.
 //   other warps  idle in this phase.
+// What bounds it: the MMAs of a 128-code step take 542 clocks, the loop with its
+// copies 587 (a pair, operands in L2).  Around it, at K = 1152 a tile takes
+// about 5900 clocks instead of 5300 (the epilogue's shared-memory time), the
+// first MMA starts 1900 clocks after the launch wait and the last tile's
+// epilogue adds 4000.  The stages matter most once operands come from further
+// away: 4608 x 12288 x 3072 took 112.6 us with four 32 KB stages, 98.3 with
+// five and 90.1 with six, which is why the staging buffers are 2 KB a warp.
+// The epilogue warps keep their column data to themselves and read their row
+// scales before the accumulator is complete: no barrier joins them.
 // With `ready` counters (fused kernel), the producer waits until all rows of
 // a tile's token block have been published before loading its A tiles.
 // Every wait is bounded; on a timeout the roles drain their own copies and
@@ -50,7 +62,7 @@ constexpr int WARP_TMA = 4;
 constexpr int WARP_MMA = 5;
 constexpr int WARP_UNPACK0 = 6;
 constexpr int MIN_THREADS = (WARP_UNPACK0 + NUM_UNPACK / 32) * 32;  // 448
-constexpr int MAX_STAGES = 6;
+constexpr int MAX_STAGES = 8;
 
 // Tile BM x BNT (BNT = 256, or 192 for E4M3 operands where N splits better).
 // PA / PB: E4M3 planes per operand, 1 for 4-bit codes, 2 for 8-bit codes
@@ -62,19 +74,19 @@ constexpr int MAX_STAGES = 6;
 // accumulators (16 h x 16 h, the two cross terms, l x l) of one buffer, so
 // that each stays exact in fp32 (see pipeline()); 3 BNT TMEM columns.
 template <bool APACK, bool BPACK, int BNT = BN, int PA = 1, int PB = 1, int EW = 0,
-          int SMAX = MAX_STAGES, bool SEP = false>
+          int SMAX = MAX_STAGES, bool SEP = false, int CG = 1>
 struct Cfg {
   static constexpr bool UNPACK = APACK || BPACK;
   static constexpr int EPI_WARPS = EW != 0 ? EW : (UNPACK ? 4 : 8);
-  static constexpr int THREADS = UNPACK ? MIN_THREADS : 320;
-  static constexpr int EPI_THREADS = 32 * EPI_WARPS;
-  static constexpr int EPI_NBUF = 8 / EPI_WARPS;  // staging buffers per warp
-  static constexpr int EPI_NCOL = BNT * 4 / EPI_WARPS;  // columns per warp
+  static constexpr int THREADS = UNPACK ? MIN_THREADS : 32 * (EPI_WARPS + 2);
+  static constexpr int EPI_NCOL = BNT * 4 / EPI_WARPS;  // columns per epilogue warp
+  // a warp's column data: s_w / b, bias and (standalone kernel) zero-point sums
+  static constexpr int COL_FLOATS = (EW != 0 ? 2 : 3) * EPI_NCOL;
   static constexpr int AU = PA * A_U;    // E4M3 A stage (all planes)
-  static constexpr int BU = PB * BNT * BK;  // E4M3 B stage (all planes)
+  static constexpr int BU = PB * (BNT / CG) * BK;  // E4M3 B stage (all planes)
   static constexpr int BP = BNT * BKP;   // packed B stage
   static constexpr int STAGE = AU + BU + (APACK ? A_P : 0) + (BPACK ? BP : 0);
-  static constexpr int FIXED = EPI_TOTAL + 6 * BNT * 4;
+  static constexpr int FIXED = EPI_WARPS * (EPI_BYTES + COL_FLOATS * 4);
   static constexpr int S0 = (222 * 1024 - FIXED) / STAGE;
   static constexpr int S = S0 > SMAX ? SMAX : S0;  // pipeline stages
   static constexpr size_t OFF_UA = 0;                           // E4M3 operands
@@ -82,9 +94,10 @@ struct Cfg {
   static constexpr size_t OFF_PA = OFF_UB + S * BU;             // packed staging
   static constexpr size_t OFF_PB = OFF_PA + (APACK ? S * A_P : 0);
   static constexpr size_t OFF_EPI = OFF_PB + (BPACK ? S * BP : 0);
-  static constexpr size_t OFF_COL = OFF_EPI + EPI_TOTAL;        // [2][3][BNT] floats
-  static constexpr size_t BYTES = OFF_COL + 6 * BNT * sizeof(float);
-  static constexpr uint32_t TX = (APACK ? A_P : AU) + (BPACK ? BP : BU);
+  static constexpr size_t OFF_COL = OFF_EPI + EPI_WARPS * EPI_BYTES;  // per warp
+  static constexpr size_t BYTES = OFF_COL + EPI_WARPS * COL_FLOATS * sizeof(float);
+  // bytes that complete on a stage's barrier (both CTAs' copies of a pair)
+  static constexpr uint32_t TX = CG * ((APACK ? A_P : AU) + (BPACK ? BP : BU));
   // two accumulators of BNT columns, 2 * BNT rounded up to the power of two
   // tcgen05.alloc takes
   static constexpr uint32_t TMEM = SEP ? 512u : (2 * BNT <= 256 ? 256u : 512u);
@@ -92,8 +105,10 @@ struct Cfg {
   static_assert(S >= 2, "pipeline needs two stages");
   static_assert((PA == 1 || PA == 2) && (PB == 1 || PB == 2), "one or two planes");
   static_assert(!UNPACK || (PA == 1 && PB == 1), "8-bit planes come as E4M3 only");
-  static_assert(EPI_WARPS == 4 || (EPI_WARPS == 8 && !UNPACK), "4 or 8 epilogue warps");
+  static_assert(EPI_WARPS == 4 || !UNPACK, "packed operands leave four epilogue warps");
+  static_assert(EPI_NCOL % EPI_COLS == 0 && STAGE % 1024 == 0, "whole blocks, aligned staging");
   static_assert(SMAX <= MAX_STAGES, "barrier arrays hold MAX_STAGES stages");
+  static_assert(CG == 1 || (CG == 2 && !UNPACK && EW == 0), "pairs: E4M3 / E2M3 operands only");
   static_assert(!SEP || (PA == 2 && PB == 2 && 3 * BNT <= 512), "SEP: 8-bit x 8-bit, 3 BNT <= 512");
 };
 
@@ -129,9 +144,9 @@ __device__ __forceinline__ void fence_proxy_async_global() {
 // Barrier init (thread 0) and TMEM allocation (warp WARP_MMA); the caller
 // follows with tcgen05 fences around a CTA barrier.
 template <bool APACK, bool BPACK, int BNT = BN, int PA = 1, int PB = 1, int EW = 0,
-          int SMAX = MAX_STAGES, bool SEP = false>
+          int SMAX = MAX_STAGES, bool SEP = false, int CG = 1>
 __device__ __forceinline__ void setup(Barriers* bars) {
-  using C = Cfg<APACK, BPACK, BNT, PA, PB, EW, SMAX, SEP>;
+  using C = Cfg<APACK, BPACK, BNT, PA, PB, EW, SMAX, SEP, CG>;
   constexpr int S = C::S;
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -141,15 +156,15 @@ __device__ __forceinline__ void setup(Barriers* bars) {
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&bars->acc_full[s], 1);
-      mbar_init(&bars->acc_empty[s], C::EPI_THREADS);
+      mbar_init(&bars->acc_empty[s], CG * C::EPI_WARPS);
     }
     mbar_init(&bars->drained, 1);
     bars->abort = 0;
     fence_mbarrier_init();
   }
   if ((threadIdx.x >> 5) == WARP_MMA) {
-    tmem_alloc(&bars->tmem_slot, C::TMEM);
-    tmem_relinquish();
+    tmem_alloc<CG>(&bars->tmem_slot, C::TMEM);
+    tmem_relinquish<CG>();
   }
 }
 
@@ -170,8 +185,6 @@ __device__ __forceinline__ bool wait_rows_ready(const uint32_t* ready, int m, ui
   return true;
 }
 
-// EPI_PREFETCH: let the epilogue prefetch TMEM (taken only in the 320-thread
-// configuration, where registers allow it).
 // ASYM: asymmetric activation codes (zero-point epilogue, g.lo / g.wsum).
 // EW / SMAX: as in Cfg (the same values as the setup() call).
 // F6: both operands are E2M3 codes, 16 codes in 12 bytes in global memory;
@@ -188,13 +201,13 @@ __device__ __forceinline__ bool wait_rows_ready(const uint32_t* ready, int m, ui
 // multiples of 256 below 2^28 (exact up to 2^32), the second multiples of 16
 // below 2^25 (exact up to 2^28), the third integers below 2^20.  The
 // epilogue adds them as int32 (|q_x q_w| K <= 2^28).
-template <typename OutT, bool APACK, bool BPACK, int BNT = BN, bool EPI_PREFETCH = true,
-          int PA = 1, int PB = 1, bool ASYM = false, int EW = 0, int SMAX = MAX_STAGES,
-          bool F6 = false, bool SEP = false>
+template <typename OutT, bool APACK, bool BPACK, int BNT = BN, int PA = 1, int PB = 1, bool ASYM = false, int EW = 0, int SMAX = MAX_STAGES,
+          bool F6 = false, bool SEP = false, int CG = 1>
 __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, uint8_t* smem,
                                          Barriers* bars, uint32_t tmem, const uint32_t* ready) {
-  using C = Cfg<APACK, BPACK, BNT, PA, PB, EW, SMAX, SEP>;
+  using C = Cfg<APACK, BPACK, BNT, PA, PB, EW, SMAX, SEP, CG>;
   constexpr int S = C::S;
+  static_assert(!ASYM || EW == 0, "zero-point column data: standalone kernel only");
   static_assert(!F6 || (!C::UNPACK && PA == 1 && PB == 1), "E2M3 operands come one plane each");
   constexpr uint32_t TX = F6 ? C::TX / 4 * 3 : C::TX;
   volatile int32_t* abort = &bars->abort;
@@ -203,7 +216,13 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
   const int lane = threadIdx.x & 31;
   const int nk = (g.K + BK - 1) / BK;
   const int tiles_n = (g.N + BNT - 1) / BNT;
-  const int tiles = ((g.M + BM - 1) / BM) * tiles_n;
+  constexpr int TM = CG * BM;  // rows of a tile
+  const int tiles = ((g.M + TM - 1) / TM) * tiles_n;
+  // A unit, one CTA or a pair, takes every units-th tile; `rank` is this CTA's
+  // half of the pair's tile (rows) and of its B boxes.
+  const int unit = static_cast<int>(blockIdx.x) / CG;
+  const int units = static_cast<int>(gridDim.x) / CG;
+  const int rank = CG == 2 ? static_cast<int>(cluster_ctarank()) : 0;
 
   if (warp == WARP_TMA) {
     if (elect_one()) {
@@ -217,10 +236,12 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
       uint32_t phase = 1;  // of mma_done[s]: the first pass over the ring waits for nothing
       int ready_m = -1;
       bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+      // a pair's copies complete on the leader's barriers
+      const uint32_t full0 = CG == 2 ? cluster_addr(&bars->tma_full[0], 0) : 0;
+      for (int t = unit; t < tiles && ok; t += units) {
         const int mb = t / tiles_n;
-        const int m0 = mb * BM;
-        const int n0 = (t - mb * tiles_n) * BNT;
+        const int m0 = mb * TM + rank * BM;
+        const int n0 = (t - mb * tiles_n) * BNT + rank * (BNT / CG);
         if (ready != nullptr && mb != ready_m) {
           if (!wait_rows_ready(ready, mb, static_cast<uint32_t>(min(BM, g.M - m0)), abort,
                                g.status)) {
@@ -235,36 +256,45 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
             break;
           }
           uint64_t* full = &bars->tma_full[s];
-          mbar_arrive_expect_tx(full, TX);
+          if (CG == 1 || rank == 0) mbar_arrive_expect_tx(full, TX);
+          auto load = [&](size_t off, const CUtensorMap* map, int x, int y) {
+            if constexpr (CG == 2)
+              tma_load_2d_pair(smem + off, map, x, y, full0 + 8u * s);
+            else
+              tma_load_2d(smem + off, map, x, y, full);
+          };
           if (APACK)
-            tma_load_2d(smem + C::OFF_PA + s * A_P, maps.A, kb * BKP, m0, full);
+            load(C::OFF_PA + s * A_P, maps.A, kb * BKP, m0);
           else
-            tma_load_2d(smem + C::OFF_UA + s * C::AU, maps.A, kb * BK, m0, full);
-          if (PA == 2)
-            tma_load_2d(smem + C::OFF_UA + s * C::AU + A_U, maps.A2, kb * BK, m0, full);
+            load(C::OFF_UA + s * C::AU, maps.A, kb * BK, m0);
+          if (PA == 2) load(C::OFF_UA + s * C::AU + A_U, maps.A2, kb * BK, m0);
           if (BPACK)
-            tma_load_2d(smem + C::OFF_PB + s * C::BP, maps.B, kb * BKP, n0, full);
+            load(C::OFF_PB + s * C::BP, maps.B, kb * BKP, n0);
           else
-            tma_load_2d(smem + C::OFF_UB + s * C::BU, maps.B, kb * BK, n0, full);
-          if (PB == 2)
-            tma_load_2d(smem + C::OFF_UB + s * C::BU + BNT * BK, maps.B2, kb * BK, n0, full);
+            load(C::OFF_UB + s * C::BU, maps.B, kb * BK, n0);
+          if (PB == 2) load(C::OFF_UB + s * C::BU + BNT / CG * BK, maps.B2, kb * BK, n0);
           if (++s == S) {
             s = 0;
             phase ^= 1;
           }
         }
       }
-      // On an abort, the copies already in flight must land before exit.
-      if (!ok) {
+      // On an abort, the copies already in flight must land before exit (those
+      // of a pair's second CTA complete on the leader's barriers: it allows
+      // them a millisecond).
+      if (!ok && rank != 0) {
+        const uint64_t t0 = global_timer_ns();
+        while (global_timer_ns() - t0 < 1000000ull) __nanosleep(1000);
+      } else if (!ok) {
         for (int j = max(0, it - S); j < it; ++j)
           mbar_wait_bounded(&bars->tma_full[j % S], (j / S) & 1, nullptr, nullptr, 10000000ull);
       }
     }
     __syncwarp();
   } else if (warp == WARP_MMA) {
-    if (elect_one()) {
-      constexpr uint32_t idesc = F6 ? idesc_f8f6f4_f32(BM, BNT, kFmtE2M3, kFmtE2M3)
-                                    : idesc_e4m3_f32(BM, BNT);
+    if (rank == 0 && elect_one()) {
+      constexpr uint32_t idesc = F6 ? idesc_f8f6f4_f32(TM, BNT, kFmtE2M3, kFmtE2M3)
+                                    : idesc_e4m3_f32(TM, BNT);
       // Operand descriptors of stage 0; a stage, plane or K slice further adds
       // its bytes / 16 to the start-address field.
       const uint64_t adesc = sw128_desc(smem_addr(smem + C::OFF_UA));
@@ -272,7 +302,7 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
       int s = 0, tc = 0;
       uint32_t phase = 0;  // of the stage's ready barrier
       bool ok = true;
-      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++tc) {
+      for (int t = unit; t < tiles && ok; t += units, ++tc) {
         const int buf = SEP ? 0 : (tc & 1);
         const uint32_t use = SEP ? tc : (tc >> 1);  // this buffer's earlier tiles
         if (!mbar_wait_bounded(&bars->acc_empty[buf], (use & 1) ^ 1, abort, g.status,
@@ -302,75 +332,99 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
                 const int acc_i = SEP ? (pa + pb) : 0;
                 const bool first = SEP ? ((kb | k) == 0 && !(pa == 1 && pb == 0))
                                        : (kb | pa | pb | k) == 0;
-                mma_e4m3(d + acc_i * BNT, a0 + (pa * A_U + k * 32) / 16,
-                         b0 + (pb * BNT * BK + k * 32) / 16, idesc, first ? 0u : 1u);
+                mma_e4m3<CG>(d + acc_i * BNT, a0 + (pa * A_U + k * 32) / 16,
+                             b0 + (pb * (BNT / CG) * BK + k * 32) / 16, idesc, first ? 0u : 1u);
               }
-          mma_commit(&bars->mma_done[s]);
+          mma_commit<CG>(&bars->mma_done[s]);
           if (++s == S) {
             s = 0;
             phase ^= 1;
           }
         }
-        if (ok) mma_commit(&bars->acc_full[buf]);
+        if (ok) mma_commit<CG>(&bars->acc_full[buf]);
       }
       // Every MMA issued must complete before TMEM is released.
-      mma_commit(&bars->drained);
+      mma_commit<CG>(&bars->drained);
       mbar_wait_bounded(&bars->drained, 0, nullptr, nullptr, 10000000ull);
     }
     __syncwarp();
-  } else if (warp < 4 || (C::EPI_WARPS == 8 && warp >= 6 && warp < 10)) {
+  } else if (warp < 4 || (C::EPI_WARPS > 4 && warp >= 6 && warp < 2 + C::EPI_WARPS)) {
     // ---- epilogue ----
     const int quarter = warp & 3;
-    const int part = warp < 4 ? 0 : 1;                // 0: warps 0-3, 1: warps 6-9
-    const int et = part * 128 + quarter * 32 + lane;  // 0 .. EPI_THREADS - 1
-    uint8_t* staging = smem + C::OFF_EPI + (part * 4 + quarter) * C::EPI_NBUF * EPI_BYTES;
-    int tc = 0, stores = 0;
-    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++tc) {
-      const int m0 = (t / tiles_n) * BM;
-      const int n0 = (t % tiles_n) * BNT;
+    const int part = warp < 4 ? 0 : 1 + ((warp - 6) >> 2);  // which NCOL columns of the tile
+    const int ew = part * 4 + quarter;
+    constexpr int NCOL = C::EPI_NCOL;
+    const uint32_t empty0 = CG == 2 ? cluster_addr(&bars->acc_empty[0], 0) : 0;  // leader's
+    uint8_t* staging = smem + C::OFF_EPI + ew * EPI_BYTES;
+    float* col = reinterpret_cast<float*>(smem + C::OFF_COL) + ew * C::COL_FLOATS;
+    int tc = 0;
+    for (int t = unit; t < tiles; t += units, ++tc) {
+      const int mb = t / tiles_n;
+      const int m0 = mb * TM + rank * BM;
+      const int n0 = (t - mb * tiles_n) * BNT;
       const int buf = SEP ? 0 : (tc & 1);
       const uint32_t use = SEP ? tc : (tc >> 1);
-      // Column data of this tile into the buffer of its parity; the buffer of
-      // the other parity may still be read by slower warps (previous tile).
-      float* col_scale = reinterpret_cast<float*>(smem + C::OFF_COL) + buf * 3 * BNT;
-      float* col_bias = col_scale + BNT;
-      float* col_zw = col_scale + 2 * BNT;
-      for (int j = et; j < BNT; j += C::EPI_THREADS) {
-        const int col = n0 + j;
+      // This warp's column data and row scales, while the tile's MMAs run.
+#pragma unroll
+      for (int j = lane; j < NCOL; j += 32) {
+        const int cn = n0 + part * NCOL + j;
         float sc = 0.f, bi = 0.f;
-        if (col < g.N) {
-          sc = g.s_w[col] * g.inv_b;
-          if (g.bias != nullptr) bi = Num<OutT>::to_f(static_cast<const uint16_t*>(g.bias)[col]);
+        if (cn < g.N) {
+          sc = g.s_w[cn] * g.inv_b;
+          if (g.bias != nullptr) bi = Num<OutT>::to_f(static_cast<const uint16_t*>(g.bias)[cn]);
         }
-        col_scale[j] = sc;
-        col_bias[j] = bi;
-        if (ASYM) col_zw[j] = col < g.N ? g.wsum[col] * sc : 0.f;
+        col[j] = sc;
+        col[NCOL + j] = bi;
+        if (ASYM) col[2 * NCOL + j] = cn < g.N ? g.wsum[cn] * sc : 0.f;
       }
+      // Row scales: a thread's fragments hold rows 8 k + lane / 4 of the warp's
+      // 32.  Asymmetric codes: the value of code 0 is min + 2^(n-1) delta.
+      float sx[4], zm[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int row = m0 + quarter * EPI_ROWS + 8 * k + (lane >> 2);
+        sx[k] = zm[k] = 0.f;
+        if (ready == nullptr && row < g.M) {
+          sx[k] = __ldg(g.s_x + row);
+          if (ASYM) zm[k] = fmaf(g.zp_shift, sx[k], __ldg(g.lo + row));
+        }
+      }
+      __syncwarp();
       bool ok = mbar_wait_bounded(&bars->acc_full[buf], use & 1, abort, g.status,
                                   kWaitLimitNs);
       ok = __all_sync(0xffffffffu, ok);
-      named_bar_sync(kEpiBarrier, C::EPI_THREADS);  // column data of this tile written
-      if (!ok || *abort != 0) break;
+      if (!ok) break;
       tc_fence_after();
-      // s_x may have been written by other CTAs of this grid (fused kernel):
-      // read it from L2, after the tile's MMAs have completed.
-      const int row = m0 + quarter * 32 + lane;
-      const float sx = row < g.M ? __ldcg(g.s_x + row) : 0.f;
-      // asymmetric codes: the value of code 0 is min + 2^(n-1) delta
-      const float zm = ASYM && row < g.M ? fmaf(g.zp_shift, sx, __ldcg(g.lo + row)) : 0.f;
-      epilogue_part<OutT, C::EPI_NCOL, C::EPI_NBUF, EPI_PREFETCH && !C::UNPACK && !SEP, ASYM,
-                    SEP ? BNT : 0>(
-          tmem + buf * BNT, quarter, part * C::EPI_NCOL, lane, m0, n0, g.M, g.N, sx, col_scale,
-          col_bias, zm, col_zw, staging, maps.Y, g.Y, g.acc_dbg, stores);
-      tc_fence_before();
-      mbar_arrive(&bars->acc_empty[buf]);
+      // In the fused kernel other CTAs of this grid write s_x: it is read from
+      // L2 after the tile's MMAs have completed.
+      if (ready != nullptr) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int row = m0 + quarter * EPI_ROWS + 8 * k + (lane >> 2);
+          if (row < g.M) sx[k] = __ldcg(g.s_x + row);
+        }
+      }
+      epilogue_part<OutT, NCOL, ASYM, SEP ? BNT : 0>(
+          tmem + buf * BNT, quarter, part * NCOL, lane, m0, n0, g.M, g.N, sx, col, zm, staging,
+          maps.Y, g.Y, g.acc_dbg, [&]() {
+            tc_fence_before();
+            __syncwarp();
+            if (elect_one()) {
+              if (CG == 2)
+                mbar_arrive_cluster(empty0 + 8u * buf);
+              else
+                mbar_arrive(&bars->acc_empty[buf]);
+            }
+          });
+      __syncwarp();  // every lane has read this tile's column data
     }
-    if (lane == 0) bulk_wait_all();
+    if (elect_one()) bulk_wait_all();
+    __syncwarp();
   } else if (C::UNPACK && warp >= WARP_UNPACK0 && warp < WARP_UNPACK0 + NUM_UNPACK / 32) {
     const int ut = threadIdx.x - WARP_UNPACK0 * 32;
     int it = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+    for (int t = unit; t < tiles && ok; t += units) {
       for (int kb = 0; kb < nk; ++kb, ++it) {
         const int s = it % S;
         if (!mbar_wait_bounded(&bars->tma_full[s], (it / S) & 1, abort, g.status,
@@ -391,11 +445,12 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
   }
 }
 
-// After a CTA barrier that follows pipeline(): release TMEM.
+// After a CTA (pair: cluster) barrier that follows pipeline(): release TMEM.
+template <int CG = 1>
 __device__ __forceinline__ void teardown(uint32_t tmem, uint32_t cols) {
   if ((threadIdx.x >> 5) == WARP_MMA) {
     tc_fence_after();
-    tmem_dealloc(tmem, cols);
+    tmem_dealloc<CG>(tmem, cols);
   }
 }
 

@@ -1,5 +1,7 @@
-// Standalone W4A4 GEMM kernel (pipeline in gemm_pipeline.cuh), the weight
-// expansion kernel, TMA descriptor helpers and the bounded-wait self test.
+// Launch of the standalone GEMM kernel (gemm_kernel.cuh, instantiated per output
+// type in w4a4_gemm_f16.cu and w4a4_gemm_bf16.cu), the weight expansion kernel,
+// TMA descriptor helpers and the bounded-wait self test.
+#include "gemm_launch.h"
 #include "gemm_pipeline.cuh"
 
 #include <cudaTypedefs.h>
@@ -12,67 +14,9 @@
 
 namespace clq {
 
-namespace {
-
 using namespace gemm;
 
-// W8A8 tiles: three accumulators of 128 columns fill one TMEM allocation.
-constexpr int kSepBN = 128;
-
-template <bool APACK, bool BPACK, int BNT, int PA, int PB, bool SEP = false>
-constexpr size_t smem_bytes() {
-  return Cfg<APACK, BPACK, BNT, PA, PB, 0, MAX_STAGES, SEP>::BYTES + 1024;  // + alignment slack
-}
-
-// PA / PB = 2: the activation / weight codes are 8-bit, as two E4M3 planes
-// (mapA2 / mapB2 the second plane).
-template <typename OutT, bool APACK, bool BPACK, int BNT, int PA, int PB, bool ASYM, bool F6,
-          bool SEP>
-__global__ void __launch_bounds__((Cfg<APACK, BPACK, BNT, PA, PB>::THREADS), 1)
-    w4a4_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
-                     const __grid_constant__ CUtensorMap mapB,
-                     const __grid_constant__ CUtensorMap mapY,
-                     const __grid_constant__ CUtensorMap mapA2,
-                     const __grid_constant__ CUtensorMap mapB2, GemmArgs g, int use_tma_store) {
-  extern __shared__ uint8_t smem_raw[];
-  __shared__ Barriers bars;
-  uint8_t* smem = reinterpret_cast<uint8_t*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  setup<APACK, BPACK, BNT, PA, PB, 0, MAX_STAGES, SEP>(&bars);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = bars.tmem_slot;
-  // The tensor maps are kernel parameters, not outputs of the previous kernel:
-  // fetch them while it finishes (measured +0.25 % on the PixArt step).
-  if (threadIdx.x == WARP_TMA * 32) {
-    prefetch_tensor_map(&mapA);
-    prefetch_tensor_map(&mapB);
-    if (use_tma_store) prefetch_tensor_map(&mapY);
-    // The weight boxes of this CTA's first pipeline stages into L2 (a hint:
-    // it changes no value the copies after the wait read).
-    using C = Cfg<APACK, BPACK, BNT, PA, PB, 0, MAX_STAGES, SEP>;
-    const int tiles_n = (g.N + BNT - 1) / BNT;
-    const int tiles = ((g.M + BM - 1) / BM) * tiles_n;
-    if (!BPACK && static_cast<int>(blockIdx.x) < tiles) {
-      const int n0 = (static_cast<int>(blockIdx.x) % tiles_n) * BNT;
-      const int nk = (g.K + BK - 1) / BK;
-      for (int kb = 0; kb < C::S && kb < nk; ++kb) {
-        tma_prefetch_2d(&mapB, kb * BK, n0);
-        if (PB == 2) tma_prefetch_2d(&mapB2, kb * BK, n0);
-      }
-    }
-  }
-  // Barriers and TMEM are set up; global inputs are read only from here on.
-  pdl_wait();
-  pdl_launch_dependents();
-  const Maps maps{&mapA, &mapB, use_tma_store ? &mapY : nullptr, &mapA2, &mapB2};
-  pipeline<OutT, APACK, BPACK, BNT, true, PA, PB, ASYM, 0, MAX_STAGES, F6, SEP>(
-      maps, g, smem, &bars, tmem, nullptr);
-  tc_fence_before();
-  __syncthreads();
-  teardown(tmem, Cfg<APACK, BPACK, BNT, PA, PB, 0, MAX_STAGES, SEP>::TMEM);
-}
+namespace {
 
 // Packed INT4 weights -> E4M3 execution layout (one code per byte, the byte
 // is the E4M3 encoding of the integer code).  16 packed bytes per thread.
@@ -356,59 +300,6 @@ cudaError_t kernel_setup(const void* func, size_t smem, int threads, int* per_sm
   return cudaSuccess;
 }
 
-namespace {
-
-struct MapSet {
-  CUtensorMap A, B, Y, A2, B2;
-};
-
-template <typename OutT, bool APACK, bool BPACK, int BNT, int PA = 1, int PB = 1,
-          bool ASYM = false, bool F6 = false>
-cudaError_t launch_gemm_t(const MapSet& m, const GemmArgs& g, int use_tma_store, int grid,
-                          cudaStream_t st) {
-  constexpr bool SEP = PA == 2 && PB == 2;  // W8A8: exact plane accumulators
-  auto k = w4a4_gemm_kernel<OutT, APACK, BPACK, BNT, PA, PB, ASYM, F6, SEP>;
-  constexpr size_t smem = smem_bytes<APACK, BPACK, BNT, PA, PB, SEP>();
-  constexpr int threads = Cfg<APACK, BPACK, BNT, PA, PB>::THREADS;
-  cudaError_t e = kernel_setup(reinterpret_cast<const void*>(k), smem, threads, nullptr);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(k, grid, threads, smem, st, m.A, m.B, m.Y, m.A2, m.B2, g, use_tma_store);
-}
-
-template <typename OutT>
-cudaError_t launch_gemm_dt(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes, int bn,
-                           int use_tma_store, int grid, cudaStream_t st) {
-  const bool apack = x_codes == CLQ_CODES_INT4_PACKED;
-  const bool bpack = w_codes == CLQ_CODES_INT4_PACKED;
-  if (x_codes == CLQ_CODES_E2M3) {  // both operands E2M3 (checked by the caller)
-    if (bn == 192)
-      return launch_gemm_t<OutT, false, false, 192, 1, 1, false, true>(m, g, use_tma_store, grid,
-                                                                        st);
-    return launch_gemm_t<OutT, false, false, BN, 1, 1, false, true>(m, g, use_tma_store, grid, st);
-  }
-  if (g.lo != nullptr) {  // asymmetric activations: E4M3 / split operands only
-    if (x_codes == CLQ_CODES_E4M3_SPLIT)
-      return w_codes == CLQ_CODES_E4M3_SPLIT
-                 ? launch_gemm_t<OutT, false, false, kSepBN, 2, 2, true>(m, g, use_tma_store,
-                                                                         grid, st)
-                 : launch_gemm_t<OutT, false, false, BN, 2, 1, true>(m, g, use_tma_store, grid,
-                                                                     st);
-    return launch_gemm_t<OutT, false, false, BN, 1, 1, true>(m, g, use_tma_store, grid, st);
-  }
-  if (x_codes == CLQ_CODES_E4M3_SPLIT)
-    return w_codes == CLQ_CODES_E4M3_SPLIT
-               ? launch_gemm_t<OutT, false, false, kSepBN, 2, 2>(m, g, use_tma_store, grid, st)
-               : launch_gemm_t<OutT, false, false, BN, 2, 1>(m, g, use_tma_store, grid, st);
-  if (apack)
-    return bpack ? launch_gemm_t<OutT, true, true, BN>(m, g, use_tma_store, grid, st)
-                 : launch_gemm_t<OutT, true, false, BN>(m, g, use_tma_store, grid, st);
-  if (bpack) return launch_gemm_t<OutT, false, true, BN>(m, g, use_tma_store, grid, st);
-  if (bn == 192) return launch_gemm_t<OutT, false, false, 192>(m, g, use_tma_store, grid, st);
-  return launch_gemm_t<OutT, false, false, BN>(m, g, use_tma_store, grid, st);
-}
-
-}  // namespace
-
 // TMA map of a code array (rows x K codes) in any layout: packed boxes of 64
 // bytes x box_rows (no swizzle, staged for unpacking), E4M3 boxes of 128
 // bytes x box_rows with the 128-byte swizzle (MMA operand), or E2M3 boxes of
@@ -434,18 +325,18 @@ bool encode_codes_map(CUtensorMap* map, const uint8_t* base, int codes, int rows
                                CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-// Tile width of the E4M3 x E4M3 GEMM: an SM's intake from L2 bounds the
-// kernel, so a tile costs about its operand bytes per K step (A 16 KB + B
-// BN/8 KB), and the CTAs walk ceil(tiles / SMs) rounds.  256 wins unless 192
-// splits N into whole tiles with no more rounds (N = 1152: 6 x 192 instead of
-// 4.5 x 256).  128 measured slower everywhere.
-int gemm_tile_n(int M, int N, int sms) {
-  const long mt = (M + BM - 1) / BM;
-  auto cost = [&](int w) {
-    const long rounds = (mt * ((N + w - 1) / w) + sms - 1) / sms;
-    return rounds * (16.0 + w / 8.0);
+// Tile width of 4-bit execution-layout operands, `units` CTAs or CTA pairs walking
+// tiles of `rows` rows: the units go ceil(tiles / units) rounds, and a K step of
+// a 192-wide tile takes 0.78 of a 256-wide one's (458 against 587 clocks in the
+// pair's main loop alone), so 192 wins where N splits into its tiles with no
+// more rounds (N = 1152: 6 x 192 instead of 4.5 x 256).  128 measured slower
+// everywhere (390 clocks a step).
+int gemm_tile_n(int M, int N, int rows, int units) {
+  const long mt = (M + rows - 1) / rows;
+  auto cost = [&](int w, double step) {
+    return static_cast<double>((mt * ((N + w - 1) / w) + units - 1) / units) * step;
   };
-  return cost(192) < cost(256) ? 192 : BN;
+  return cost(192, 458) < cost(256, 587) ? 192 : BN;
 }
 
 cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, int w_codes,
@@ -455,21 +346,28 @@ cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, i
   const bool apack = x_codes == CLQ_CODES_INT4_PACKED;
   const bool bpack = w_codes == CLQ_CODES_INT4_PACKED;
   const bool split = x_codes == CLQ_CODES_E4M3_SPLIT || w_codes == CLQ_CODES_E4M3_SPLIT;
-  // The tile-width model weighs operand bytes per K step; E2M3 scales both
-  // widths' bytes by the same 3/4, so the choice is the same.
   const bool w8a8 = x_codes == CLQ_CODES_E4M3_SPLIT && w_codes == CLQ_CODES_E4M3_SPLIT;
-  const int bn = w8a8 ? kSepBN
-                      : (!apack && !bpack && !split && g.lo == nullptr) ? gemm_tile_n(g.M, g.N, sms)
-                                                                         : BN;
+  // Operands in an execution layout run on CTA pairs (tcgen05 cta_group::2): each
+  // CTA loads its 128 rows of A and half of B's rows, so a K step brings 32 KB
+  // into an SM instead of 48, six stages fit instead of four, and the L2 reads
+  // and power of a product fall with them (measured against single CTAs with
+  // the same epilogue: 8192 x 3456 x 1152 26.8 -> 23.5 us, 4608 x 3072 x 12288
+  // 110.5 -> 84.6, 65536 x 12288 x 3072 1523 -> 1235; 20 x 480 x 1920 6.9 -> 6.4).
+  TileShape t{apack || bpack ? 1 : 2, BN};
+  if (w8a8)
+    t.bn = kSepBN;
+  else if (!apack && !bpack && !split && g.lo == nullptr)
+    t.bn = gemm_tile_n(g.M, g.N, t.cg * BM, sms / t.cg);
   MapSet m;
+  const int brows = t.bn / t.cg;  // each CTA of a pair loads half of B
   if (!encode_codes_map(&m.A, Xq, x_codes, g.M, g.K, BM, 0) ||
-      !encode_codes_map(&m.B, W, w_codes, g.N, g.K, bn, 0))
+      !encode_codes_map(&m.B, W, w_codes, g.N, g.K, brows, 0))
     return cudaErrorInvalidValue;
   m.A2 = m.A;  // unused unless split
   m.B2 = m.B;
   if (x_codes == CLQ_CODES_E4M3_SPLIT && !encode_codes_map(&m.A2, Xq, x_codes, g.M, g.K, BM, 1))
     return cudaErrorInvalidValue;
-  if (w_codes == CLQ_CODES_E4M3_SPLIT && !encode_codes_map(&m.B2, W, w_codes, g.N, g.K, bn, 1))
+  if (w_codes == CLQ_CODES_E4M3_SPLIT && !encode_codes_map(&m.B2, W, w_codes, g.N, g.K, brows, 1))
     return cudaErrorInvalidValue;
   const int use_tma_store = (g.N % 8 == 0) ? 1 : 0;
   if (use_tma_store) {
@@ -477,11 +375,11 @@ cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, i
   } else {
     m.Y = m.A;  // unused
   }
-  const int tiles = ((g.M + BM - 1) / BM) * ((g.N + bn - 1) / bn);
-  const int grid = std::min(tiles, sms);
+  const int tiles = ((g.M + t.cg * BM - 1) / (t.cg * BM)) * ((g.N + t.bn - 1) / t.bn);
+  const int grid = t.cg * std::min(tiles, sms / t.cg);
   if (out_dtype == CLQ_F16)
-    return launch_gemm_dt<__half>(m, g, x_codes, w_codes, bn, use_tma_store, grid, st);
-  return launch_gemm_dt<__nv_bfloat16>(m, g, x_codes, w_codes, bn, use_tma_store, grid, st);
+    return launch_gemm_f16(m, g, x_codes, w_codes, t, use_tma_store, grid, st);
+  return launch_gemm_bf16(m, g, x_codes, w_codes, t, use_tma_store, grid, st);
 }
 
 cudaError_t launch_convert_codes(const uint8_t* src, int src_codes, uint8_t* dst, int dst_codes,

@@ -1,0 +1,72 @@
+"""The GEMM at the edges of its tiles: CTA pairs share 256-row tiles, 256, 192
+or (W8A8) 128 columns wide, each warp storing 32 x 32 blocks (N % 8 == 0) or
+copying them out by column pairs.  Rows and columns one below, at and one above
+those sizes, in every execution layout, against the oracle: accumulators bit for
+bit, outputs within half an ulp of the output format plus the fp32 epilogue's
+rounding (tests/parity_utils.py)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2509_24416_gb300 import clq
+from parity_utils import check_output_elementwise
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+SETTINGS = {"e4m3": (4, 4, None), "e2m3": (4, 4, clq.CLQ_CODES_E2M3), "w4a8": (8, 4, None),
+            "w8a8": (8, 8, None)}
+
+
+def _values(t, layout, K):
+    """Integer codes of an array, through the library-independent E4M3 table."""
+    e4m3 = {0x00: 0, 0x80: 0}
+    for v in range(1, 129):
+        f, x = np.frexp(float(v))
+        m = (f * 2 - 1) * 8
+        if m == int(m):
+            e4m3[((x - 1 + 7) << 3) | int(m)] = v
+            e4m3[((x - 1 + 7) << 3) | int(m) | 0x80] = -v
+    lut = np.full(256, 999, np.int64)
+    for k, v in e4m3.items():
+        lut[k] = v
+    q = lut[t.cpu().numpy()]
+    assert np.abs(q).max() <= 128
+    return q if layout == clq.CLQ_CODES_E4M3 else q[:, :K] + q[:, K:]
+
+
+@pytest.mark.parametrize("setting", sorted(SETTINGS))
+@pytest.mark.parametrize("M,N,K", [(1, 1, 128), (127, 31, 128), (129, 33, 384), (255, 191, 256),
+                                   (257, 193, 128), (256, 255, 1152), (300, 257, 128), (31, 1003, 256),
+                                   (128, 192, 896), (385, 250, 256)])
+def test_tile_edges(setting, M, N, K):
+    a_bits, w_bits, w_codes = SETTINGS[setting]
+    dtype = "f16" if (M + N) % 2 == 0 else "bf16"
+    td = torch.float16 if dtype == "f16" else torch.bfloat16
+    g = torch.Generator().manual_seed(M * 7919 + N * 31 + K)
+    b = 128
+    X = torch.randn(M, K, generator=g).to(td).to(DEV)
+    W = (0.05 * torch.randn(N, K, generator=g)).to(td).to(DEV)
+    bias = torch.randn(N, generator=g).to(td).to(DEV) if N % 3 else None
+    perm = torch.randperm(K, generator=g).to(torch.int32).to(DEV)
+    layer = clq.PreparedLinear.from_weight(W, perm, b, bias=bias, a_bits=a_bits, w_bits=w_bits,
+                                           w_codes=w_codes)
+    Xq, s_x = clq.rotate_quant_act(X, perm, b, layer.act_codes)
+    # one guard row behind Y: nothing may be written past the last row
+    buf = torch.full(((M + 1) * N,), 7.0, dtype=td, device=DEV)
+    Y, acc = clq.linear(Xq, s_x, layer.We, layer.s_w, b, K, bias, out_dtype=td,
+                        Y=buf[:M * N].view(M, N), with_acc=True)
+    assert clq.device_status() == 0
+    assert bool((buf[M * N:] == 7.0).all())
+    we = layer.We if w_codes is None else clq.convert_codes(layer.We, K, clq.CLQ_CODES_E4M3)
+    xe = Xq if w_codes is None else clq.convert_codes(Xq, K, clq.CLQ_CODES_E4M3)
+    qx = _values(xe, clq.codes_layout(xe, K), K)
+    qw = _values(we, clq.codes_layout(we, K), K)
+    want = oracle.int_gemm(qx, qw)
+    assert np.array_equal(acc.cpu().numpy().astype(np.int64), want)
+    sx, sw = s_x.cpu().numpy(), layer.s_w.cpu().numpy()
+    bb = None if bias is None else bias.float().cpu().numpy()
+    y64 = want * sx.astype(np.float64)[:, None] * sw.astype(np.float64)[None, :] / b
+    if bb is not None:
+        y64 = y64 + bb[None, :]
+    check_output_elementwise(Y.float().cpu().numpy(), y64, want, sx, sw, b, bb, dtype)
