@@ -1,4 +1,5 @@
-"""Build libclq.so (the sm_103a kernels and the C ABI) in-tree with nvcc.
+"""Build libclq.so (the sm_103a kernels and the C ABI) in-tree with nvcc, and
+_clq_host.so (the native form of a layer's call from Python) with g++.
 
 Each .cu under csrc/ compiles to its own object in parallel; the objects
 link into paper_2509_24416_gb300/libclq.so.  Rebuilds only what changed.
@@ -8,12 +9,15 @@ import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libclq.so")
+HOST_SRC = os.path.join(CSRC, "host_layer.cpp")
+HOST = os.path.join(PKG, "_clq_host.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
          "--expt-relaxed-constexpr", "-Xptxas", "-O3"]
@@ -44,8 +48,44 @@ def _compile(src, obj, extra):
     return r.stderr
 
 
+def _host_object():
+    """Object of the host module, named by the torch it was compiled against."""
+    import torch
+    return os.path.join(BUILD, "host_layer-%s.o" % torch.__version__)
+
+
+def _compile_host(obj):
+    import torch
+    root = os.path.dirname(torch.__file__)
+    nvcc = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-I" + os.path.join(root, "include"),
+           "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           "-I" + sysconfig.get_paths()["include"], "-I" + os.path.join(nvcc, "include"),
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+           "-c", HOST_SRC, "-o", obj]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("g++ failed for %s:\n%s%s" % (HOST_SRC, r.stdout, r.stderr))
+    return ""
+
+
+def _link_host(obj):
+    import torch
+    lib = os.path.join(os.path.dirname(torch.__file__), "lib")
+    cmd = ["g++", "-shared", "-o", HOST, obj, "-L" + lib, "-lc10", "-lc10_cuda", "-ltorch_cpu",
+           "-ltorch_python", "-L" + PKG, "-l:" + os.path.basename(LIB),
+           "-Wl,-rpath,$ORIGIN", "-Wl,-rpath," + lib]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("link failed:\n%s%s" % (r.stdout, r.stderr))
+
+
 def build(verbose=False, force=False, extra_flags=()):
     os.makedirs(BUILD, exist_ok=True)
+    host_obj = _host_object()
+    host_new = force or not os.path.exists(host_obj) or os.path.getmtime(host_obj) < max(
+        os.path.getmtime(HOST_SRC),
+        os.path.getmtime(os.path.join(ROOT, "include", "clq.h")))
     srcs = sorted(glob.glob(os.path.join(CSRC, "*.cu")))
     dep_t = _deps()
     jobs = []
@@ -56,10 +96,12 @@ def build(verbose=False, force=False, extra_flags=()):
         if force or not os.path.exists(o) or os.path.getmtime(o) < max(
                 os.path.getmtime(s), dep_t):
             jobs.append((s, o))
-    if jobs:
-        with concurrent.futures.ThreadPoolExecutor(len(jobs)) as ex:
+    if jobs or host_new:
+        with concurrent.futures.ThreadPoolExecutor(len(jobs) + 1) as ex:
             futs = [ex.submit(_compile, s, o, list(extra_flags))
                     for s, o in jobs]
+            if host_new:
+                futs.append(ex.submit(_compile_host, host_obj))
             for f in futs:
                 msg = f.result()
                 if verbose and msg:
@@ -69,6 +111,8 @@ def build(verbose=False, force=False, extra_flags=()):
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("link failed:\n%s%s" % (r.stdout, r.stderr))
+    if host_new or not os.path.exists(HOST) or os.path.getmtime(HOST) < os.path.getmtime(host_obj):
+        _link_host(host_obj)
     return LIB
 
 
