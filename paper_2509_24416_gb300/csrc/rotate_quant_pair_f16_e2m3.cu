@@ -4,10 +4,10 @@
 
 namespace clq {
 
-cudaError_t launch_rotate_quant_pair_f16_e2m3(const RotateQuantArgs& a, int logb, int half,
+cudaError_t launch_rotate_quant_pair_f16_e2m3(const RotateQuantArgs& a, int half,
                                               int threads, size_t smem, int sms,
                                               cudaStream_t st) {
-  return rq::launch_rotate_quant_pair_t<__half, 3>(a, logb, half, threads, smem, sms, st);
+  return rq::launch_rotate_quant_pair_t<__half, 3>(a, half, threads, smem, sms, st);
 }
 
 cudaError_t launch_rotate_quant_wide_f16_e2m3(const RotateQuantArgs& a, int logb, int stage,

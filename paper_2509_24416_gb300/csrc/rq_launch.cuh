@@ -27,14 +27,14 @@ cudaError_t launch_rotate_quant_wide_bf16_e4m3(const RotateQuantArgs& a, int log
 cudaError_t launch_rotate_quant_wide_bf16_e2m3(const RotateQuantArgs& a, int logb, int stage,
                                                int threads, size_t smem, int sms, cudaStream_t st);
 // Paired-row kernel per input type and code layout (rotate_quant_pair_*.cu).
-cudaError_t launch_rotate_quant_pair_f16_e4m3(const RotateQuantArgs& a, int logb, int half,
-                                              int threads, size_t smem, int sms, cudaStream_t st);
-cudaError_t launch_rotate_quant_pair_f16_e2m3(const RotateQuantArgs& a, int logb, int half,
-                                              int threads, size_t smem, int sms, cudaStream_t st);
-cudaError_t launch_rotate_quant_pair_bf16_e4m3(const RotateQuantArgs& a, int logb, int half,
-                                               int threads, size_t smem, int sms, cudaStream_t st);
-cudaError_t launch_rotate_quant_pair_bf16_e2m3(const RotateQuantArgs& a, int logb, int half,
-                                               int threads, size_t smem, int sms, cudaStream_t st);
+cudaError_t launch_rotate_quant_pair_f16_e4m3(const RotateQuantArgs& a, int half, int threads,
+                                              size_t smem, int sms, cudaStream_t st);
+cudaError_t launch_rotate_quant_pair_f16_e2m3(const RotateQuantArgs& a, int half, int threads,
+                                              size_t smem, int sms, cudaStream_t st);
+cudaError_t launch_rotate_quant_pair_bf16_e4m3(const RotateQuantArgs& a, int half, int threads,
+                                               size_t smem, int sms, cudaStream_t st);
+cudaError_t launch_rotate_quant_pair_bf16_e2m3(const RotateQuantArgs& a, int half, int threads,
+                                               size_t smem, int sms, cudaStream_t st);
 
 namespace rq {
 
@@ -77,33 +77,21 @@ cudaError_t launch_pair_geom(const RotateQuantArgs& a, int threads, size_t smem,
   return launch_ex(kern, g, threads, smem, st, a.serial == 0, a);
 }
 
-template <typename T, int CODES, int HALF, bool ROT>
-cudaError_t launch_pair_b(const RotateQuantArgs& a, int logb, int threads, size_t smem, int sms,
-                          cudaStream_t st) {
-  switch (logb) {
-    case 5: return launch_pair_geom<T, 5, CODES, HALF, ROT>(a, threads, smem, sms, st);
-    case 6: return launch_pair_geom<T, 6, CODES, HALF, ROT>(a, threads, smem, sms, st);
-    case 7: return launch_pair_geom<T, 7, CODES, HALF, ROT>(a, threads, smem, sms, st);
-    default: return launch_pair_geom<T, 8, CODES, HALF, ROT>(a, threads, smem, sms, st);
-  }
-}
-
+// The paired kernel for CODES (1 E4M3, 3 E2M3), b = 32; `half` is the half-stage
+// size rotate_quant_pair_config chose.
 template <typename T, int CODES, bool ROT>
-cudaError_t launch_pair_h(const RotateQuantArgs& a, int logb, int half, int threads, size_t smem,
-                          int sms, cudaStream_t st) {
+cudaError_t launch_pair_h(const RotateQuantArgs& a, int half, int threads, size_t smem, int sms,
+                          cudaStream_t st) {
   return half == kPairHalfSmall
-             ? launch_pair_b<T, CODES, kPairHalfSmall, ROT>(a, logb, threads, smem, sms, st)
-             : launch_pair_b<T, CODES, kPairHalfLarge, ROT>(a, logb, threads, smem, sms, st);
+             ? launch_pair_geom<T, 5, CODES, kPairHalfSmall, ROT>(a, threads, smem, sms, st)
+             : launch_pair_geom<T, 5, CODES, kPairHalfLarge, ROT>(a, threads, smem, sms, st);
 }
 
-// The paired kernel for CODES (1 E4M3, 3 E2M3), 32 <= b <= 256; `half` is the
-// half-stage size rotate_quant_pair_config chose.
 template <typename T, int CODES>
-cudaError_t launch_rotate_quant_pair_t(const RotateQuantArgs& a, int logb, int half, int threads,
+cudaError_t launch_rotate_quant_pair_t(const RotateQuantArgs& a, int half, int threads,
                                        size_t smem, int sms, cudaStream_t st) {
-  if (a.rot != nullptr)
-    return launch_pair_h<T, CODES, true>(a, logb, half, threads, smem, sms, st);
-  return launch_pair_h<T, CODES, false>(a, logb, half, threads, smem, sms, st);
+  if (a.rot != nullptr) return launch_pair_h<T, CODES, true>(a, half, threads, smem, sms, st);
+  return launch_pair_h<T, CODES, false>(a, half, threads, smem, sms, st);
 }
 
 // Wide-segment kernel (rq_wide.cuh): a.rows_per_tile = rows of a tile.
@@ -123,14 +111,20 @@ cudaError_t launch_wide_geom(const RotateQuantArgs& a, int threads, size_t smem,
 template <typename T, int CODES, int STAGE, bool ROT>
 cudaError_t launch_wide_b(const RotateQuantArgs& a, int logb, int threads, size_t smem, int sms,
                           cudaStream_t st) {
-  (void)logb;  // b = 64 only
   if constexpr (CODES == 1)
-    if (a.lo != nullptr)
-      return launch_wide_geom<T, 6, CODES, STAGE, ROT, true>(a, threads, smem, sms, st);
-  return launch_wide_geom<T, 6, CODES, STAGE, ROT>(a, threads, smem, sms, st);
+    if (a.lo != nullptr) switch (logb) {
+        case 6: return launch_wide_geom<T, 6, CODES, STAGE, ROT, true>(a, threads, smem, sms, st);
+        case 7: return launch_wide_geom<T, 7, CODES, STAGE, ROT, true>(a, threads, smem, sms, st);
+        default: return launch_wide_geom<T, 8, CODES, STAGE, ROT, true>(a, threads, smem, sms, st);
+      }
+  switch (logb) {
+    case 6: return launch_wide_geom<T, 6, CODES, STAGE, ROT>(a, threads, smem, sms, st);
+    case 7: return launch_wide_geom<T, 7, CODES, STAGE, ROT>(a, threads, smem, sms, st);
+    default: return launch_wide_geom<T, 8, CODES, STAGE, ROT>(a, threads, smem, sms, st);
+  }
 }
 
-// The wide kernel for CODES (1 E4M3, 3 E2M3), b = 64, K % 64 == 0; `stage`
+// The wide kernel for CODES (1 E4M3, 3 E2M3), 64 <= b <= 256; `stage`
 // is the stage size rotate_quant_wide_config chose.
 template <typename T, int CODES>
 cudaError_t launch_rotate_quant_wide_t(const RotateQuantArgs& a, int logb, int stage, int threads,

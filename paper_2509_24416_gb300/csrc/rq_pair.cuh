@@ -64,6 +64,12 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return d;
 }
 
+__device__ __forceinline__ float min3(float a, float b, float c) {
+  float d;
+  asm("min.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 // max_k |v[k]| over the 32 values of a segment (a tree of three-input maxima).
 __device__ __forceinline__ float seg_absmax(const float2 (&v)[16]) {
   float m[11];

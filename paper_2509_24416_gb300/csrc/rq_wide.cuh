@@ -1,21 +1,28 @@
 // Wide-segment rotate-quantize: the hot-path variant of the tile loop for
-// 4-bit activation codes when b >= 64 and K % 64 == 0 (the OBS transform of
-// arxiv 2509.24416 Sec. 3.3 and the per-token quantization of Sec. 3.1 /
-// Eq. 1, symmetric, or asymmetric with the row's minimum and maximum, as in
-// rq_device.cuh).
+// 4-bit activation codes when b >= 64 (the OBS transform of arxiv 2509.24416
+// Sec. 3.3 and the per-token quantization of Sec. 3.1 / Eq. 1, symmetric, or
+// asymmetric with the row's minimum and maximum, as in rq_device.cuh).
 //
 // Each thread owns 64 consecutive permuted positions of one row, so a block
-// of b = 64 is transformed entirely in its registers (b = 128 / 256 keep one /
-// two stages across lanes): the cross-lane shuffles, which load the shared
-// memory pipe as much as the gather does, drop out (b = 64) or halve.  The
-// 64 gather offsets (bytes from the stage start, below 64 KB) are kept two to
-// a register, so the thread holds as many address registers as the 32-wide
-// loop while doing twice the work per tile.  The rest follows rq_pair.cuh:
-// round-robin tiles, STAGES stages in flight, three-input maxima, one CTA
-// barrier per tile, the XOR-ordered gather whose sign flips the store undoes,
-// and a prologue that runs while the previous kernel drains: barriers, an L2
-// prefetch of the first tiles and the gather offsets from the swap vector (a
-// layer constant), with X read only after the programmatic-launch wait.
+// of b = 64 is transformed entirely in its registers; b = 128 / 256 add one /
+// two stages across lanes that exchange half of the registers each.  The
+// cross-lane shuffles, which load the shared-memory pipe as much as the gather
+// does, so drop out (b = 64), or come to half / one an element instead of two /
+// three with 32-wide segments.  The 64 gather offsets (bytes from the stage
+// start, below 64 KB) are kept two to a register, so the thread holds as many
+// address registers as the 32-wide loop while doing twice the work per tile.  The
+// rest follows rq_pair.cuh: round-robin tiles, STAGES stages in flight,
+// three-input maxima, one CTA barrier per tile, the XOR-ordered gather whose sign
+// flips the store undoes, and a prologue that runs while the previous kernel
+// drains: barriers, an L2 prefetch of the first tiles and the gather offsets from
+// the swap vector (a layer constant), with X read only after the
+// programmatic-launch wait.
+//
+// What bounds it: the gather (one 16-bit load an element at scattered columns,
+// about 3 wavefronts a load) and the latencies that 12 warps a SM leave exposed.
+// Measured, back to back, E4M3 codes: 8192 x 1152 8.2 / 9.4 us at b = 64 / 128
+// (copies alone 3.5), 65536 x 1152 44.4 / 52.4, 4608 x 12288 37.5 / 42.2; with
+// 32-wide segments b = 128 took 11.2, 63.0 and 53.2.
 #pragma once
 
 #include "rq_pair.cuh"
@@ -31,85 +38,137 @@ __host__ __device__ inline size_t wide_smem_bytes(int RH, int stage, int stages)
   return static_cast<size_t>(stages) * stage + 24u * RH + 8u + 8u * stages + 16u;
 }
 
-// max_k v[k] and min_k v[k] over the 64 values of a segment.
+// max_k v[k] and min_k v[k] over a thread's 64 values: four chains of three-input
+// maxima and minima (a tree's intermediate values cost registers that the loop
+// does not have).
 __device__ __forceinline__ void wide_minmax(const float2 (&v)[32], float& mx, float& mn) {
-  float a[16], b[16];
+  float a[4], b[4];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    a[i] = max3(fmaxf(v[2 * i].x, v[2 * i].y), v[2 * i + 1].x, v[2 * i + 1].y);
-    b[i] = fminf(fminf(v[2 * i].x, v[2 * i].y), fminf(v[2 * i + 1].x, v[2 * i + 1].y));
+  for (int i = 0; i < 4; ++i) {
+    a[i] = fmaxf(v[i].x, v[i].y);
+    b[i] = fminf(v[i].x, v[i].y);
   }
 #pragma unroll
-  for (int w = 8; w >= 1; w >>= 1)
-#pragma unroll
-    for (int i = 0; i < w; ++i) {
-      a[i] = fmaxf(a[i], a[i + w]);
-      b[i] = fminf(b[i], b[i + w]);
-    }
-  mx = a[0];
-  mn = b[0];
+  for (int i = 4; i < 32; ++i) {
+    a[i & 3] = max3(a[i & 3], v[i].x, v[i].y);
+    b[i & 3] = min3(b[i & 3], v[i].x, v[i].y);
+  }
+  mx = fmaxf(max3(a[0], a[1], a[2]), a[3]);
+  mn = fminf(min3(b[0], b[1], b[2]), b[3]);
 }
 
-// max_k |v[k]| over the 64 values of a segment.
+// max_k |v[k]| over a thread's 64 values, the same way.
 __device__ __forceinline__ float wide_absmax(const float2 (&v)[32]) {
-  float m[22];
+  float m[4];
 #pragma unroll
-  for (int i = 0; i < 21; ++i) {
-    const int e = 3 * i;  // elements e, e + 1, e + 2 of the 64
-    const float x0 = (e & 1) ? v[e >> 1].y : v[e >> 1].x;
-    const float x1 = ((e + 1) & 1) ? v[(e + 1) >> 1].y : v[(e + 1) >> 1].x;
-    const float x2 = ((e + 2) & 1) ? v[(e + 2) >> 1].y : v[(e + 2) >> 1].x;
-    m[i] = max3_abs(x0, x1, x2);
-  }
-  m[21] = fabsf(v[31].y);
-  float n[8];
+  for (int i = 0; i < 4; ++i) m[i] = fmaxf(fabsf(v[i].x), fabsf(v[i].y));
 #pragma unroll
-  for (int i = 0; i < 7; ++i) n[i] = max3(m[3 * i], m[3 * i + 1], m[3 * i + 2]);
-  n[7] = m[21];
-  return max3(max3(n[0], n[1], n[2]), max3(n[3], n[4], n[5]), fmaxf(n[6], n[7]));
+  for (int i = 4; i < 32; ++i) m[i & 3] = max3_abs(m[i & 3], v[i].x, v[i].y);
+  return fmaxf(max3(m[0], m[1], m[2]), m[3]);
 }
 
-// Butterfly stages of a 64-wide segment: strides 2 .. min(b, 64) / 2 in
-// registers (v[k] holds positions 2k, 2k + 1, stride 1 done), then strides
-// 64 .. b / 2 across lanes.
+// Butterfly stages of a 64-wide segment: strides 2 .. 32 in registers (v[k]
+// holds positions 2k, 2k + 1, stride 1 done), then strides 64 .. b / 2 across the
+// 2 or 4 lanes of a block, each stage exchanging half of the registers: lane l
+// and its partner l ^ 1 (l ^ 2) each keep the outputs of one half of the index
+// range, send the other half and form both the sum and the difference of what
+// they then hold, 32 shuffles a stage where keeping one's own segment takes 64.
+// For the partner to hold the other half in the same registers, the last
+// in-register stages of a lane with that bit set leave their sum and difference
+// swapped (a multiplication by -1 that rounds nothing).  Every output is the same
+// sum, rounded in the same order, as with whole segments; differences in lanes
+// with the bit set come out negated, which wide_flip accounts for.
+//
+// Where a register ends up: with X = log2(b) - 6 stages across lanes, register
+// chunk c (registers 16 c .. 16 c + 15) holds the block's positions
+// wide_chunk<X>(c, lane) .. + 15.
 template <int LOGB>
 __device__ __forceinline__ void wide_butterflies(float2 (&v)[32], int lane) {
   const float2 neg1 = make_float2(-1.f, -1.f);
 #pragma unroll
-  for (int hp = 1; hp < 32; hp <<= 1) {
-    if (2 * hp < (1 << LOGB)) {
+  for (int hp = 1; hp < 8; hp <<= 1)
 #pragma unroll
-      for (int k = 0; k < 32; ++k) {
+    for (int k = 0; k < 32; ++k)
+      if ((k & hp) == 0) {
+        const float2 x0 = v[k], x1 = v[k + hp];
+        v[k] = __fadd2_rn(x0, x1);
+        v[k + hp] = __ffma2_rn(x1, neg1, x0);
+      }
+#pragma unroll
+  for (int hp = 8; hp < 32; hp <<= 1) {
+    constexpr int X = LOGB - 6;
+    const int bit = hp == 16 ? 1 : 2;  // lane bit that swaps this stage's outputs
+    if (X >= (hp == 16 ? 1 : 2)) {
+      const float sg = (lane & bit) ? -1.f : 1.f;
+      const float2 p = make_float2(sg, sg), m = make_float2(-sg, -sg);
+#pragma unroll
+      for (int k = 0; k < 32; ++k)
+        if ((k & hp) == 0) {
+          const float2 x0 = v[k], x1 = v[k + hp];
+          v[k] = __ffma2_rn(x1, p, x0);
+          v[k + hp] = __ffma2_rn(x1, m, x0);
+        }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 32; ++k)
         if ((k & hp) == 0) {
           const float2 x0 = v[k], x1 = v[k + hp];
           v[k] = __fadd2_rn(x0, x1);
           v[k + hp] = __ffma2_rn(x1, neg1, x0);
         }
-      }
     }
   }
 #pragma unroll
-  for (int hl = 1; hl < 4; hl <<= 1) {
-    if (LOGB > 6 && hl < (1 << (LOGB > 6 ? LOGB - 6 : 0))) {
-      const float sg = (lane & hl) ? -1.f : 1.f;
-      const float2 sg2 = make_float2(sg, sg);
+  for (int x = 0; x < LOGB - 6; ++x) {
+    const int hp = 16 >> x;  // keep v[k], send v[k + hp]
 #pragma unroll
-      for (int k = 0; k < 32; ++k) {
-        float2 p;
-        p.x = __shfl_xor_sync(0xffffffffu, v[k].x, hl);
-        p.y = __shfl_xor_sync(0xffffffffu, v[k].y, hl);
-        v[k] = __ffma2_rn(v[k], sg2, p);  // lower lane: x + p, upper lane: p - x
+    for (int k = 0; k < 32; ++k)
+      if ((k & hp) == 0) {
+        float2 q;
+        q.x = __shfl_xor_sync(0xffffffffu, v[k + hp].x, 1 << x);
+        q.y = __shfl_xor_sync(0xffffffffu, v[k + hp].y, 1 << x);
+        const float2 own = v[k];
+        v[k] = __fadd2_rn(own, q);
+        v[k + hp] = __ffma2_rn(q, neg1, own);
       }
-    }
   }
 }
 
-// Scale, codes and stores of one row's 64-wide segment; `am` is the row's
-// |x| maximum; bit q of `flip` flips the signs of codes 4q .. 4q + 3.
-template <int CODES, bool ROT>
+// First position, within the block of b = 64 << X, of register chunk c (16
+// registers) after wide_butterflies.
+template <int X>
+__device__ __forceinline__ int wide_chunk(int c, int lane) {
+  if (X == 0) return 16 * c;
+  if (X == 1) return (c >> 1) * 64 + (lane & 1) * 32 + (c & 1) * 16;
+  return (c & 1) * 128 + (c >> 1) * 64 + (lane & 1) * 32 + ((lane >> 1) & 1) * 16;
+}
+
+// Bit q: registers 4 q .. 4 q + 3 hold the negated transform, from the XOR order
+// xm of the gather (output i of a segment gets the sign (-1)^popc(i & xm)) and
+// from the differences of the lanes whose bit is set.
+template <int X>
+__device__ __forceinline__ uint32_t wide_flip(int xm, int lane) {
+  uint32_t flip = 0;
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const int c = q >> 2;
+    const int i = (wide_chunk<X>(c, lane) & 63) + 4 * (q & 3);
+    int neg = __popc(i & xm);
+    if (X >= 1) neg += (c >> 1) & lane;
+    if (X >= 2) neg += c & (lane >> 1);
+    flip |= static_cast<uint32_t>(neg & 1) << q;
+  }
+  return flip;
+}
+
+// Scale, codes and stores of one row's 64 values of a thread; `am` is the row's
+// |x| maximum; bit q of `flip` flips the signs of registers 4q .. 4q + 3.
+template <int CODES, bool ROT, int X>
 __device__ __forceinline__ void wide_quant_store(const RotateQuantArgs& a, float2 (&v)[32],
-                                                 int row, int seg, float am, uint32_t flip) {
+                                                 int row, int seg, float am, uint32_t flip,
+                                                 int lane) {
   const int K = a.K;
+  const int block = (seg >> X) << (6 + X);  // first position of the thread's block
   // s = am / 7 by division by a constant known in advance (Brisebarre,
   // Muller and Raina, IEEE Trans. Computers 53(8), 2004), as in rq_device.cuh
   constexpr float rdiv = 1.0f / 7.0f;
@@ -117,12 +176,12 @@ __device__ __forceinline__ void wide_quant_store(const RotateQuantArgs& a, float
   const float s_row = fmaf(fmaf(-7.0f, q1, am), rdiv, q1);
   if (seg == 0) a.S[row] = s_row;
   if (ROT) {
-    float4* dst = reinterpret_cast<float4*>(a.rot + static_cast<size_t>(row) * K + seg * 64);
+    float* dst = a.rot + static_cast<size_t>(row) * K + block;
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
       const float sg = ((flip >> q) & 1u) ? -1.f : 1.f;
-      dst[q] = make_float4(sg * v[2 * q].x, sg * v[2 * q].y, sg * v[2 * q + 1].x,
-                           sg * v[2 * q + 1].y);
+      *reinterpret_cast<float4*>(dst + wide_chunk<X>(q >> 2, lane) + 4 * (q & 3)) =
+          make_float4(sg * v[2 * q].x, sg * v[2 * q].y, sg * v[2 * q + 1].x, sg * v[2 * q + 1].y);
     }
   }
   // v <- rint(v / s) + 1.5 * 2^23 (ties to even), v / s as v * rcp(s); a zero
@@ -140,13 +199,13 @@ __device__ __forceinline__ void wide_quant_store(const RotateQuantArgs& a, float
   for (int k = 0; k < 32; ++k) v[k] = __ffma2_rn(v[k], rc2, magic);
   const float2 nmagic = make_float2(-12582912.0f, -12582912.0f);
   if constexpr (CODES == 1) {
-    uint4* qrow = reinterpret_cast<uint4*>(a.Q + static_cast<size_t>(row) * K + seg * 64);
+    uint8_t* qrow = a.Q + static_cast<size_t>(row) * K + block;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {  // 16 codes a store
       uint32_t w[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int k = 8 * c + 2 * j;  // v[k], v[k + 1]: codes 2k .. 2k + 3
+        const int k = 8 * c + 2 * j;  // v[k], v[k + 1]: registers 2k .. 2k + 3
         uint16_t e0, e1;
         const float2 q0 = __fadd2_rn(v[k], nmagic), q1v = __fadd2_rn(v[k + 1], nmagic);
         asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(e0) : "f"(q0.y), "f"(q0.x));
@@ -154,35 +213,50 @@ __device__ __forceinline__ void wide_quant_store(const RotateQuantArgs& a, float
         w[j] = (static_cast<uint32_t>(e0) | (static_cast<uint32_t>(e1) << 16)) ^
                ((0u - ((flip >> (k >> 1)) & 1u)) & 0x80808080u);
       }
-      qrow[c] = make_uint4(w[0], w[1], w[2], w[3]);
+      *reinterpret_cast<uint4*>(qrow + wide_chunk<X>(c, lane)) = make_uint4(w[0], w[1], w[2], w[3]);
     }
   } else {
-    // E2M3: 16 codes in 12 bytes (the packing of rq_device.cuh); 64 codes are
-    // 48 bytes, three 16-byte stores
-    uint32_t g[16];
+    // E2M3: 16 codes in 12 bytes (the packing of rq_device.cuh); runs of 64, 32
+    // or 16 codes are 48, 24 or 12 bytes
+    uint8_t* qrow = a.Q + static_cast<size_t>(row) * (3 * K / 4) + 3 * block / 4;
+    constexpr int RUN = 4 >> X;  // consecutive chunks of 16 codes
 #pragma unroll
-    for (int k = 0; k < 32; k += 2) {
-      uint16_t e0, e1;
-      const float2 q0 = __fadd2_rn(v[k], nmagic), q1v = __fadd2_rn(v[k + 1], nmagic);
-      asm("cvt.rn.satfinite.e2m3x2.f32 %0, %1, %2;" : "=h"(e0) : "f"(q0.y), "f"(q0.x));
-      asm("cvt.rn.satfinite.e2m3x2.f32 %0, %1, %2;" : "=h"(e1) : "f"(q1v.y), "f"(q1v.x));
-      uint32_t c = static_cast<uint32_t>(e0) | (static_cast<uint32_t>(e1) << 16);
-      c ^= (0u - ((flip >> (k >> 1)) & 1u)) & 0x20202020u;
-      const uint32_t t = c - 3u * ((c >> 2) & 0x0FC00FC0u);
-      g[k >> 1] = t - 15u * ((t >> 4) & 0x00FFF000u);
-    }
-    uint32_t o[12];
+    for (int c0 = 0; c0 < 4; c0 += RUN) {
+      uint32_t o[3 * RUN];
 #pragma unroll
-    for (int h = 0; h < 4; ++h) {  // each group of 16 codes: g[4h .. 4h + 3] -> 3 words
-      o[3 * h] = g[4 * h] | (g[4 * h + 1] << 24);
-      o[3 * h + 1] = (g[4 * h + 1] >> 8) | (g[4 * h + 2] << 16);
-      o[3 * h + 2] = (g[4 * h + 2] >> 16) | (g[4 * h + 3] << 8);
+      for (int c = 0; c < RUN; ++c) {  // a group of 16 codes -> 3 words
+        uint32_t g[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int k = 8 * (c0 + c) + 2 * j;
+          uint16_t e0, e1;
+          const float2 q0 = __fadd2_rn(v[k], nmagic), q1v = __fadd2_rn(v[k + 1], nmagic);
+          asm("cvt.rn.satfinite.e2m3x2.f32 %0, %1, %2;" : "=h"(e0) : "f"(q0.y), "f"(q0.x));
+          asm("cvt.rn.satfinite.e2m3x2.f32 %0, %1, %2;" : "=h"(e1) : "f"(q1v.y), "f"(q1v.x));
+          uint32_t w = static_cast<uint32_t>(e0) | (static_cast<uint32_t>(e1) << 16);
+          w ^= (0u - ((flip >> (k >> 1)) & 1u)) & 0x20202020u;
+          const uint32_t t = w - 3u * ((w >> 2) & 0x0FC00FC0u);
+          g[j] = t - 15u * ((t >> 4) & 0x00FFF000u);
+        }
+        o[3 * c] = g[0] | (g[1] << 24);
+        o[3 * c + 1] = (g[1] >> 8) | (g[2] << 16);
+        o[3 * c + 2] = (g[2] >> 16) | (g[3] << 8);
+      }
+      uint8_t* q = qrow + 3 * wide_chunk<X>(c0, lane) / 4;
+      if constexpr (RUN == 4) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          reinterpret_cast<uint4*>(q)[j] =
+              make_uint4(o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
+      } else if constexpr (RUN == 2) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          reinterpret_cast<uint2*>(q)[j] = make_uint2(o[2 * j], o[2 * j + 1]);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 3; ++j) reinterpret_cast<uint32_t*>(q)[j] = o[j];
+      }
     }
-    uint4* qrow =
-        reinterpret_cast<uint4*>(a.Q + static_cast<size_t>(row) * (3 * K / 4) + seg * 48);
-    qrow[0] = make_uint4(o[0], o[1], o[2], o[3]);
-    qrow[1] = make_uint4(o[4], o[5], o[6], o[7]);
-    qrow[2] = make_uint4(o[8], o[9], o[10], o[11]);
   }
 }
 
@@ -191,11 +265,12 @@ __device__ __forceinline__ void wide_quant_store(const RotateQuantArgs& a, float
 // 15 by the same division by a constant, q = rint((v - min) / delta) stored
 // centered as q - 8 in E4M3 bytes; kmax / kmin are the row's order keys of
 // max and -min.  v holds the true transform (signs already restored).
-template <bool ROT>
+template <bool ROT, int X>
 __device__ __forceinline__ void wide_quant_store_asym(const RotateQuantArgs& a, float2 (&v)[32],
                                                       int row, int seg, uint32_t kmax,
-                                                      uint32_t kmin) {
+                                                      uint32_t kmin, int lane) {
   const int K = a.K;
+  const int block = (seg >> X) << (6 + X);
   constexpr float div = 15.0f;
   constexpr float rdiv = 1.0f / 15.0f;
   const float row_lo = -order_key_inv(kmin);
@@ -207,10 +282,11 @@ __device__ __forceinline__ void wide_quant_store_asym(const RotateQuantArgs& a, 
     a.lo[row] = row_lo;
   }
   if (ROT) {
-    float4* dst = reinterpret_cast<float4*>(a.rot + static_cast<size_t>(row) * K + seg * 64);
+    float* dst = a.rot + static_cast<size_t>(row) * K + block;
 #pragma unroll
     for (int q = 0; q < 16; ++q)
-      dst[q] = make_float4(v[2 * q].x, v[2 * q].y, v[2 * q + 1].x, v[2 * q + 1].y);
+      *reinterpret_cast<float4*>(dst + wide_chunk<X>(q >> 2, lane) + 4 * (q & 3)) =
+          make_float4(v[2 * q].x, v[2 * q].y, v[2 * q + 1].x, v[2 * q + 1].y);
   }
   // v <- rint((v - min) * 15 / span) + 1.5 * 2^23 - 8 (the centered code in
   // the low mantissa bits); a constant row gets q = 0; a subnormal span takes
@@ -234,7 +310,7 @@ __device__ __forceinline__ void wide_quant_store_asym(const RotateQuantArgs& a, 
     for (int k = 0; k < 32; ++k) v[k] = __ffma2_rn(__fadd2_rn(v[k], nlo), inv2, mg);
   }
   const float2 nmagic = make_float2(-12582912.0f, -12582912.0f);
-  uint4* qrow = reinterpret_cast<uint4*>(a.Q + static_cast<size_t>(row) * K + seg * 64);
+  uint8_t* qrow = a.Q + static_cast<size_t>(row) * K + block;
 #pragma unroll
   for (int c = 0; c < 4; ++c) {  // 16 codes a store
     uint32_t w[4];
@@ -247,7 +323,7 @@ __device__ __forceinline__ void wide_quant_store_asym(const RotateQuantArgs& a, 
       asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(e1) : "f"(q1v.y), "f"(q1v.x));
       w[j] = static_cast<uint32_t>(e0) | (static_cast<uint32_t>(e1) << 16);
     }
-    qrow[c] = make_uint4(w[0], w[1], w[2], w[3]);
+    *reinterpret_cast<uint4*>(qrow + wide_chunk<X>(c, lane)) = make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
@@ -301,10 +377,8 @@ __global__ void __maxnreg__(kWideMaxRegs) rotate_quant_wide_kernel(RotateQuantAr
   // the sign (-1)^popc(i & m) on output i, constant over each 8 codes.
   const bool xor_order = (reinterpret_cast<uintptr_t>(a.perm) & 15u) == 0;
   const int xm = xor_order ? ((8 * (lane >> (LOGB - 6))) & 56) : 0;
-  uint32_t flip = 0;
-#pragma unroll
-  for (int q = 0; q < 16; ++q)
-    if (__popc((4 * q) & xm) & 1) flip |= 1u << q;
+  constexpr int X = LOGB - 6;  // butterfly stages across lanes
+  const uint32_t flip = wide_flip<X>(xm, lane);
   // Gather offsets (bytes from the stage start) of positions (2k) ^ m and
   // (2k + 1) ^ m, low and high halves of ow[k].  An index outside [0, K) is
   // reported and replaced by column 0.
@@ -386,10 +460,12 @@ __global__ void __maxnreg__(kWideMaxRegs) rotate_quant_wide_kernel(RotateQuantAr
       wide_butterflies<LOGB>(v, lane);
       if constexpr (ASYM) {
         // the bounds are signed: restore each 4-code group's sign first
-        if (xor_order) {
+        if (X > 0 || xor_order) {
+          uint32_t f = flip;
+          asm volatile("" : "+r"(f));  // 16 factors kept over the loop would spill
 #pragma unroll
           for (int q = 0; q < 16; ++q) {
-            const float sg = ((flip >> q) & 1u) ? -1.f : 1.f;
+            const float sg = ((f >> q) & 1u) ? -1.f : 1.f;
             const float2 sg2 = make_float2(sg, sg);
             v[2 * q] = __fmul2_rn(v[2 * q], sg2);
             v[2 * q + 1] = __fmul2_rn(v[2 * q + 1], sg2);
@@ -415,11 +491,11 @@ __global__ void __maxnreg__(kWideMaxRegs) rotate_quant_wide_kernel(RotateQuantAr
       // ---- 3. scale, codes, stores --------------------------------------------
       if (active && r < n) {
         if constexpr (ASYM)
-          wide_quant_store_asym<ROT>(a, v, row0 + r, seg, amax[par * RH + r],
-                                     amin[par * RH + r]);
+          wide_quant_store_asym<ROT, X>(a, v, row0 + r, seg, amax[par * RH + r],
+                                        amin[par * RH + r], lane);
         else
-          wide_quant_store<CODES, ROT>(a, v, row0 + r, seg,
-                                       __uint_as_float(amax[par * RH + r]), flip);
+          wide_quant_store<CODES, ROT, X>(a, v, row0 + r, seg,
+                                          __uint_as_float(amax[par * RH + r]), flip, lane);
       }
       if (tid < RH) {
         amax[((j + 2) % 3) * RH + tid] = 0u;

@@ -1,0 +1,72 @@
+"""The wide rotate-quantize loop (b = 64, 128, 256; symmetric E4M3 and E2M3 codes,
+asymmetric E4M3 codes) against the general loop on the same rows, which writes
+packed nibbles: both form every output by the same sums in the same order, so
+codes, scales, bounds and rotated rows agree bit for bit (a zero code may be
+written as either zero)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2509_24416_gb300 import clq
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+E4M3_INT = {0x00: 0, 0x38: 1, 0x40: 2, 0x44: 3, 0x48: 4, 0x4A: 5, 0x4C: 6, 0x4E: 7, 0x50: 8}
+
+
+def _lut():
+    t = torch.full((256,), 99, dtype=torch.int16)
+    for byte, v in E4M3_INT.items():
+        t[byte] = v
+        t[byte | 0x80] = -v
+    return t.to(DEV)
+
+
+def _nibbles(p):
+    lo, hi = (p & 15).to(torch.int16), (p >> 4).to(torch.int16)
+    q = torch.stack([lo, hi], dim=2).reshape(p.shape[0], -1)
+    return torch.where(q >= 8, q - 16, q)
+
+
+def _rows(M, K, dtype, seed):
+    g = torch.Generator().manual_seed(seed)
+    x = torch.randn(M, K, generator=g)
+    x[:, torch.randperm(K, generator=g)[:3]] *= 40
+    x[M // 2] = 0  # a zero row
+    x[M - 1, :] = 0
+    x[M - 1, K // 3] = -1e-7 if dtype == torch.float16 else -1e-39  # a spike in the subnormals
+    if M > 2:
+        x[1] = 5.0  # every block sums to one large value and zeros
+    return x.to(dtype).to(DEV)
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+@pytest.mark.parametrize("b,K", [(64, 64), (64, 192), (64, 1152), (128, 128), (128, 1152), (128, 4736),
+                                 (256, 256), (256, 1280), (256, 12288), (128, 16384)])
+@pytest.mark.parametrize("M", [1, 7, 300])
+def test_wide_equals_general(b, K, M, dtype):
+    X = _rows(M, K, dtype, b + K + M)
+    perm = torch.randperm(K, generator=torch.Generator().manual_seed(K)).to(torch.int32).to(DEV)
+    shifted = torch.empty(K + 1, dtype=torch.int32, device=DEV)[1:].copy_(perm)  # 4-byte aligned
+    wide = torch.zeros(M, K + 8, dtype=dtype, device=DEV)
+    wide[:, :K] = X
+    lut = _lut()
+    want, s_want, rot_want = clq.rotate_quant_act(X, perm, b, with_rot=True)
+    want = _nibbles(want)
+    a_want, d_want, l_want = clq.rotate_quant_act_asym(X, perm, b, codes=clq.CLQ_CODES_INT4_PACKED)
+    a_want = _nibbles(a_want)
+    for p in (perm, shifted):
+        for x in (X, wide[:, :K]):
+            q, s = clq.rotate_quant_act(x, p, b, clq.CLQ_CODES_E4M3)
+            assert torch.equal(lut[q.long()], want) and torch.equal(s, s_want)
+            q, d, lo = clq.rotate_quant_act_asym(x, p, b)
+            assert torch.equal(lut[q.long()], a_want)
+            assert torch.equal(d, d_want) and torch.equal(lo, l_want)
+            if K % 128 == 0:
+                q, s = clq.rotate_quant_act(x, p, b, clq.CLQ_CODES_E2M3)
+                packed = clq.convert_codes(q, K, clq.CLQ_CODES_INT4_PACKED)
+                assert torch.equal(_nibbles(packed), want) and torch.equal(s, s_want)
+    q, s, rot = clq.rotate_quant_act(X, perm, b, clq.CLQ_CODES_E4M3, with_rot=True)
+    assert torch.equal(rot, rot_want) and torch.equal(lut[q.long()], want)
+    assert clq.device_status() == 0
+    assert np.isfinite(s.cpu().numpy()).all()
