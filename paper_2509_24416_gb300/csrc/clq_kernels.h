@@ -60,9 +60,10 @@ struct GemmArgs {
 // ([rows][K/2]), CLQ_CODES_E4M3 ([rows][K]) or, for 8-bit codes,
 // CLQ_CODES_E4M3_SPLIT ([rows][2][K]; A split with B E4M3 or split); TMA maps
 // are built here.
-// Output-channel tile width (192 or 256) of the product of 4-bit
-// execution-layout operands, tiles of `rows` rows dealt to `units` CTAs or pairs.
-int gemm_tile_n(int M, int N, int rows, int units);
+// Output-channel tile width (256, 192, 128 or 64) of the product of
+// execution-layout operands, tiles of `rows` rows dealt to `units` CTAs or pairs;
+// mid: 192 is built for them, narrow: 128 and 64 are.
+int gemm_tile_n(int M, int N, int K, int rows, int units, bool mid, bool narrow);
 cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, int w_codes,
                              const GemmArgs& g, int out_dtype, cudaStream_t st);
 

@@ -231,7 +231,7 @@ cudaError_t launch_concurrent(const RotateQuantArgs& rq_in, const uint8_t* W, in
   const int R = std::min(kTeamCompute / segs, kConcStride / (2 * rq.K));
   if (R < 1) return cudaErrorInvalidValue;
   rq.rows_per_tile = R;
-  const int bn = gemm_tile_n(g.M, g.N, BM, sms);
+  const int bn = gemm_tile_n(g.M, g.N, g.K, BM, sms, true, false);
   const size_t gemm_off = bn == 192 ? Conc<192>::RQ_OFF : Conc<256>::RQ_OFF;
   const size_t smem = gemm_off + rq::smem_bytes(R, kConcStride, kConcStages) + 1024;
   if (smem > 227u * 1024u - 2048u) return cudaErrorInvalidValue;

@@ -1,6 +1,6 @@
 // Standalone GEMM kernel around gemm::pipeline and its launch for every operand
-// layout and tile shape; included once per output type so that the variants
-// compile in parallel.
+// layout and tile shape; included once per operand family and output type so that
+// the variants compile in parallel.
 #pragma once
 
 #include "gemm_launch.h"
@@ -91,36 +91,62 @@ cudaError_t launch_gemm_t(const MapSet& m, const GemmArgs& g, int use_tma_store,
 }
 
 // CTA pairs for operands in an execution layout, single CTAs for packed ones
-// (whose unpack warps work on a whole tile's operands); t.bn is the tile width
-// that gemm_tile chose.
+// (whose unpack warps work on a whole tile's operands).
+#define CLQ_GO(...) return launch_gemm_t<OutT, __VA_ARGS__>(m, g, use_tma_store, grid, st)
+
 template <typename OutT>
-cudaError_t launch_gemm_dt(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
-                           TileShape t, int use_tma_store, int grid, cudaStream_t st) {
+cudaError_t launch_gemm_e4m3(const MapSet& m, const GemmArgs& g, int, int, TileShape t,
+                             int use_tma_store, int grid, cudaStream_t st) {
+  switch (t.bn) {
+    case 64: CLQ_GO(false, false, 64, 2);
+    case 128: CLQ_GO(false, false, 128, 2);
+    case 192: CLQ_GO(false, false, 192, 2);
+    default: CLQ_GO(false, false, 256, 2);
+  }
+}
+
+template <typename OutT>
+cudaError_t launch_gemm_e2m3(const MapSet& m, const GemmArgs& g, int, int, TileShape t,
+                             int use_tma_store, int grid, cudaStream_t st) {
+  switch (t.bn) {
+    case 64: CLQ_GO(false, false, 64, 2, 1, 1, false, true);
+    case 128: CLQ_GO(false, false, 128, 2, 1, 1, false, true);
+    case 192: CLQ_GO(false, false, 192, 2, 1, 1, false, true);
+    default: CLQ_GO(false, false, 256, 2, 1, 1, false, true);
+  }
+}
+
+template <typename OutT>
+cudaError_t launch_gemm_bits(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
+                             TileShape t, int use_tma_store, int grid, cudaStream_t st) {
+  const bool a8 = x_codes == CLQ_CODES_E4M3_SPLIT, w8 = w_codes == CLQ_CODES_E4M3_SPLIT;
+  if (g.lo != nullptr) {  // asymmetric activations
+    if (a8 && w8) CLQ_GO(false, false, 128, 2, 2, 2, true);
+    if (a8) CLQ_GO(false, false, 256, 2, 2, 1, true);
+    switch (t.bn) {
+      case 64: CLQ_GO(false, false, 64, 2, 1, 1, true);
+      case 128: CLQ_GO(false, false, 128, 2, 1, 1, true);
+      default: CLQ_GO(false, false, 256, 2, 1, 1, true);
+    }
+  }
+  if (w8) CLQ_GO(false, false, 128, 2, 2, 2);
+  switch (t.bn) {
+    case 64: CLQ_GO(false, false, 64, 2, 2, 1);
+    case 128: CLQ_GO(false, false, 128, 2, 2, 1);
+    default: CLQ_GO(false, false, 256, 2, 2, 1);
+  }
+}
+
+template <typename OutT>
+cudaError_t launch_gemm_packed(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
+                               TileShape, int use_tma_store, int grid, cudaStream_t st) {
   const bool apack = x_codes == CLQ_CODES_INT4_PACKED;
   const bool bpack = w_codes == CLQ_CODES_INT4_PACKED;
-#define CLQ_GO(...) return launch_gemm_t<OutT, __VA_ARGS__>(m, g, use_tma_store, grid, st)
-  if (x_codes == CLQ_CODES_E2M3) {  // both operands E2M3 (checked by the caller)
-    if (t.bn == 192) CLQ_GO(false, false, 192, 2, 1, 1, false, true);
-    CLQ_GO(false, false, BN, 2, 1, 1, false, true);
-  }
-  if (g.lo != nullptr) {  // asymmetric activations: E4M3 / split operands only
-    if (x_codes == CLQ_CODES_E4M3_SPLIT) {
-      if (w_codes == CLQ_CODES_E4M3_SPLIT) CLQ_GO(false, false, kSepBN, 2, 2, 2, true);
-      CLQ_GO(false, false, BN, 2, 2, 1, true);
-    }
-    CLQ_GO(false, false, BN, 2, 1, 1, true);
-  }
-  if (x_codes == CLQ_CODES_E4M3_SPLIT) {
-    if (w_codes == CLQ_CODES_E4M3_SPLIT) CLQ_GO(false, false, kSepBN, 2, 2, 2);
-    CLQ_GO(false, false, BN, 2, 2, 1);
-  }
   if (apack && bpack) CLQ_GO(true, true, BN);
   if (apack) CLQ_GO(true, false, BN);
-  if (bpack) CLQ_GO(false, true, BN);
-  if (t.bn == 192) CLQ_GO(false, false, 192, 2);
-  CLQ_GO(false, false, BN, 2);
-#undef CLQ_GO
+  CLQ_GO(false, true, BN);
 }
+#undef CLQ_GO
 
 }  // namespace
 }  // namespace clq

@@ -6,22 +6,39 @@
 
 namespace clq {
 
-// W8A8 tiles: three accumulators of 128 columns fill one TMEM allocation.
-constexpr int kSepBN = 128;
-
 // Tensor maps of a launch: operands, output, second planes of 8-bit operands.
 struct MapSet {
   CUtensorMap A, B, Y, A2, B2;
 };
 
-// Tile shape of a launch: cg * 128 rows (a CTA or a CTA pair) x bn columns.
+// Tile shape of a launch: cg * 128 rows (a CTA or a CTA pair) x bn columns (256,
+// 192, 128 or 64 for execution-layout operands, 256 for packed ones, 128 or 64
+// for W8A8).
 struct TileShape {
   int cg, bn;
 };
 
-cudaError_t launch_gemm_f16(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
-                            TileShape t, int use_tma_store, int grid, cudaStream_t st);
-cudaError_t launch_gemm_bf16(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
-                             TileShape t, int use_tma_store, int grid, cudaStream_t st);
+// One launcher per operand family and output type, each in its own translation
+// unit (gemm_*.cu) so that they compile in parallel:
+//   e4m3: E4M3 x E4M3, symmetric
+//   e2m3: E2M3 x E2M3
+//   bits: 8-bit (split) activations, symmetric or asymmetric, and asymmetric 4-bit E4M3
+//   packed: packed nibbles on either side
+cudaError_t launch_gemm_e4m3_f16(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
+                                 TileShape t, int use_tma_store, int grid, cudaStream_t st);
+cudaError_t launch_gemm_e4m3_bf16(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
+                                  TileShape t, int use_tma_store, int grid, cudaStream_t st);
+cudaError_t launch_gemm_e2m3_f16(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
+                                 TileShape t, int use_tma_store, int grid, cudaStream_t st);
+cudaError_t launch_gemm_e2m3_bf16(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
+                                  TileShape t, int use_tma_store, int grid, cudaStream_t st);
+cudaError_t launch_gemm_bits_f16(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
+                                 TileShape t, int use_tma_store, int grid, cudaStream_t st);
+cudaError_t launch_gemm_bits_bf16(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
+                                  TileShape t, int use_tma_store, int grid, cudaStream_t st);
+cudaError_t launch_gemm_packed_f16(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
+                                   TileShape t, int use_tma_store, int grid, cudaStream_t st);
+cudaError_t launch_gemm_packed_bf16(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
+                                    TileShape t, int use_tma_store, int grid, cudaStream_t st);
 
 }  // namespace clq

@@ -1,5 +1,5 @@
-// Launch of the standalone GEMM kernel (gemm_kernel.cuh, instantiated per output
-// type in w4a4_gemm_f16.cu and w4a4_gemm_bf16.cu), the weight expansion kernel,
+// Launch of the standalone GEMM kernel (gemm_kernel.cuh, instantiated per operand
+// family and output type in gemm_*.cu), the weight expansion kernel,
 // TMA descriptor helpers and the bounded-wait self test.
 #include "gemm_launch.h"
 #include "gemm_pipeline.cuh"
@@ -325,18 +325,37 @@ bool encode_codes_map(CUtensorMap* map, const uint8_t* base, int codes, int rows
                                CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
-// Tile width of 4-bit execution-layout operands, `units` CTAs or CTA pairs walking
-// tiles of `rows` rows: the units go ceil(tiles / units) rounds, and a K step of
-// a 192-wide tile takes 0.78 of a 256-wide one's (458 against 587 clocks in the
-// pair's main loop alone), so 192 wins where N splits into its tiles with no
-// more rounds (N = 1152: 6 x 192 instead of 4.5 x 256).  128 measured slower
-// everywhere (390 clocks a step).
-int gemm_tile_n(int M, int N, int rows, int units) {
+// Tile width of execution-layout operands, `units` CTAs or CTA pairs walking tiles
+// of `rows` rows.  The units go ceil(tiles / units) rounds; a tile takes its K
+// steps (clocks a step of a pair's main loop, measured alone: 587 / 458 / 390 for
+// 256 / 192 / 128 columns, and what 20 KB of operands take to arrive for 64) or
+// its epilogue, whichever is longer, and the last one's epilogue comes on top
+// (1000 clocks a 32-column block, a quarter of the columns each).  256 wins on
+// large products, 192 where N splits into its tiles with no more rounds (N =
+// 1152: 6 x 192 instead of 4.5 x 256), 128 and 64 where the wider tiles leave
+// units idle (us at 256 / 192 / 128 / 64 columns: 256 x 1152 x 1152 6.8 / 5.8 /
+// 4.9 / 4.4, 256 x 3072 x 12288 29.6 / 22.9 / 16.4 / 16.1, 1024 x 4608 x 1152 7.8 /
+// 8.1 / 7.6 / 9.6, 2048 x 4608 x 1152 10.6 / 10.6 / 11.0 / 15.1, 8192 x 1152 x
+// 4608 34.0 / 27.6 / 28.0 / 44.6; this rule is within 4 % of the best of them on 15
+// such shapes in each layout).  `narrow`: 64 and 128 are built for these operands; `mid`: 192 is.
+int gemm_tile_n(int M, int N, int K, int rows, int units, bool mid, bool narrow) {
   const long mt = (M + rows - 1) / rows;
-  auto cost = [&](int w, double step) {
-    return static_cast<double>((mt * ((N + w - 1) / w) + units - 1) / units) * step;
-  };
-  return cost(192, 458) < cost(256, 587) ? 192 : BN;
+  const double nk = (K + BK - 1) / BK;
+  const int width[4] = {256, 192, 128, 64};
+  const double step[4] = {587, 458, 390, 300};
+  int best = BN;
+  double best_cost = 1e300;
+  for (int i = 0; i < 4; ++i) {
+    if ((width[i] == 192 && !mid) || (width[i] < 192 && !narrow)) continue;
+    const long rounds = (mt * ((N + width[i] - 1) / width[i]) + units - 1) / units;
+    const double epi = 1000.0 * width[i] / 64;
+    const double cost = rounds * std::max(nk * step[i], epi + 500) + epi;
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = width[i];
+    }
+  }
+  return best;
 }
 
 cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, int w_codes,
@@ -355,9 +374,9 @@ cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, i
   // 110.5 -> 84.6, 65536 x 12288 x 3072 1523 -> 1235; 20 x 480 x 1920 6.9 -> 6.4).
   TileShape t{apack || bpack ? 1 : 2, BN};
   if (w8a8)
-    t.bn = kSepBN;
-  else if (!apack && !bpack && !split && g.lo == nullptr)
-    t.bn = gemm_tile_n(g.M, g.N, t.cg * BM, sms / t.cg);
+    t.bn = 128;  // three accumulators of 128 columns fill one TMEM allocation
+  else if (!apack && !bpack && !(split && g.lo != nullptr))
+    t.bn = gemm_tile_n(g.M, g.N, g.K, t.cg * BM, sms / t.cg, !split && g.lo == nullptr, true);
   MapSet m;
   const int brows = t.bn / t.cg;  // each CTA of a pair loads half of B
   if (!encode_codes_map(&m.A, Xq, x_codes, g.M, g.K, BM, 0) ||
@@ -377,9 +396,12 @@ cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, i
   }
   const int tiles = ((g.M + t.cg * BM - 1) / (t.cg * BM)) * ((g.N + t.bn - 1) / t.bn);
   const int grid = t.cg * std::min(tiles, sms / t.cg);
-  if (out_dtype == CLQ_F16)
-    return launch_gemm_f16(m, g, x_codes, w_codes, t, use_tma_store, grid, st);
-  return launch_gemm_bf16(m, g, x_codes, w_codes, t, use_tma_store, grid, st);
+  const bool f16 = out_dtype == CLQ_F16;
+  auto* go = apack || bpack                ? (f16 ? launch_gemm_packed_f16 : launch_gemm_packed_bf16)
+             : x_codes == CLQ_CODES_E2M3   ? (f16 ? launch_gemm_e2m3_f16 : launch_gemm_e2m3_bf16)
+             : split || g.lo != nullptr    ? (f16 ? launch_gemm_bits_f16 : launch_gemm_bits_bf16)
+                                           : (f16 ? launch_gemm_e4m3_f16 : launch_gemm_e4m3_bf16);
+  return go(m, g, x_codes, w_codes, t, use_tma_store, grid, st);
 }
 
 cudaError_t launch_convert_codes(const uint8_t* src, int src_codes, uint8_t* dst, int dst_codes,

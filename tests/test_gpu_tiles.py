@@ -1,5 +1,5 @@
-"""The GEMM at the edges of its tiles: CTA pairs share 256-row tiles, 256, 192
-or (W8A8) 128 columns wide, each warp storing 32 x 32 blocks (N % 8 == 0) or
+"""The GEMM at the edges of its tiles: CTA pairs share 256-row tiles, 256, 192,
+128 or 64 columns wide, each warp storing 32 x 32 blocks (N % 8 == 0) or
 copying them out by column pairs.  Rows and columns one below, at and one above
 those sizes, in every execution layout, against the oracle: accumulators bit for
 bit, outputs within half an ulp of the output format plus the fp32 epilogue's
@@ -70,3 +70,51 @@ def test_tile_edges(setting, M, N, K):
     if bb is not None:
         y64 = y64 + bb[None, :]
     check_output_elementwise(Y.float().cpu().numpy(), y64, want, sx, sw, b, bb, dtype)
+
+
+@pytest.mark.parametrize("setting", sorted(SETTINGS) + ["asym"])
+@pytest.mark.parametrize("M,N,K", [(4001, 2051, 1152), (2600, 2504, 896), (4601, 1501, 1152),
+                                   (300, 8195, 256)])
+def test_tile_widths(setting, M, N, K):
+    """Shapes for which the launcher takes 256, 128, 192 and 64 columns (where the
+    setting has them), several tiles a unit, against fp64 products of the codes on
+    the GPU (integers, so exact)."""
+    a_bits, w_bits, w_codes = SETTINGS.get(setting, (4, 4, None))
+    g = torch.Generator(device=DEV).manual_seed(M)
+    b = 128
+    X = torch.randn(M, K, generator=g, device=DEV).half()
+    W = (0.05 * torch.randn(N, K, generator=g, device=DEV)).half()
+    bias = torch.randn(N, generator=g, device=DEV).half()
+    perm = torch.randperm(K, generator=g, device=DEV).to(torch.int32)
+    layer = clq.PreparedLinear.from_weight(W, perm, b, bias=bias, a_bits=a_bits, w_bits=w_bits,
+                                           w_codes=w_codes)
+    if setting == "asym":
+        Xq, s_x, lo = clq.rotate_quant_act_asym(X, perm, b)
+        wsum = clq.weight_code_sums(layer.We, K)
+        Y, acc = clq.linear_asym(Xq, s_x, lo, layer.We, layer.s_w, wsum, b, K, bias, with_acc=True)
+    else:
+        Xq, s_x = clq.rotate_quant_act(X, perm, b, layer.act_codes)
+        Y, acc = clq.linear(Xq, s_x, layer.We, layer.s_w, b, K, bias, with_acc=True)
+    assert clq.device_status() == 0
+
+    def codes(t):
+        if w_codes is not None:
+            t = clq.convert_codes(t, K, clq.CLQ_CODES_E4M3)
+        q = torch.from_numpy(_values(t, clq.codes_layout(t, K), K))
+        return q.to(DEV).double()
+
+    qx, qw = codes(Xq), codes(layer.We)
+    want = qx @ qw.t()
+    assert torch.equal(acc.double(), want)
+    scale = layer.s_w.double()[None, :] / b
+    y64 = want * s_x.double()[:, None] * scale
+    size = y64.abs()
+    if setting == "asym":
+        zp = (lo.double() + 8 * s_x.double())[:, None] * qw.sum(1)[None, :] * scale
+        y64 = y64 + zp
+        size = size + zp.abs()
+    y64 = y64 + bias.double()[None, :]
+    size = size + bias.double().abs()[None, :]
+    # half an ulp of fp16, three fp32 roundings of the terms, the smallest subnormal
+    err = (Y.double() - y64).abs()
+    assert bool((err <= 2.0 ** -11 * y64.abs() + 1e-6 * size + 2.0 ** -24).all())
