@@ -187,10 +187,10 @@ __device__ __forceinline__ void store_block_direct(const uint8_t* staging, int l
 // eight-byte loads of column data a warp where one row a lane took 16
 // sixteen-byte ones; the packed pairs leave by stmatrix.
 //
-// SEP3 > 0: the accumulator is the sum of three TMEM accumulators SEP3
+// SEP > 0: the accumulator is the sum of SEP (2 or 3) TMEM accumulators BNT
 // columns apart, each an exact integer in fp32 (the W8A8 plane products); they
 // are added as int32 and the block goes on with that (exact) sum.
-template <typename OutT, int NCOL, bool ASYM, int SEP3, typename Release>
+template <typename OutT, int NCOL, bool ASYM, int SEP, int BNT, typename Release>
 __device__ __forceinline__ void epilogue_part(uint32_t tmem_acc, int quarter, int col0, int lane,
                                               int m0, int n0, int M, int N, const float (&sx)[4],
                                               const float* col, const float (&zm)[4],
@@ -223,20 +223,22 @@ __device__ __forceinline__ void epilogue_part(uint32_t tmem_acc, int quarter, in
     }
     tmem_ld_wait_tie(r[0]);
     tmem_ld_wait_tie(r[1]);
-    if constexpr (SEP3 > 0) {
+    if constexpr (SEP > 0) {
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
-        uint32_t r1[16], r2[16];
         const uint32_t at = lane_base + (static_cast<uint32_t>(half * 16) << 16) + c;
-        tmem_ld_frag(at + SEP3, r1);
-        tmem_ld_frag(at + 2 * SEP3, r2);
-        tmem_ld_wait_tie(r1);
-        tmem_ld_wait_tie(r2);
+        uint32_t r1[SEP - 1][16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-          r[half][j] = static_cast<uint32_t>(__float2int_rn(__uint_as_float(r[half][j])) +
-                                             __float2int_rn(__uint_as_float(r1[j])) +
-                                             __float2int_rn(__uint_as_float(r2[j])));
+        for (int p = 1; p < SEP; ++p) tmem_ld_frag(at + p * BNT, r1[p - 1]);
+#pragma unroll
+        for (int p = 1; p < SEP; ++p) tmem_ld_wait_tie(r1[p - 1]);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          int sum = __float2int_rn(__uint_as_float(r[half][j]));
+#pragma unroll
+          for (int p = 1; p < SEP; ++p) sum += __float2int_rn(__uint_as_float(r1[p - 1][j]));
+          r[half][j] = static_cast<uint32_t>(sum);
+        }
       }
     }
     if (i == nblk - 1) release();
@@ -250,7 +252,7 @@ __device__ __forceinline__ void epilogue_part(uint32_t tmem_acc, int quarter, in
           const uint32_t v = r[k >> 1][4 * (j >> 1) + 2 * (k & 1) + (j & 1)];
           if (row < M && cn < N)
             acc_dbg[static_cast<size_t>(row) * N + cn] =
-                SEP3 > 0 ? static_cast<int32_t>(v) : __float2int_rn(__uint_as_float(v));
+                SEP > 0 ? static_cast<int32_t>(v) : __float2int_rn(__uint_as_float(v));
         }
     }
     // The store that last used the staging buffer has finished reading it.
@@ -264,7 +266,7 @@ __device__ __forceinline__ void epilogue_part(uint32_t tmem_acc, int quarter, in
       for (int g = 0; g < 4; ++g) {
         const uint32_t v0 = r[k >> 1][4 * g + 2 * (k & 1)];
         const uint32_t v1 = r[k >> 1][4 * g + 2 * (k & 1) + 1];
-        const float2 acc = SEP3 > 0 ? make_float2(static_cast<float>(static_cast<int32_t>(v0)),
+        const float2 acc = SEP > 0 ? make_float2(static_cast<float>(static_cast<int32_t>(v0)),
                                                   static_cast<float>(static_cast<int32_t>(v1)))
                                     : make_float2(__uint_as_float(v0), __uint_as_float(v1));
         const float2 bias = ASYM ? __ffma2_rn(make_float2(zm[k], zm[k]), cz[g], cb[g]) : cb[g];

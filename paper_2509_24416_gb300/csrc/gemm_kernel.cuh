@@ -11,14 +11,14 @@ namespace {
 
 using namespace gemm;
 
-template <bool APACK, bool BPACK, int BNT, int PA, int PB, bool SEP, int CG>
+template <bool APACK, bool BPACK, int BNT, int PA, int PB, int SEP, int CG>
 using KernelCfg = Cfg<APACK, BPACK, BNT, PA, PB, 0, MAX_STAGES, SEP, CG>;
 
 // PA / PB = 2: the activation / weight codes are 8-bit, as two E4M3 planes
 // (mapA2 / mapB2 the second plane).  CG 2: launched as clusters of two CTAs,
 // each pair sharing 256 x BNT tiles (tcgen05 cta_group::2).
 template <typename OutT, bool APACK, bool BPACK, int BNT, int PA, int PB, bool ASYM, bool F6,
-          bool SEP, int CG>
+          int SEP, int CG>
 __global__ void __launch_bounds__((KernelCfg<APACK, BPACK, BNT, PA, PB, SEP, CG>::THREADS), 1)
     w4a4_gemm_kernel(const __grid_constant__ CUtensorMap mapA,
                      const __grid_constant__ CUtensorMap mapB,
@@ -77,10 +77,9 @@ __global__ void __launch_bounds__((KernelCfg<APACK, BPACK, BNT, PA, PB, SEP, CG>
 }
 
 template <typename OutT, bool APACK, bool BPACK, int BNT, int CG = 1, int PA = 1, int PB = 1,
-          bool ASYM = false, bool F6 = false>
+          bool ASYM = false, bool F6 = false, int SEP = 0>
 cudaError_t launch_gemm_t(const MapSet& m, const GemmArgs& g, int use_tma_store, int grid,
                           cudaStream_t st) {
-  constexpr bool SEP = PA == 2 && PB == 2;  // W8A8: exact plane accumulators
   using C = KernelCfg<APACK, BPACK, BNT, PA, PB, SEP, CG>;
   auto k = w4a4_gemm_kernel<OutT, APACK, BPACK, BNT, PA, PB, ASYM, F6, SEP, CG>;
   constexpr size_t smem = C::BYTES + 1024;  // + alignment slack
@@ -121,7 +120,8 @@ cudaError_t launch_gemm_bits(const MapSet& m, const GemmArgs& g, int x_codes, in
                              TileShape t, int use_tma_store, int grid, cudaStream_t st) {
   const bool a8 = x_codes == CLQ_CODES_E4M3_SPLIT, w8 = w_codes == CLQ_CODES_E4M3_SPLIT;
   if (g.lo != nullptr) {  // asymmetric activations
-    if (a8 && w8) CLQ_GO(false, false, 128, 2, 2, 2, true);
+    if (a8 && w8 && g.K > kSep2MaxK) CLQ_GO(false, false, 128, 2, 2, 2, true, false, 3);
+    if (a8 && w8) CLQ_GO(false, false, 128, 2, 2, 2, true, false, 2);
     if (a8) CLQ_GO(false, false, 256, 2, 2, 1, true);
     switch (t.bn) {
       case 64: CLQ_GO(false, false, 64, 2, 1, 1, true);
@@ -129,7 +129,9 @@ cudaError_t launch_gemm_bits(const MapSet& m, const GemmArgs& g, int x_codes, in
       default: CLQ_GO(false, false, 256, 2, 1, 1, true);
     }
   }
-  if (w8) CLQ_GO(false, false, 128, 2, 2, 2);
+  if (w8 && g.K > kSep2MaxK) CLQ_GO(false, false, 128, 2, 2, 2, false, false, 3);
+  if (w8 && t.bn == 64) CLQ_GO(false, false, 64, 2, 2, 2, false, false, 2);
+  if (w8) CLQ_GO(false, false, 128, 2, 2, 2, false, false, 2);
   switch (t.bn) {
     case 64: CLQ_GO(false, false, 64, 2, 2, 1);
     case 128: CLQ_GO(false, false, 128, 2, 2, 1);

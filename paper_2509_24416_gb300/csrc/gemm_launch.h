@@ -6,6 +6,10 @@
 
 namespace clq {
 
+// Largest K for which W8A8's cross and low products share one exact fp32
+// accumulator: at most 2112 a code pair (gemm_pipeline.cuh), 2112 K < 2^24.
+constexpr int kSep2MaxK = 7936;
+
 // Tensor maps of a launch: operands, output, second planes of 8-bit operands.
 struct MapSet {
   CUtensorMap A, B, Y, A2, B2;

@@ -70,11 +70,10 @@ constexpr int MAX_STAGES = 8;
 // values, so the MMAs of the two planes add up to q in one accumulator).
 // EW: epilogue warps (0: 4 with unpack warps, else 8); SMAX: stage cap, for
 // a CTA that keeps shared memory for other work.
-// SEP (8-bit x 8-bit codes, PA = PB = 2): the plane products go to three
-// accumulators (16 h x 16 h, the two cross terms, l x l) of one buffer, so
-// that each stays exact in fp32 (see pipeline()); 3 BNT TMEM columns.
+// SEP (8-bit x 8-bit codes, PA = PB = 2): the plane products go to SEP = 2 or 3
+// accumulators of BNT columns, so that each stays exact in fp32 (see pipeline()).
 template <bool APACK, bool BPACK, int BNT = BN, int PA = 1, int PB = 1, int EW = 0,
-          int SMAX = MAX_STAGES, bool SEP = false, int CG = 1>
+          int SMAX = MAX_STAGES, int SEP = 0, int CG = 1>
 struct Cfg {
   static constexpr bool UNPACK = APACK || BPACK;
   static constexpr int EPI_WARPS = EW != 0 ? EW : (UNPACK ? 4 : 8);
@@ -98,10 +97,11 @@ struct Cfg {
   static constexpr size_t BYTES = OFF_COL + EPI_WARPS * COL_FLOATS * sizeof(float);
   // bytes that complete on a stage's barrier (both CTAs' copies of a pair)
   static constexpr uint32_t TX = CG * ((APACK ? A_P : AU) + (BPACK ? BP : BU));
-  // two accumulators of BNT columns, 2 * BNT rounded up to the power of two
+  // accumulator buffers (tiles in flight) of ACC columns; the power of two that
   // tcgen05.alloc takes
-  static constexpr uint32_t TMEM = SEP ? 512u : (2 * BNT <= 256 ? 256u : 512u);
-  static constexpr int NBUF = SEP ? 1 : 2;  // accumulator buffers (tiles in flight)
+  static constexpr int ACC = (SEP > 0 ? SEP : 1) * BNT;
+  static constexpr int NBUF = 2 * ACC <= 512 ? 2 : 1;
+  static constexpr uint32_t TMEM = NBUF * ACC <= 128 ? 128u : NBUF * ACC <= 256 ? 256u : 512u;
   static_assert(S >= 2, "pipeline needs two stages");
   static_assert((PA == 1 || PA == 2) && (PB == 1 || PB == 2), "one or two planes");
   static_assert(!UNPACK || (PA == 1 && PB == 1), "8-bit planes come as E4M3 only");
@@ -109,7 +109,9 @@ struct Cfg {
   static_assert(EPI_NCOL % EPI_COLS == 0 && STAGE % 1024 == 0, "whole blocks, aligned staging");
   static_assert(SMAX <= MAX_STAGES, "barrier arrays hold MAX_STAGES stages");
   static_assert(CG == 1 || (CG == 2 && !UNPACK && EW == 0), "pairs: E4M3 / E2M3 operands only");
-  static_assert(!SEP || (PA == 2 && PB == 2 && 3 * BNT <= 512), "SEP: 8-bit x 8-bit, 3 BNT <= 512");
+  static_assert((SEP != 0) == (PA == 2 && PB == 2) && (SEP == 0 || SEP == 2 || SEP == 3),
+                "SEP: two or three accumulators, 8-bit x 8-bit codes");
+  static_assert(ACC <= 512, "one buffer fits tensor memory");
 };
 
 struct __align__(8) Barriers {
@@ -144,7 +146,7 @@ __device__ __forceinline__ void fence_proxy_async_global() {
 // Barrier init (thread 0) and TMEM allocation (warp WARP_MMA); the caller
 // follows with tcgen05 fences around a CTA barrier.
 template <bool APACK, bool BPACK, int BNT = BN, int PA = 1, int PB = 1, int EW = 0,
-          int SMAX = MAX_STAGES, bool SEP = false, int CG = 1>
+          int SMAX = MAX_STAGES, int SEP = 0, int CG = 1>
 __device__ __forceinline__ void setup(Barriers* bars) {
   using C = Cfg<APACK, BPACK, BNT, PA, PB, EW, SMAX, SEP, CG>;
   constexpr int S = C::S;
@@ -197,12 +199,17 @@ __device__ __forceinline__ bool wait_rows_ready(const uint32_t* ready, int m, ui
 // SEP (W8A8): plane 0 holds 16 h and plane 1 l of each 8-bit code (q = 16 h
 // + l), so q_x q_w = (16 h_x)(16 h_w) + [(16 h_x) l_w + l_x (16 h_w)] + l_x l_w.
 // One fp32 accumulator would round once partial sums pass 2^24 (K > 896 at
-// +-127).  Kept apart, each stays exact to K = 16384: the first sums
-// multiples of 256 below 2^28 (exact up to 2^32), the second multiples of 16
-// below 2^25 (exact up to 2^28), the third integers below 2^20.  The
-// epilogue adds them as int32 (|q_x q_w| K <= 2^28).
+// +-127).  The first term sums multiples of 256 below 2^28 (exact up to 2^32) for
+// every K <= 16384 and gets its own accumulator.  The rest: |16 h| <= 128 and |l|
+// <= 8 make a code pair's three products at most 2 * 1024 + 64 = 2112, so all of
+// them together stay below 2^24, exact in any order, up to K = 7943; SEP = 2 puts
+// them in one accumulator, and two tiles fit tensor memory, so the epilogue
+// overlaps the next tile's MMAs.  SEP = 3, for larger K, keeps the cross terms
+// (multiples of 16 below 2^25, exact up to 2^28) and l l (below 2^20) apart and
+// one tile at a time.  The epilogue adds the accumulators as int32 (|q_x q_w| K
+// <= 2^28).
 template <typename OutT, bool APACK, bool BPACK, int BNT = BN, int PA = 1, int PB = 1, bool ASYM = false, int EW = 0, int SMAX = MAX_STAGES,
-          bool F6 = false, bool SEP = false, int CG = 1>
+          bool F6 = false, int SEP = 0, int CG = 1>
 __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, uint8_t* smem,
                                          Barriers* bars, uint32_t tmem, const uint32_t* ready) {
   using C = Cfg<APACK, BPACK, BNT, PA, PB, EW, SMAX, SEP, CG>;
@@ -303,15 +310,15 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
       uint32_t phase = 0;  // of the stage's ready barrier
       bool ok = true;
       for (int t = unit; t < tiles && ok; t += units, ++tc) {
-        const int buf = SEP ? 0 : (tc & 1);
-        const uint32_t use = SEP ? tc : (tc >> 1);  // this buffer's earlier tiles
+        const int buf = C::NBUF == 1 ? 0 : (tc & 1);
+        const uint32_t use = C::NBUF == 1 ? tc : (tc >> 1);  // this buffer's earlier tiles
         if (!mbar_wait_bounded(&bars->acc_empty[buf], (use & 1) ^ 1, abort, g.status,
                                kWaitLimitNs)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t d = tmem + buf * BNT;
+        const uint32_t d = tmem + buf * C::ACC;
         for (int kb = 0; kb < nk; ++kb) {
           uint64_t* ready_bar = C::UNPACK ? &bars->unpacked[s] : &bars->tma_full[s];
           if (!mbar_wait_bounded(ready_bar, phase, abort, g.status, kWaitLimitNs)) {
@@ -327,11 +334,12 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
             for (int pb = 0; pb < PB; ++pb)
 #pragma unroll
               for (int k = 0; k < BK / 32; ++k) {
-                // SEP: accumulator 0 (16h x 16h), 1 (cross terms), 2 (l x l); the
-                // cross terms' second product always accumulates
-                const int acc_i = SEP ? (pa + pb) : 0;
-                const bool first = SEP ? ((kb | k) == 0 && !(pa == 1 && pb == 0))
-                                       : (kb | pa | pb | k) == 0;
+                // SEP: accumulator 0 takes 16h x 16h; 3: 1 the cross terms, 2 l x l;
+                // 2: 1 all of them.  A tile's first product into each replaces it.
+                const int acc_i = SEP == 3 ? pa + pb : SEP == 2 ? (pa | pb) : 0;
+                const bool first =
+                    (kb | k) == 0 && (SEP == 0 ? (pa | pb) == 0
+                                               : pa == 0 || (SEP == 3 && pb == 1));
                 mma_e4m3<CG>(d + acc_i * BNT, a0 + (pa * A_U + k * 32) / 16,
                              b0 + (pb * (BNT / CG) * BK + k * 32) / 16, idesc, first ? 0u : 1u);
               }
@@ -362,8 +370,8 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
       const int mb = t / tiles_n;
       const int m0 = mb * TM + rank * BM;
       const int n0 = (t - mb * tiles_n) * BNT;
-      const int buf = SEP ? 0 : (tc & 1);
-      const uint32_t use = SEP ? tc : (tc >> 1);
+      const int buf = C::NBUF == 1 ? 0 : (tc & 1);
+      const uint32_t use = C::NBUF == 1 ? tc : (tc >> 1);
       // This warp's column data and row scales, while the tile's MMAs run.
 #pragma unroll
       for (int j = lane; j < NCOL; j += 32) {
@@ -404,8 +412,8 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
           if (row < g.M) sx[k] = __ldcg(g.s_x + row);
         }
       }
-      epilogue_part<OutT, NCOL, ASYM, SEP ? BNT : 0>(
-          tmem + buf * BNT, quarter, part * NCOL, lane, m0, n0, g.M, g.N, sx, col, zm, staging,
+      epilogue_part<OutT, NCOL, ASYM, SEP, BNT>(
+          tmem + buf * C::ACC, quarter, part * NCOL, lane, m0, n0, g.M, g.N, sx, col, zm, staging,
           maps.Y, g.Y, g.acc_dbg, [&]() {
             tc_fence_before();
             __syncwarp();

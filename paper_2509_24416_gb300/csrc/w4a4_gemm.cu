@@ -373,8 +373,13 @@ cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, i
   // the same epilogue: 8192 x 3456 x 1152 26.8 -> 23.5 us, 4608 x 3072 x 12288
   // 110.5 -> 84.6, 65536 x 12288 x 3072 1523 -> 1235; 20 x 480 x 1920 6.9 -> 6.4).
   TileShape t{apack || bpack ? 1 : 2, BN};
-  if (w8a8)
-    t.bn = 128;  // three accumulators of 128 columns fill one TMEM allocation
+  if (w8a8) {
+    // 128 columns (two or three accumulators of them fill tensor memory), 64 where
+    // that leaves pairs idle and the product's accumulators allow it
+    t.bn = 128;
+    const int pairs = ((g.M + t.cg * BM - 1) / (t.cg * BM)) * ((g.N + 127) / 128);
+    if (g.lo == nullptr && g.K <= kSep2MaxK && 2 * pairs <= sms / t.cg) t.bn = 64;
+  }
   else if (!apack && !bpack && !(split && g.lo != nullptr))
     t.bn = gemm_tile_n(g.M, g.N, g.K, t.cg * BM, sms / t.cg, !split && g.lo == nullptr, true);
   MapSet m;

@@ -118,3 +118,32 @@ def test_tile_widths(setting, M, N, K):
     # half an ulp of fp16, three fp32 roundings of the terms, the smallest subnormal
     err = (Y.double() - y64).abs()
     assert bool((err <= 2.0 ** -11 * y64.abs() + 1e-6 * size + 2.0 ** -24).all())
+
+
+@pytest.mark.parametrize("K", [1024, 7936, 7968, 16384])
+@pytest.mark.parametrize("M,N", [(130, 40), (3000, 3000)])
+def test_w8a8_accumulators_at_their_limit(K, M, N):
+    """K at and past the point where W8A8's cross and low products stop sharing an
+    accumulator, with the code whose products there are largest (120 = 128 - 8:
+    2 * 128 * -8 + 64 a pair) in every place but a few: |acc| up to 14400 K."""
+    def split(q):
+        h = torch.div(q + 8, 16, rounding_mode="floor")
+        lut = torch.zeros(257, dtype=torch.uint8, device=DEV)
+        for v in range(-128, 129):
+            a = abs(v)
+            f, x = np.frexp(float(a)) if a else (0.0, 0)
+            m = (f * 2 - 1) * 8
+            if a and m == int(m):
+                lut[v + 128] = ((x - 1 + 7) << 3) | int(m) | (0x80 if v < 0 else 0)
+        return torch.cat([lut[(16 * h + 128).long()], lut[(q - 16 * h + 128).long()]], dim=1)
+
+    g = torch.Generator(device=DEV).manual_seed(K)
+    qx = torch.full((M, K), 120, dtype=torch.int32, device=DEV)
+    qw = torch.full((N, K), 120, dtype=torch.int32, device=DEV)
+    qx[:, :5] = torch.randint(-127, 128, (M, 5), generator=g, device=DEV, dtype=torch.int32)
+    qw[1::2] = -qw[1::2]
+    ones = torch.ones(M, device=DEV), torch.ones(N, device=DEV)
+    Y, acc = clq.linear(split(qx), ones[0], split(qw), ones[1], 32, K, None, with_acc=True)
+    want = qx.double() @ qw.double().t()
+    assert torch.equal(acc.double(), want)
+    assert clq.device_status() == 0
