@@ -161,26 +161,30 @@ cudaError_t launch_rotate_quant(const RotateQuantArgs& a, int dtype, int logb,
   size_t smem = 0;
   const int sms = sm_count();
   if (sms <= 0) return cudaErrorInvalidDevice;
-  // 4-bit activation codes in the E4M3 or E2M3 layout (asymmetric: E4M3): the wide
-  // kernel for b >= 64, the paired-row kernel for symmetric codes at b = 32.  The
+  // Unclipped codes in an execution layout: the wide kernel for b >= 64, the
+  // paired-row kernel for symmetric 4-bit codes at b = 32.  The
   // wide kernel against the paired one (asymmetric: the general one), us at b =
   // 128 / 256: 16384 rows x 1152 / 1280 16.3 / 18.4 against 18.8 / 25.8, 4608 x
   // 12288 42 / 42 against 53 / 62 (E2M3 42 / 49 against 57 / 64; asymmetric 46 / 46
-  // against 67 / 72); at 256 rows, a launch of about 2.7 us, it is up to 0.2 us
-  // slower.
-  const bool hot = a.lo == nullptr && a.clip == nullptr && (a.e4m3 == 1 || a.e4m3 == 3);
-  const bool hot_asym = a.lo != nullptr && a.clip == nullptr && a.e4m3 == 1;
-  if ((hot || hot_asym) && logb >= 6) {  // b divides K, so K % 64 == 0
+  // against 67 / 72; 8-bit codes at b = 64 / 128 against the general one:
+  // 8192 x 1152 10.4 / 11.7 against 14.4 / 15.3, 4608 x 12288 49 / 55 against 79 / 83);
+  // at 256 rows, a launch of about 2.7 us, it is up to 0.2 us slower.
+  const bool hot = a.clip == nullptr && a.e4m3 != 0;  // not packed, not clipped
+  if (hot && logb >= 6) {  // b divides K, so K % 64 == 0
     int stage = 0;
     rotate_quant_wide_config(a.M, a.K, sms, &args.rows_per_tile, &threads, &smem, &stage);
     const bool e2 = a.e4m3 == 3;
+    if (a.e4m3 == 2)
+      return dtype == CLQ_F16
+                 ? launch_rotate_quant_wide_f16_split(args, logb, stage, threads, smem, sms, st)
+                 : launch_rotate_quant_wide_bf16_split(args, logb, stage, threads, smem, sms, st);
     if (dtype == CLQ_F16)
       return e2 ? launch_rotate_quant_wide_f16_e2m3(args, logb, stage, threads, smem, sms, st)
                 : launch_rotate_quant_wide_f16_e4m3(args, logb, stage, threads, smem, sms, st);
     return e2 ? launch_rotate_quant_wide_bf16_e2m3(args, logb, stage, threads, smem, sms, st)
               : launch_rotate_quant_wide_bf16_e4m3(args, logb, stage, threads, smem, sms, st);
   }
-  if (hot && logb == 5) {
+  if (hot && a.lo == nullptr && a.e4m3 != 2 && logb == 5) {
     int half = 0;
     rotate_quant_pair_config(a.M, a.K, sms, &args.rows_per_tile, &threads, &smem, &half);
     const bool e2 = a.e4m3 == 3;

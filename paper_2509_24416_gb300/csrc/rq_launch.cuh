@@ -17,7 +17,13 @@ cudaError_t launch_rotate_quant_f16(const RotateQuantArgs& a, int logb, int thre
                                     int sms, cudaStream_t st);
 cudaError_t launch_rotate_quant_bf16(const RotateQuantArgs& a, int logb, int threads,
                                      size_t smem, int sms, cudaStream_t st);
-// Wide-segment kernel per input type and code layout (rotate_quant_pair_*.cu).
+// Wide-segment kernel per input type and code layout (rotate_quant_pair_*.cu,
+// rotate_quant_split_*.cu).
+cudaError_t launch_rotate_quant_wide_f16_split(const RotateQuantArgs& a, int logb, int stage,
+                                               int threads, size_t smem, int sms, cudaStream_t st);
+cudaError_t launch_rotate_quant_wide_bf16_split(const RotateQuantArgs& a, int logb, int stage,
+                                                int threads, size_t smem, int sms,
+                                                cudaStream_t st);
 cudaError_t launch_rotate_quant_wide_f16_e4m3(const RotateQuantArgs& a, int logb, int stage,
                                               int threads, size_t smem, int sms, cudaStream_t st);
 cudaError_t launch_rotate_quant_wide_f16_e2m3(const RotateQuantArgs& a, int logb, int stage,
@@ -111,7 +117,7 @@ cudaError_t launch_wide_geom(const RotateQuantArgs& a, int threads, size_t smem,
 template <typename T, int CODES, int STAGE, bool ROT>
 cudaError_t launch_wide_b(const RotateQuantArgs& a, int logb, int threads, size_t smem, int sms,
                           cudaStream_t st) {
-  if constexpr (CODES == 1)
+  if constexpr (CODES != 3)
     if (a.lo != nullptr) switch (logb) {
         case 6: return launch_wide_geom<T, 6, CODES, STAGE, ROT, true>(a, threads, smem, sms, st);
         case 7: return launch_wide_geom<T, 7, CODES, STAGE, ROT, true>(a, threads, smem, sms, st);
@@ -124,7 +130,7 @@ cudaError_t launch_wide_b(const RotateQuantArgs& a, int logb, int threads, size_
   }
 }
 
-// The wide kernel for CODES (1 E4M3, 3 E2M3), 64 <= b <= 256; `stage`
+// The wide kernel for CODES (1 E4M3, 2 split, 3 E2M3), 64 <= b <= 256; `stage`
 // is the stage size rotate_quant_wide_config chose.
 template <typename T, int CODES>
 cudaError_t launch_rotate_quant_wide_t(const RotateQuantArgs& a, int logb, int stage, int threads,

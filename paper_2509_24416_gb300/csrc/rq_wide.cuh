@@ -1,5 +1,5 @@
 // Wide-segment rotate-quantize: the hot-path variant of the tile loop for
-// 4-bit activation codes when b >= 64 (the OBS transform of arxiv 2509.24416
+// 4-bit (E4M3, E2M3) and 8-bit (split-plane) codes when b >= 64 (the OBS transform of arxiv 2509.24416
 // Sec. 3.3 and the per-token quantization of Sec. 3.1 / Eq. 1, symmetric, or
 // asymmetric with the row's minimum and maximum, as in rq_device.cuh).
 //
@@ -161,6 +161,72 @@ __device__ __forceinline__ uint32_t wide_flip(int xm, int lane) {
   return flip;
 }
 
+// 1.5 * 2^23 + 8: a code q added to it by an fma comes out rounded (ties to even:
+// the constant is even) as q + 8 in the low mantissa bits.
+constexpr float kSplitMagic = 12582920.0f;
+
+// Split-plane stores of a thread's 64 codes, v holding q + kSplitMagic (SCALE:
+// values that +-rcp, by the bits of flip, turns into it): 16 h = floor((q + 8) /
+// 16) * 16 by one addition that rounds down at 16, the ulp of 1.5 * 2^27, then l =
+// q - 16 h, both exact; E4M3 bytes, 16 codes a store and plane.
+template <int X, bool SCALE>
+__device__ __forceinline__ void wide_store_split(const RotateQuantArgs& a, float2 (&v)[32],
+                                                 int row, int block, int lane, float rcp,
+                                                 uint32_t flip) {
+  const int K = a.K;
+  constexpr float big = 201326592.0f;  // 1.5 * 2^27
+  constexpr float up = big - 12582912.0f;
+  uint8_t* qrow = a.Q + static_cast<size_t>(row) * 2 * K + block;
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    uint32_t wh[4], wl[4];
+    // one chunk after the other: interleaved, their temporaries spill
+    asm volatile("" : "+r"(flip)::"memory");
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      uint16_t eh[2], el[2];
+      const float rs = ((flip >> (4 * c + j)) & 1u) ? -rcp : rcp;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        float2 x = v[8 * c + 2 * j + i];
+        if (SCALE)
+          x = __ffma2_rn(x, make_float2(rs, rs), make_float2(kSplitMagic, kSplitMagic));
+        const float2 h16 = __fadd2_rn(__fadd2_rd(x, make_float2(up, up)), make_float2(-big, -big));
+        const float2 q = __fadd2_rn(x, make_float2(-kSplitMagic, -kSplitMagic));
+        const float2 l = __ffma2_rn(h16, make_float2(-1.f, -1.f), q);
+        asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(eh[i]) : "f"(h16.y), "f"(h16.x));
+        asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(el[i]) : "f"(l.y), "f"(l.x));
+      }
+      wh[j] = static_cast<uint32_t>(eh[0]) | (static_cast<uint32_t>(eh[1]) << 16);
+      wl[j] = static_cast<uint32_t>(el[0]) | (static_cast<uint32_t>(el[1]) << 16);
+    }
+    uint8_t* q = qrow + wide_chunk<X>(c, lane);
+    *reinterpret_cast<uint4*>(q) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
+    *reinterpret_cast<uint4*>(q + K) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+  }
+}
+
+// The same for a row with a subnormal scale: values times 2^64 (exact) against
+// `rcp`, the reciprocal of the scale times 2^64.  A call of its own, on a copy of
+// the values: as a branch of the hot path it cost that path 80 bytes of spills.
+template <int X>
+static __device__ __noinline__ void wide_store_split_tiny(uint8_t* qrow, int K, const float2* t,
+                                                          float rcp, uint32_t flip, int lane) {
+#pragma unroll 1
+  for (int r = 0; r < 64; ++r) {
+    const float v = ((r & 1) ? t[r >> 1].y : t[r >> 1].x) * kTwo64;
+    const float x = fmaf(v, ((flip >> (r >> 2)) & 1u) ? -rcp : rcp, kSplitMagic);
+    const float q = x - kSplitMagic;
+    const float h16 = 16.f * floorf((q + 8.f) * 0.0625f);
+    uint16_t eh, el;
+    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(eh) : "f"(0.f), "f"(h16));
+    asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(el) : "f"(0.f), "f"(q - h16));
+    uint8_t* at = qrow + wide_chunk<X>(r >> 4, lane) + (r & 15);
+    at[0] = static_cast<uint8_t>(eh);
+    at[K] = static_cast<uint8_t>(el);
+  }
+}
+
 // Scale, codes and stores of one row's 64 values of a thread; `am` is the row's
 // |x| maximum; bit q of `flip` flips the signs of registers 4q .. 4q + 3.
 template <int CODES, bool ROT, int X>
@@ -169,11 +235,12 @@ __device__ __forceinline__ void wide_quant_store(const RotateQuantArgs& a, float
                                                  int lane) {
   const int K = a.K;
   const int block = (seg >> X) << (6 + X);  // first position of the thread's block
-  // s = am / 7 by division by a constant known in advance (Brisebarre,
+  // s = am / qmax by division by a constant known in advance (Brisebarre,
   // Muller and Raina, IEEE Trans. Computers 53(8), 2004), as in rq_device.cuh
-  constexpr float rdiv = 1.0f / 7.0f;
+  constexpr float qmax = CODES == 2 ? 127.0f : 7.0f;
+  constexpr float rdiv = 1.0f / qmax;
   const float q1 = am * rdiv;
-  const float s_row = fmaf(fmaf(-7.0f, q1, am), rdiv, q1);
+  const float s_row = fmaf(fmaf(-qmax, q1, am), rdiv, q1);
   if (seg == 0) a.S[row] = s_row;
   if (ROT) {
     float* dst = a.rot + static_cast<size_t>(row) * K + block;
@@ -186,6 +253,21 @@ __device__ __forceinline__ void wide_quant_store(const RotateQuantArgs& a, float
   }
   // v <- rint(v / s) + 1.5 * 2^23 (ties to even), v / s as v * rcp(s); a zero
   // row gets zero codes; a subnormal s is scaled with v by 2^64 first.
+  if constexpr (CODES == 2) {
+    if (s_row > 0.f && s_row < 1.17549435e-38f) {
+      float2 t[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k) t[k] = v[k];
+      wide_store_split_tiny<X>(a.Q + static_cast<size_t>(row) * 2 * K + block, K, t,
+                               rcp_approx(s_row * kTwo64), flip, lane);
+      return;
+    }
+    const float rcp = s_row > 0.f ? rcp_approx(s_row) : 0.f;
+    // 8-bit codes: the planes 16 h and l of -q are not those of q negated, so the
+    // signs go into the reciprocal (v * -rcp rounds as -v * rcp)
+    wide_store_split<X, true>(a, v, row, block, lane, rcp, flip);
+    return;
+  }
   const float2 magic = make_float2(12582912.0f, 12582912.0f);
   float s_div = s_row;
   if (s_row > 0.f && s_row < 1.17549435e-38f) {
@@ -262,17 +344,17 @@ __device__ __forceinline__ void wide_quant_store(const RotateQuantArgs& a, float
 
 // Asymmetric codes of one row's 64-wide segment (Eq. 1 with the row's
 // minimum and maximum as bounds, as in rq_device.cuh): delta = (max - min) /
-// 15 by the same division by a constant, q = rint((v - min) / delta) stored
-// centered as q - 8 in E4M3 bytes; kmax / kmin are the row's order keys of
+// (2^n - 1) by the same division by a constant, q = rint((v - min) / delta) stored
+// centered as q - 2^(n-1), 4 bits in E4M3 bytes (CODES 1) or 8 in split planes (2); kmax / kmin are the row's order keys of
 // max and -min.  v holds the true transform (signs already restored).
-template <bool ROT, int X>
+template <int CODES, bool ROT, int X>
 __device__ __forceinline__ void wide_quant_store_asym(const RotateQuantArgs& a, float2 (&v)[32],
                                                       int row, int seg, uint32_t kmax,
                                                       uint32_t kmin, int lane) {
   const int K = a.K;
   const int block = (seg >> X) << (6 + X);
-  constexpr float div = 15.0f;
-  constexpr float rdiv = 1.0f / 15.0f;
+  constexpr float div = CODES == 2 ? 255.0f : 15.0f;
+  constexpr float rdiv = 1.0f / div;
   const float row_lo = -order_key_inv(kmin);
   const float am = __fsub_rn(order_key_inv(kmax), row_lo);
   const float q1 = am * rdiv;
@@ -288,10 +370,11 @@ __device__ __forceinline__ void wide_quant_store_asym(const RotateQuantArgs& a, 
       *reinterpret_cast<float4*>(dst + wide_chunk<X>(q >> 2, lane) + 4 * (q & 3)) =
           make_float4(v[2 * q].x, v[2 * q].y, v[2 * q + 1].x, v[2 * q + 1].y);
   }
-  // v <- rint((v - min) * 15 / span) + 1.5 * 2^23 - 8 (the centered code in
-  // the low mantissa bits); a constant row gets q = 0; a subnormal span takes
-  // exact divisions.
-  const float2 mg = make_float2(12582912.0f - 8.0f, 12582912.0f - 8.0f);
+  // v <- rint((v - min) * (2^n - 1) / span) + 1.5 * 2^23 - 2^(n-1) (the centered
+  // code in the low mantissa bits; 8 more for split planes); a constant row gets q
+  // = 0; a subnormal span takes exact divisions.
+  constexpr float mgc = CODES == 2 ? kSplitMagic - 128.0f : 12582912.0f - 8.0f;
+  const float2 mg = make_float2(mgc, mgc);
   const float2 nlo = make_float2(-row_lo, -row_lo);
   // exact divisions also where rcp(span) would be subnormal (span >= 2^126,
   // bf16 inputs near their top), which rcp.approx.ftz flushes to zero
@@ -308,6 +391,10 @@ __device__ __forceinline__ void wide_quant_store_asym(const RotateQuantArgs& a, 
     const float2 inv2 = make_float2(inv, inv);
 #pragma unroll
     for (int k = 0; k < 32; ++k) v[k] = __ffma2_rn(__fadd2_rn(v[k], nlo), inv2, mg);
+  }
+  if constexpr (CODES == 2) {
+    wide_store_split<X, false>(a, v, row, block, lane, 0.f, 0u);
+    return;
   }
   const float2 nmagic = make_float2(-12582912.0f, -12582912.0f);
   uint8_t* qrow = a.Q + static_cast<size_t>(row) * K + block;
@@ -327,8 +414,8 @@ __device__ __forceinline__ void wide_quant_store_asym(const RotateQuantArgs& a, 
   }
 }
 
-// CODES 1 (E4M3) or 3 (E2M3); 64 <= b <= 256 (LOGB 6 .. 8); K % 64 == 0.
-// ASYM: asymmetric codes (a.lo != null), E4M3 only.
+// CODES 1 (E4M3), 2 (8-bit split planes) or 3 (E2M3); 64 <= b <= 256 (LOGB 6 ..
+// 8); K % 64 == 0.  ASYM: asymmetric codes (a.lo != null), not E2M3.
 // a.rows_per_tile = RH rows a tile (RH * 2K <= STAGE, RH * K / 64 <=
 // blockDim.x).
 template <typename T, int LOGB, int CODES, int STAGE, int STAGES, bool ROT, bool ASYM = false>
@@ -336,7 +423,7 @@ __global__ void __maxnreg__(kWideMaxRegs) rotate_quant_wide_kernel(RotateQuantAr
   extern __shared__ __align__(16) uint8_t smem[];
   static_assert(LOGB >= 6 && LOGB <= 8, "wide loop: 64 <= b <= 256");
   static_assert(STAGE <= 65536, "gather offsets are 16-bit");
-  static_assert(!ASYM || CODES == 1, "asymmetric codes in E4M3 bytes only");
+  static_assert(!ASYM || CODES != 3, "no asymmetric E2M3 codes");
   const int K = a.K;
   const int segs = K >> 6;
   const int RH = a.rows_per_tile;
@@ -491,8 +578,8 @@ __global__ void __maxnreg__(kWideMaxRegs) rotate_quant_wide_kernel(RotateQuantAr
       // ---- 3. scale, codes, stores --------------------------------------------
       if (active && r < n) {
         if constexpr (ASYM)
-          wide_quant_store_asym<ROT, X>(a, v, row0 + r, seg, amax[par * RH + r],
-                                        amin[par * RH + r], lane);
+          wide_quant_store_asym<CODES, ROT, X>(a, v, row0 + r, seg, amax[par * RH + r],
+                                               amin[par * RH + r], lane);
         else
           wide_quant_store<CODES, ROT, X>(a, v, row0 + r, seg,
                                           __uint_as_float(amax[par * RH + r]), flip, lane);

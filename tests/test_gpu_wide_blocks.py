@@ -1,8 +1,9 @@
 """The wide rotate-quantize loop (b = 64, 128, 256; symmetric E4M3 and E2M3 codes,
-asymmetric E4M3 codes) against the general loop on the same rows, which writes
-packed nibbles: both form every output by the same sums in the same order, so
-codes, scales, bounds and rotated rows agree bit for bit (a zero code may be
-written as either zero)."""
+asymmetric E4M3 codes, 8-bit split planes) against the general loop on the same
+rows, which writes packed nibbles (and, given clip bounds that never bind, 8-bit
+codes): both form every output by the same sums in the same order, so codes,
+scales, bounds and rotated rows agree bit for bit (a zero code may be written as
+either zero)."""
 import numpy as np
 import pytest
 import torch
@@ -26,6 +27,22 @@ def _nibbles(p):
     lo, hi = (p & 15).to(torch.int16), (p >> 4).to(torch.int16)
     q = torch.stack([lo, hi], dim=2).reshape(p.shape[0], -1)
     return torch.where(q >= 8, q - 16, q)
+
+
+def _planes(q, K):
+    """Integer codes of split planes: bytes of 16 h and of l."""
+    lut = torch.full((256,), 9999, dtype=torch.int32)
+    for v in range(-128, 129):
+        a = abs(v)
+        f, x = np.frexp(float(a)) if a else (0.0, 0)
+        m = (f * 2 - 1) * 8
+        if a and m == int(m):
+            lut[((x - 1 + 7) << 3) | int(m) | (0x80 if v < 0 else 0)] = v
+    lut[0x00] = lut[0x80] = 0
+    v = lut.to(DEV)[q.long()]
+    hi, lo = v[:, :K], v[:, K:]
+    assert bool((hi % 16 == 0).all()) and int(lo.min()) >= -8 and int(lo.max()) <= 7
+    return hi + lo
 
 
 def _rows(M, K, dtype, seed):
@@ -66,6 +83,31 @@ def test_wide_equals_general(b, K, M, dtype):
                 q, s = clq.rotate_quant_act(x, p, b, clq.CLQ_CODES_E2M3)
                 packed = clq.convert_codes(q, K, clq.CLQ_CODES_INT4_PACKED)
                 assert torch.equal(_nibbles(packed), want) and torch.equal(s, s_want)
+    # 8-bit symmetric codes: weight preparation with a clip takes the general loop
+    S8 = clq.CLQ_CODES_E4M3_SPLIT
+    clip = torch.full((M,), 3e38, device=DEV)
+    q8_want, s8_want, rot8 = clq.prepare_weights(X, perm, b, clip=clip, codes=S8, with_rot=True)
+    assert torch.equal(rot8, rot_want)
+    v8_want = _planes(q8_want, K)
+    for p in (perm, shifted):
+        q8, s8 = clq.rotate_quant_act(wide[:, :K], p, b, S8)
+        # rows with a subnormal scale take exact divisions in the general loop and a
+        # scaled reciprocal in this one
+        rows = s8_want >= 1.2e-38
+        assert torch.equal(s8, s8_want)
+        assert torch.equal(_planes(q8, K)[rows], v8_want[rows])
+        assert int((_planes(q8, K)[~rows] - v8_want[~rows]).abs().max() if (~rows).any() else 0) <= 1
+    qa, da, la = clq.rotate_quant_act_asym(X, perm, b, codes=S8)
+    x64 = rot_want.double()
+    lo, span = x64.amin(1, keepdim=True), x64.amax(1, keepdim=True) - x64.amin(1, keepdim=True)
+    ratio = torch.where(span > 0, (x64 - lo) / span.clamp(min=1e-300) * 255, torch.zeros_like(x64))
+    codes = _planes(qa, K).double() + 128
+    assert torch.equal(la, l_want)
+    # delta: 2 ulp (2.5e-7), or one step 2^-149 of the subnormal grid, times 255
+    assert bool(((da.double() * 255 - span[:, 0]).abs()
+                 <= 2.5e-7 * span[:, 0] + 255 * 2.0 ** -149).all())
+    # 8-bit ratios reach 255: fp32 keeps them within 1e-4 (tests/parity_utils.py)
+    assert bool(((codes - ratio).abs() <= 0.5 + 1e-4).all())
     q, s, rot = clq.rotate_quant_act(X, perm, b, clq.CLQ_CODES_E4M3, with_rot=True)
     assert torch.equal(rot, rot_want) and torch.equal(lut[q.long()], want)
     assert clq.device_status() == 0
