@@ -133,9 +133,33 @@ __device__ __forceinline__ void encode_group(uint8_t* __restrict__ row, int code
   }
 }
 
+// Four E4M3 bytes of integer codes -> the codes' two's-complement nibbles, one a
+// byte: magnitudes 0x00 0x38 0x40 0x44 0x48 0x4A 0x4C 0x4E are 0 .. 7.
+__device__ __forceinline__ uint32_t e4m3_to_nibbles(uint32_t w) {
+  constexpr uint32_t ones = 0x01010101u;
+  const uint32_t b6 = (w >> 6) & ones, b3 = (w >> 3) & ones;
+  const uint32_t hi = (b6 & b3) * 0xFFu;           // 4 .. 7: two mantissa bits
+  const uint32_t mid = (b6 & (b3 ^ ones)) * 0xFFu;  // 2, 3: one
+  const uint32_t low = (b6 ^ ones) * 0xFFu;         // 0, 1
+  const uint32_t v = (hi & (0x04040404u | ((w >> 1) & 0x03030303u))) |
+                     (mid & (0x02020202u | ((w >> 2) & ones))) | (low & ((w >> 5) & ones));
+  const uint32_t neg = (w >> 7) & ones;
+  return ((v ^ (neg * 0x0Fu)) + neg) & 0x0F0F0F0Fu;
+}
+
+// Four nibbles, one a byte -> two packed bytes.
+__device__ __forceinline__ uint32_t pack_nibbles(uint32_t n) {
+  const uint32_t x = n | (n >> 4);
+  return (x & 0xFFu) | ((x >> 8) & 0xFF00u);
+}
+
 // Code array in one 4-bit layout -> another, one thread a group of 16 codes.
 // A code outside [-7, 7] (packed -8) or a field that holds no integer is
-// written as 0 and reported.
+// written as 0 and reported.  Between E4M3 bytes and packed nibbles whole words
+// are converted, checked by the way back, and only a group that holds something
+// else goes code by code; with one byte a load and store the kernel took 24 us for
+// 9216 x 3072 codes E4M3 -> packed, 46 back (copying them 6); now 15.4 and
+// 7.3.
 __global__ void convert_codes_kernel(const uint8_t* __restrict__ src, int src_codes,
                                      uint8_t* __restrict__ dst, int dst_codes, int rows, int K,
                                      int32_t* status) {
@@ -144,6 +168,36 @@ __global__ void convert_codes_kernel(const uint8_t* __restrict__ src, int src_co
   const size_t sb = codes_row_bytes(src_codes, K), db = codes_row_bytes(dst_codes, K);
   for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<size_t>(gridDim.x) * blockDim.x) {
+    if (src_codes == CLQ_CODES_E4M3 && dst_codes == CLQ_CODES_INT4_PACKED) {
+      const uint4 w = reinterpret_cast<const uint4*>(src)[i];  // rows are whole groups
+      uint2 o;
+      o.x = pack_nibbles(e4m3_to_nibbles(w.x)) | (pack_nibbles(e4m3_to_nibbles(w.y)) << 16);
+      o.y = pack_nibbles(e4m3_to_nibbles(w.z)) | (pack_nibbles(e4m3_to_nibbles(w.w)) << 16);
+      const uint2 a = nibbles_to_e4m3(o.x), b = nibbles_to_e4m3(o.y);
+      // a zero code may carry a sign: compare magnitudes there (0 - 1 borrows, so
+      // only a byte that is 0x00 or 0x80 both ways is let off)
+      auto differs = [](uint32_t x, uint32_t back) {
+        const uint32_t d = x ^ back;
+        const uint32_t zero = ((back & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) & 0x80808080u;  // 0x80: non-zero
+        return (d & ~(~zero & 0x80808080u)) != 0;
+      };
+      if (!(differs(w.x, a.x) || differs(w.y, a.y) || differs(w.z, b.x) || differs(w.w, b.y))) {
+        reinterpret_cast<uint2*>(dst)[i] = o;
+        continue;
+      }
+    } else if (src_codes == CLQ_CODES_INT4_PACKED && dst_codes == CLQ_CODES_E4M3) {
+      const uint2 w = reinterpret_cast<const uint2*>(src)[i];
+      // a nibble of 8 (the code -8): its low three bits are zero and its top bit set
+      auto minus8 = [](uint32_t x) {
+        const uint32_t low = x & 0x77777777u;
+        return (~(low + 0x77777777u) & ~low & x & 0x88888888u) != 0;
+      };
+      if (!(minus8(w.x) || minus8(w.y))) {
+        const uint2 a = nibbles_to_e4m3(w.x), b = nibbles_to_e4m3(w.y);
+        reinterpret_cast<uint4*>(dst)[i] = make_uint4(a.x, a.y, b.x, b.y);
+        continue;
+      }
+    }
     const size_t r = i / groups;
     const int g = static_cast<int>(i - r * groups);
     int c[16];
