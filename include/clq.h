@@ -54,12 +54,13 @@
  *    reads the swap vector `perm`, a layer constant.  So that `perm` must not
  *    be written by the kernel enqueued just before the call on the same
  *    stream: the writes of a kernel are guaranteed visible to the next one
- *    only once the latter has waited for it.  No call of this library writes
- *    a swap vector (clq_build_permutation runs on the host); a copy or
- *    another call of this library enqueued between the writing kernel and
- *    the call restores the usual order.  The weight-preparation calls and
- *    clq_clip_search launch without the overlap, so a swap vector computed
- *    on the device just before them is safe.
+ *    only once the latter has waited for it.  Of the calls of this library only
+ *    clq_build_permutation_device writes a swap vector on the device
+ *    (clq_build_permutation runs on the host); a copy or another call of this
+ *    library enqueued between the writing kernel and the call restores the
+ *    usual order.  The weight-preparation calls and clq_clip_search launch
+ *    without the overlap, so a swap vector computed on the device just before
+ *    them is safe.
  *  - The library keeps no per-call state and is safe to call from several
  *    host threads.
  *  - The hot-path calls (rotate-quant, the products, the fused kernel) launch
@@ -197,6 +198,15 @@ clq_status clq_outlier_scores_metric(const void* calib, clq_dtype dtype, int32_t
  */
 clq_status clq_build_permutation(const float* host_scores, int32_t K,
                                  int32_t* host_perm);
+
+/*
+ * The same vector from scores on the DEVICE (fp32 [K], 1 <= K <= 16384), into perm
+ * (device int32 [K]), without a copy to the host.  *bad (device int32) receives 1
+ * if a score is NaN, and perm is then the identity; else 0.
+ */
+clq_status clq_build_permutation_device(const float* scores, int32_t K,
+                                        int32_t* perm, int32_t* bad,
+                                        void* stream);
 
 /*
  * Offline weight preparation (Sec. 3.3, "Overhead Analysis": W~ = G^T-side

@@ -39,7 +39,7 @@ EXPORTS = ("clq_status_string", "clq_version", "clq_outlier_scores",
            "clq_rotate_quant_act_asym", "clq_weight_code_sums",
            "clq_linear_asym", "clq_clip_search_workspace_size",
            "clq_clip_search", "clq_convert_codes", "clq_peak_operand_stream",
-           "clq_peak_rq_stream")
+           "clq_peak_rq_stream", "clq_build_permutation_device")
 
 _lib = None
 _P = ctypes.c_void_p
@@ -80,6 +80,7 @@ _SIGS = {
     "clq_weight_code_sums": (_I, [_P, _I, _I, _I, _P, _P]),
     "clq_linear_asym": (_I, [_P, _I, _P, _P, _P, _I, _P, _P, _P, _I, _I, _I,
                              _I, _I, _P, _P, _P]),
+    "clq_build_permutation_device": (_I, [_P, _I, _P, _P, _P]),
     "clq_clip_search_workspace_size": (_Z, [_I, _I, _I, _P, _I]),
     "clq_clip_search": (_I, [_P, _I, _I, _I, _I, _P, _I, _P, _I, _I, _P, _P,
                              _P, _I, _P, _P, _P, _P, _Z, _P]),
@@ -136,6 +137,10 @@ def clq_outlier_scores(calib, dtype, B, T, K, scores, stream):
 
 def clq_build_permutation(host_scores, K, host_perm):
     return load().clq_build_permutation(host_scores, K, host_perm)
+
+
+def clq_build_permutation_device(scores, K, perm, bad, stream):
+    return load().clq_build_permutation_device(scores, K, perm, bad, stream)
 
 
 def clq_prepare_weights(W, dtype, N, K, ldw, perm, b, clip, Wq, s_w,
@@ -334,6 +339,18 @@ def build_permutation(scores):
     _check(clq_build_permutation(_ptr(s), K, _ptr(perm)),
            "clq_build_permutation")
     return perm
+
+
+def build_permutation_device(scores, stream=None):
+    """Column-swap vector from scores [K] fp32 on the GPU, without a copy to the
+    host -> (perm int32 [K], bad int32 [1], 1 if a score is NaN), on the GPU."""
+    K = scores.numel()
+    scores = scores.contiguous()
+    perm = torch.empty(K, dtype=torch.int32, device=scores.device)
+    bad = torch.empty(1, dtype=torch.int32, device=scores.device)
+    _check(clq_build_permutation_device(_ptr(scores), K, _ptr(perm), _ptr(bad),
+                                        _stream(stream)), "clq_build_permutation_device")
+    return perm, bad
 
 
 def codes_width(codes, K):
@@ -714,7 +731,12 @@ class PreparedLinear:
         best)."""
         K = W.shape[1]
         scores = outlier_scores(calib, metric=metric, stream=stream)
-        perm = build_permutation(scores).to(W.device)
+        if K > 16384 or scores.device != W.device:
+            perm, bad = build_permutation(scores).to(W.device), None
+        else:  # on the GPU: no copy, no sort on the host, one wait, at the end
+            perm, bad = build_permutation_device(scores, stream=stream)
+            if stream is not None:
+                torch.cuda.current_stream().wait_stream(stream)
         clip = errors = best = None
         if clip_grid is not None and w_bits == 4:
             Xcal = calib.reshape(-1, K).contiguous()
@@ -729,6 +751,8 @@ class PreparedLinear:
                                              grid=clip_grid, stream=stream)
         layer = cls.from_weight(W, perm, b, bias=bias, clip=clip, a_bits=a_bits,
                                 w_bits=w_bits)
+        if bad is not None and bad.item():  # NaN scores, as build_permutation refuses them
+            raise ClqError(1, "clq_build_permutation")
         return layer, dict(scores=scores, perm=perm, clip=clip, errors=errors, best=best)
 
     @property

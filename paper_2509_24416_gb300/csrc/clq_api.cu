@@ -331,6 +331,18 @@ clq_status clq_outlier_scores_metric(const void* calib, clq_dtype dtype, int32_t
                                               scores, static_cast<cudaStream_t>(stream)));
 }
 
+clq_status clq_build_permutation_device(const float* scores, int32_t K, int32_t* perm,
+                                        int32_t* bad, void* stream) {
+  if (scores == nullptr || perm == nullptr || bad == nullptr || K < 1) return CLQ_ERR_INVALID_ARG;
+  if (K > 16384) return CLQ_ERR_SHAPE;
+  if (!aligned(scores, 4) || !aligned(perm, 4) || !aligned(bad, 4)) return CLQ_ERR_ALIGN;
+  int32_t* status = nullptr;
+  const clq_status st = device_setup(&status);
+  if (st != CLQ_OK) return st;
+  return from_cuda(clq::launch_build_permutation(scores, K, perm, bad,
+                                                 static_cast<cudaStream_t>(stream)));
+}
+
 clq_status clq_prepare_weights(const void* W, clq_dtype dtype, int32_t N, int32_t K, int32_t ldw,
                                const int32_t* perm, int32_t b, const float* clip, uint8_t* Wq,
                                float* s_w, float* w_rot_dbg, void* stream) {

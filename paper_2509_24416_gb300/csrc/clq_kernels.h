@@ -39,6 +39,10 @@ cudaError_t launch_outlier_scores(const void* calib, int dtype, int B, int T, in
 cudaError_t launch_outlier_metric(const void* calib, int dtype, int B, int T, int K, int metric,
                                   float* scores, cudaStream_t st);
 
+// Column-swap vector from device scores, K <= 16384; *bad = 1 on a NaN score.
+cudaError_t launch_build_permutation(const float* scores, int K, int32_t* perm, int32_t* bad,
+                                     cudaStream_t st);
+
 struct GemmArgs {
   const float* s_x;   // [M]
   const float* s_w;   // [N]

@@ -135,4 +135,109 @@ cudaError_t launch_outlier_metric(const void* calib, int dtype, int B, int T, in
   return cudaGetLastError();
 }
 
+namespace {
+
+constexpr int kPermThreads = 1024;
+constexpr int kPermPer = 16;  // channels a thread, K <= 16384
+
+// Sum of x over the block, in every thread.
+__device__ __forceinline__ int block_sum(int x, int* red) {
+  x = __reduce_add_sync(0xffffffffu, x);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) red[w] = x;
+  __syncthreads();
+  const int r = __reduce_add_sync(0xffffffffu, red[lane]);
+  __syncthreads();
+  return r;
+}
+
+// Sum of x over the threads before this one.
+__device__ __forceinline__ int block_scan(int x, int* red) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int s = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, s, o);
+    if (lane >= o) s += t;
+  }
+  if (lane == 31) red[w] = s;
+  __syncthreads();
+  const int before = __reduce_add_sync(0xffffffffu, lane < w ? red[lane] : 0);
+  __syncthreads();
+  return before + s - x;
+}
+
+// The column-swap vector (Sec. 3.3, "Outlier Detection") from scores on the
+// device: the K / 2 channels of the highest scores, ties to the lower index, in
+// ascending order, then the others.  One block: the K / 2-th largest score by a
+// bitwise search on order-preserving keys (32 block-wide counts), the ties and the
+// positions by prefix sums over the channels, which threads own in index order.
+// It takes the place of a copy to the host, a sort there (157 us for K = 3072) and
+// a copy back.  NaN scores: *bad = 1 and the identity.
+__global__ void __launch_bounds__(kPermThreads) build_permutation_kernel(
+    const float* __restrict__ scores, int K, int32_t* __restrict__ perm,
+    int32_t* __restrict__ bad) {
+  __shared__ int red[32];
+  const int per = (K + kPermThreads - 1) / kPermThreads;
+  const int k0 = static_cast<int>(threadIdx.x) * per;
+  const int h = K / 2;
+  uint32_t key[kPermPer];
+  int nan = 0;
+#pragma unroll
+  for (int i = 0; i < kPermPer; ++i) {
+    key[i] = 0;  // below every float's key
+    if (i < per && k0 + i < K) {
+      const float f = scores[k0 + i] + 0.0f;  // -0 equals 0
+      nan |= f != f;
+      const uint32_t u = __float_as_uint(f);
+      key[i] = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+    }
+  }
+  nan = __syncthreads_or(nan);
+  if (threadIdx.x == 0) *bad = nan ? 1 : 0;
+  uint32_t cut = 0;  // the h-th largest key
+  for (int bit = 31; bit >= 0 && h > 0; --bit) {
+    const uint32_t t = cut | (1u << bit);
+    int c = 0;
+#pragma unroll
+    for (int i = 0; i < kPermPer; ++i) c += key[i] >= t;
+    if (block_sum(c, red) >= h) cut = t;
+  }
+  int above = 0, equal = 0;
+#pragma unroll
+  for (int i = 0; i < kPermPer; ++i) {
+    above += key[i] > cut;
+    equal += key[i] == cut;
+  }
+  const int left = h - block_sum(above, red);  // of the channels at the cut, the first `left`
+  int rank = block_scan(equal, red);
+  uint32_t high = 0;
+#pragma unroll
+  for (int i = 0; i < kPermPer; ++i) {
+    if (key[i] > cut || (key[i] == cut && rank < left)) high |= 1u << i;
+    rank += key[i] == cut;
+  }
+  if (h == 0) high = 0;
+  int pos = block_scan(__popc(high), red);  // high channels before this thread's
+#pragma unroll
+  for (int i = 0; i < kPermPer; ++i) {
+    const int k = k0 + i;
+    if (i >= per || k >= K) break;
+    const bool hi = (high >> i) & 1u;
+    if (nan)
+      perm[k] = k;
+    else
+      perm[hi ? pos : h + (k - pos)] = k;
+    pos += hi;
+  }
+}
+
+}  // namespace
+
+cudaError_t launch_build_permutation(const float* scores, int K, int32_t* perm, int32_t* bad,
+                                     cudaStream_t st) {
+  build_permutation_kernel<<<1, kPermThreads, 0, st>>>(scores, K, perm, bad);
+  return cudaGetLastError();
+}
+
 }  // namespace clq
