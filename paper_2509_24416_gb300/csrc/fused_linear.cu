@@ -103,6 +103,21 @@ constexpr int kConcStride = 18 * 1024;
 constexpr int kConcStages = 3;
 constexpr int kConcGemmStages = 3;
 
+// Zeroes the readiness counters and the tile counter of a call.  A kernel rather
+// than a memset, so that the fused kernel behind it may be launched with
+// programmatic overlap: its barriers, tensor memory and gather offsets are set up
+// while this one runs (a launch behind a memset waits for it to drain first).
+__global__ void zero_counters_kernel(uint32_t* ready, int n) {
+  pdl_wait();
+  pdl_launch_dependents();
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    ready[i] = 0u;
+}
+
+cudaError_t launch_zero_counters(uint32_t* ready, int n, cudaStream_t st) {
+  return launch_pdl(zero_counters_kernel, std::min((n + 255) / 256, 64), 256, 0, st, ready, n);
+}
+
 template <int BNT>
 struct Conc {
   using C = Cfg<false, false, BNT, 1, 1, 4, kConcGemmStages>;
@@ -166,6 +181,7 @@ __global__ void __launch_bounds__(FT, 1)
     rq::run<T, -1, false, kConcStride, kConcStages, false, false, PublishRows, true>(
         rq, smem + Conc<BNT>::RQ_OFF, tile_counter, PublishRows{ready, team}, team);
   } else {
+    pdl_wait();  // the counters are zeroed, and Y is this kernel's to write
     const Maps maps{&mapA, &mapB, use_tma_store ? &mapY : nullptr, nullptr, nullptr};
     pipeline<T, false, false, BNT, 1, 1, false, 4, kConcGemmStages, F6>(maps, g, smem,
                                                                               &bars, tmem, ready);
@@ -184,8 +200,8 @@ cudaError_t launch_conc(const CUtensorMap& mapA, const CUtensorMap& mapB,
   auto k = fused_concurrent_kernel<T, BNT, F6>;
   cudaError_t e = kernel_setup(reinterpret_cast<const void*>(k), smem, FT, nullptr);
   if (e != cudaSuccess) return e;
-  k<<<grid, FT, smem, st>>>(mapA, mapB, mapY, rq, g, ready, tile_counter, use_tma_store);
-  return cudaGetLastError();
+  return launch_pdl(k, grid, FT, smem, st, mapA, mapB, mapY, rq, g, ready, tile_counter,
+                    use_tma_store);
 }
 
 template <typename T, bool BPACK, int BNT, bool F6>
@@ -196,8 +212,8 @@ cudaError_t launch_t(const CUtensorMap& mapA, const CUtensorMap& mapB, const CUt
   auto k = fused_linear_kernel<T, BPACK, BNT, F6>;
   cudaError_t e = kernel_setup(reinterpret_cast<const void*>(k), smem, FT, nullptr);
   if (e != cudaSuccess) return e;
-  k<<<grid, FT, smem, st>>>(mapA, mapB, mapY, rq, g, ready, tile_counter, use_tma_store);
-  return cudaGetLastError();
+  return launch_pdl(k, grid, FT, smem, st, mapA, mapB, mapY, rq, g, ready, tile_counter,
+                    use_tma_store);
 }
 
 
@@ -237,8 +253,7 @@ cudaError_t launch_concurrent(const RotateQuantArgs& rq_in, const uint8_t* W, in
   if (smem > 227u * 1024u - 2048u) return cudaErrorInvalidValue;
 
   const int tiles_m = (g.M + BM - 1) / BM;
-  cudaError_t e =
-      cudaMemsetAsync(ready, 0, sizeof(uint32_t) * (static_cast<size_t>(tiles_m) + 1), st);
+  cudaError_t e = launch_zero_counters(ready, tiles_m + 1, st);
   if (e != cudaSuccess) return e;
   CUtensorMap mapA, mapB, mapY;
   if (!encode_codes_map(&mapA, rq.Q, a_codes, g.M, g.K, BM, 0) ||
@@ -295,8 +310,7 @@ cudaError_t launch_fused_linear(const RotateQuantArgs& rq_in, const uint8_t* W, 
   const size_t smem = std::max(gemm_bytes, rq_bytes) + 1024;
 
   const int tiles_m = (g.M + BM - 1) / BM;
-  cudaError_t e =
-      cudaMemsetAsync(ready, 0, sizeof(uint32_t) * (static_cast<size_t>(tiles_m) + 1), st);
+  cudaError_t e = launch_zero_counters(ready, tiles_m + 1, st);
   if (e != cudaSuccess) return e;
 
   CUtensorMap mapA, mapB, mapY;
