@@ -67,7 +67,8 @@ struct GemmArgs {
 // Output-channel tile width (256, 192, 128 or 64) of the product of
 // execution-layout operands, tiles of `rows` rows dealt to `units` CTAs or pairs;
 // mid: 192 is built for them, narrow: 128 and 64 are.
-int gemm_tile_n(int M, int N, int K, int rows, int units, bool mid, bool narrow);
+int gemm_tile_n(int M, int N, int K, int rows, int units, bool mid, bool narrow,
+                int epi = 1000);
 cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, int w_codes,
                              const GemmArgs& g, int out_dtype, cudaStream_t st);
 

@@ -384,15 +384,16 @@ bool encode_codes_map(CUtensorMap* map, const uint8_t* base, int codes, int rows
 // steps (clocks a step of a pair's main loop, measured alone: 587 / 458 / 390 for
 // 256 / 192 / 128 columns, and what 20 KB of operands take to arrive for 64) or
 // its epilogue, whichever is longer, and the last one's epilogue comes on top
-// (1000 clocks a 32-column block, a quarter of the columns each).  256 wins on
-// large products, 192 where N splits into its tiles with no more rounds (N =
-// 1152: 6 x 192 instead of 4.5 x 256), 128 and 64 where the wider tiles leave
-// units idle (us at 256 / 192 / 128 / 64 columns: 256 x 1152 x 1152 6.8 / 5.8 /
-// 4.9 / 4.4, 256 x 3072 x 12288 29.6 / 22.9 / 16.4 / 16.1, 1024 x 4608 x 1152 7.8 /
-// 8.1 / 7.6 / 9.6, 2048 x 4608 x 1152 10.6 / 10.6 / 11.0 / 15.1, 8192 x 1152 x
-// 4608 34.0 / 27.6 / 28.0 / 44.6; this rule is within 4 % of the best of them on 15
-// such shapes in each layout).  `narrow`: 64 and 128 are built for these operands; `mid`: 192 is.
-int gemm_tile_n(int M, int N, int K, int rows, int units, bool mid, bool narrow) {
+// (`epi` clocks for each 64 columns: 1000 with eight epilogue warps, 1100 with the
+// fused kernel's four).  256 wins on large products, 192 where N splits into its
+// tiles with no more rounds (N = 1152: 6 x 192 instead of 4.5 x 256), 128 and 64
+// where the wider tiles leave units idle (us at 256 / 192 / 128 / 64 columns: 256 x
+// 1152 x 1152 6.8 / 5.8 / 4.9 / 4.4, 256 x 3072 x 12288 29.6 / 22.9 / 16.4 / 16.1,
+// 1024 x 4608 x 1152 7.8 / 8.1 / 7.6 / 9.6, 2048 x 4608 x 1152 10.6 / 10.6 / 11.0 /
+// 15.1, 8192 x 1152 x 4608 34.0 / 27.6 / 28.0 / 44.6; this rule is within 4 % of
+// the best of them on 15 such shapes in each layout).  `narrow`: 64 and 128 are
+// built for these operands; `mid`: 192 is.
+int gemm_tile_n(int M, int N, int K, int rows, int units, bool mid, bool narrow, int epi) {
   const long mt = (M + rows - 1) / rows;
   const double nk = (K + BK - 1) / BK;
   const int width[4] = {256, 192, 128, 64};
@@ -402,8 +403,8 @@ int gemm_tile_n(int M, int N, int K, int rows, int units, bool mid, bool narrow)
   for (int i = 0; i < 4; ++i) {
     if ((width[i] == 192 && !mid) || (width[i] < 192 && !narrow)) continue;
     const long rounds = (mt * ((N + width[i] - 1) / width[i]) + units - 1) / units;
-    const double epi = 1000.0 * width[i] / 64;
-    const double cost = rounds * std::max(nk * step[i], epi + 500) + epi;
+    const double drain = epi * width[i] / 64.0;
+    const double cost = rounds * std::max(nk * step[i], drain + 500) + drain;
     if (cost < best_cost) {
       best_cost = cost;
       best = width[i];
