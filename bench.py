@@ -88,9 +88,10 @@ def peaks():
 # Source files each kernel is built from (globs under csrc/): a recorded ncu
 # figure stays valid while these files are unchanged.
 KERNEL_SOURCES = {
-    "w4a4_gemm": ("w4a4_gemm.cu", "gemm_*.cuh", "clq_device.cuh", "clq_kernels.h"),
+    "w4a4_gemm": ("w4a4_gemm.cu", "gemm_*.cu", "gemm_*.cuh", "gemm_launch.h", "clq_device.cuh",
+                  "clq_kernels.h"),
     "rotate_quant": ("rotate_quant*.cu", "rq_*.cuh", "clq_device.cuh", "clq_kernels.h"),
-    "fused_linear": ("fused_linear.cu", "gemm_*.cuh", "rq_*.cuh", "clq_device.cuh",
+    "fused_linear": ("fused_*.cu", "fused_*.cuh", "gemm_*.cuh", "rq_*.cuh", "clq_device.cuh",
                      "clq_kernels.h"),
 }
 
@@ -138,9 +139,10 @@ def gemm_intake_bound(M, shapes, sms, sm_mhz, bytes_per_clk):
     the same run by clq_peak_operand_stream, counted in shared-memory bytes,
     which are 128 per row and K step for E4M3 and E2M3 alike), and each 128 x w
     output tile brings (128 + w) K operand bytes in and sends 2 x 128 w output
-    bytes out through the same engine.  Tiles are those the launcher picks
-    (w = 192 when it covers N in whole tiles with no more rounds, else 256),
-    dealt round-robin, so a layer takes ceil(tiles / SMs) tile-times.  Returns
+    bytes out through the same engine.  Tiles of one CTA, the widths the launcher
+    takes for large products (w = 192 when it covers N in whole tiles with no more
+    rounds, else 256; its CTA pairs bring half of B per SM, so they may exceed
+    this), dealt round-robin, so a layer takes ceil(tiles / SMs) tile-times.  Returns
     TFLOP/s over the layer set."""
     rate = bytes_per_clk * sm_mhz * 1e6
     mt = (M + 127) // 128
@@ -1105,7 +1107,8 @@ def main():
             "bytes_per_clk_per_sm": round(fill, 2),
             "model": "TMA fill of shared memory per SM measured in this run "
                      "(clq_peak_operand_stream, no MMA) at the median SM clock, output "
-                     "writes through the same engine, the launcher's tiles"}
+                     "writes through the same engine, 128-row tiles of one CTA each (the "
+                     "launcher's CTA pairs bring half of B per SM)"}
     rq_roof = None
     if not args.fused:
         rq_ach = rq_bytes_all / rq_total_s / 1e9

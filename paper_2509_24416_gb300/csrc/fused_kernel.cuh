@@ -24,7 +24,7 @@
 //
 // Concurrent form (fused_concurrent_kernel; E4M3 weights, K <= 9216): the
 // two run side by side.  Warps 0-5 of every CTA are the GEMM pipeline with
-// four epilogue warps and three stages; warps 6-14 rotate and quantize token
+// four epilogue warps and three to six stages; warps 6-14 rotate and quantize token
 // rows in the shared memory the GEMM leaves free, and warp 15 claims their
 // tiles, loads and publishes them (rq::run's loader mode).  The GEMM of a
 // token block starts as soon as its rows are published.

@@ -7,10 +7,11 @@
 // (ASYM) asymmetrically with the row's min and max as bounds (Eq. 1 with
 // dynamic l and r), stored as centered codes q - 2^(n-1).
 //
-// The standalone activation path with symmetric 4-bit codes in the E4M3 or
-// E2M3 layout and b >= 32 runs the specialized loops of rq_pair.cuh and
-// rq_wide.cuh; this general loop serves every other setting (packed codes,
-// b < 32, 8-bit and asymmetric codes, clipped weights) and the fused kernel.
+// Unclipped codes in an execution layout run the specialized loops where those
+// reach: rq_wide.cuh at b >= 64 (E4M3, E2M3, split planes, asymmetric codes),
+// rq_pair.cuh at b = 32 (symmetric E4M3 and E2M3).  This general loop serves every
+// other setting (packed codes, smaller blocks, clipped weights) and the fused
+// kernel.
 //
 // Every thread of the CTA takes part.  The CTA walks tiles of R rows.  Raw
 // rows stream into a ring of STAGES shared-memory buffers (STRIDE bytes

@@ -1,5 +1,5 @@
 // Paired-row rotate-quantize: the hot-path variant of the tile loop in
-// rq_device.cuh, for symmetric 4-bit activation codes (b >= 16, no clip):
+// rq_device.cuh, for symmetric 4-bit codes (launched at b = 32, no clip):
 // the OBS transform of arxiv 2509.24416 Sec. 3.3 (column gather by the swap
 // vector, block Sylvester Hadamard H_b) followed by per-token symmetric
 // quantization with a dynamic fp32 scale (Sec. 3.1, Eq. 1 with l = -r).
