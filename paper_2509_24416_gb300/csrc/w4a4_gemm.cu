@@ -133,24 +133,22 @@ __device__ __forceinline__ void encode_group(uint8_t* __restrict__ row, int code
   }
 }
 
-// Four E4M3 bytes of integer codes -> the codes' two's-complement nibbles, one a
-// byte: magnitudes 0x00 0x38 0x40 0x44 0x48 0x4A 0x4C 0x4E are 0 .. 7.
-__device__ __forceinline__ uint32_t e4m3_to_nibbles(uint32_t w) {
-  constexpr uint32_t ones = 0x01010101u;
-  const uint32_t b6 = (w >> 6) & ones, b3 = (w >> 3) & ones;
-  const uint32_t hi = (b6 & b3) * 0xFFu;           // 4 .. 7: two mantissa bits
-  const uint32_t mid = (b6 & (b3 ^ ones)) * 0xFFu;  // 2, 3: one
-  const uint32_t low = (b6 ^ ones) * 0xFFu;         // 0, 1
-  const uint32_t v = (hi & (0x04040404u | ((w >> 1) & 0x03030303u))) |
-                     (mid & (0x02020202u | ((w >> 2) & ones))) | (low & ((w >> 5) & ones));
-  const uint32_t neg = (w >> 7) & ones;
-  return ((v ^ (neg * 0x0Fu)) + neg) & 0x0F0F0F0Fu;
-}
-
-// Four nibbles, one a byte -> two packed bytes.
-__device__ __forceinline__ uint32_t pack_nibbles(uint32_t n) {
-  const uint32_t x = n | (n >> 4);
-  return (x & 0xFFu) | ((x >> 8) & 0xFF00u);
+// Eight E4M3 bytes of integer codes -> packed nibbles.  The magnitudes 0x00 0x38
+// 0x40 0x44 0x48 0x4A 0x4C 0x4E of 0 .. 7 differ in the three bits b3 ^ b5, b2 ^ b4,
+// b1 ^ b6, which index two byte tables, the codes' nibbles and their negatives'.
+// Bytes that are no such code give some nibble in [-7, 7].
+__device__ __forceinline__ uint32_t e4m3_to_packed(uint32_t x, uint32_t y) {
+  const uint32_t P0 = 0x03010200u, P1 = 0x06070405u;  // 0 2 1 3 5 4 7 6
+  const uint32_t N0 = 0x0D0F0E00u, N1 = 0x0A090C0Bu;  // their negatives, mod 16
+  auto index = [](uint32_t w) {
+    return ((w >> 1) ^ ((w >> 3) & 0x06060606u) ^ ((w >> 6) & 0x01010101u)) & 0x07070707u;
+  };
+  const uint32_t sel = index(x) | (index(y) << 4);  // nibbles x0 y0 x1 y1 x2 y2 x3 y3
+  const uint32_t m0 = prmt(x, y, 0xD9C8u), m1 = prmt(x, y, 0xFBEAu);  // their signs
+  const uint32_t lo = (prmt(P0, P1, sel) & ~m0) | (prmt(N0, N1, sel) & m0);
+  const uint32_t hi = (prmt(P0, P1, sel >> 16) & ~m1) | (prmt(N0, N1, sel >> 16) & m1);
+  // x0 | x1 << 4 and y0 | y1 << 4 in the low bytes of the first, x2.. and y2.. of the other
+  return prmt(lo | (lo >> 12), hi | (hi >> 12), 0x5140u);
 }
 
 // Code array in one 4-bit layout -> another, one thread a group of 16 codes.
@@ -170,18 +168,10 @@ __global__ void convert_codes_kernel(const uint8_t* __restrict__ src, int src_co
        i += static_cast<size_t>(gridDim.x) * blockDim.x) {
     if (src_codes == CLQ_CODES_E4M3 && dst_codes == CLQ_CODES_INT4_PACKED) {
       const uint4 w = reinterpret_cast<const uint4*>(src)[i];  // rows are whole groups
-      uint2 o;
-      o.x = pack_nibbles(e4m3_to_nibbles(w.x)) | (pack_nibbles(e4m3_to_nibbles(w.y)) << 16);
-      o.y = pack_nibbles(e4m3_to_nibbles(w.z)) | (pack_nibbles(e4m3_to_nibbles(w.w)) << 16);
+      const uint2 o = make_uint2(e4m3_to_packed(w.x, w.y), e4m3_to_packed(w.z, w.w));
       const uint2 a = nibbles_to_e4m3(o.x), b = nibbles_to_e4m3(o.y);
-      // a zero code may carry a sign: compare magnitudes there (0 - 1 borrows, so
-      // only a byte that is 0x00 or 0x80 both ways is let off)
-      auto differs = [](uint32_t x, uint32_t back) {
-        const uint32_t d = x ^ back;
-        const uint32_t zero = ((back & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) & 0x80808080u;  // 0x80: non-zero
-        return (d & ~(~zero & 0x80808080u)) != 0;
-      };
-      if (!(differs(w.x, a.x) || differs(w.y, a.y) || differs(w.z, b.x) || differs(w.w, b.y))) {
+      // magnitudes only: a code's sign went through, and a zero code may carry one
+      if ((((w.x ^ a.x) | (w.y ^ a.y) | (w.z ^ b.x) | (w.w ^ b.y)) & 0x7F7F7F7Fu) == 0) {
         reinterpret_cast<uint2*>(dst)[i] = o;
         continue;
       }
