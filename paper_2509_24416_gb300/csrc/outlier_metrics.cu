@@ -140,44 +140,32 @@ namespace {
 constexpr int kPermThreads = 1024;
 constexpr int kPermPer = 16;  // channels a thread, K <= 16384
 
-// Sum of x over the block, in every thread.
-__device__ __forceinline__ int block_sum(int x, int* red) {
+// Sums of (x, y) over the block, in every thread, through red (32 entries that
+// nothing else reads or writes until the next barrier but one).
+__device__ __forceinline__ int2 block_sum2(int x, int y, int2* red) {
   x = __reduce_add_sync(0xffffffffu, x);
+  y = __reduce_add_sync(0xffffffffu, y);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) red[w] = x;
+  if (lane == 0) red[w] = make_int2(x, y);
   __syncthreads();
-  const int r = __reduce_add_sync(0xffffffffu, red[lane]);
-  __syncthreads();
-  return r;
-}
-
-// Sum of x over the threads before this one.
-__device__ __forceinline__ int block_scan(int x, int* red) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int s = x;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, s, o);
-    if (lane >= o) s += t;
-  }
-  if (lane == 31) red[w] = s;
-  __syncthreads();
-  const int before = __reduce_add_sync(0xffffffffu, lane < w ? red[lane] : 0);
-  __syncthreads();
-  return before + s - x;
+  const int2 r = red[lane];
+  return make_int2(__reduce_add_sync(0xffffffffu, r.x), __reduce_add_sync(0xffffffffu, r.y));
 }
 
 // The column-swap vector (Sec. 3.3, "Outlier Detection") from scores on the
 // device: the K / 2 channels of the highest scores, ties to the lower index, in
 // ascending order, then the others.  One block: the K / 2-th largest score by a
-// bitwise search on order-preserving keys (32 block-wide counts), the ties and the
-// positions by prefix sums over the channels, which threads own in index order.
-// It takes the place of a copy to the host, a sort there (157 us for K = 3072) and
-// a copy back.  NaN scores: *bad = 1 and the identity.
+// search on order-preserving keys, two bits a round (three block-wide counts, two
+// of them in one word), until a threshold has just K / 2 keys at or above it; the
+// ties and the positions by one prefix sum over the channels, which threads own in
+// index order.  It takes the place of a copy to the host, a sort there (157 us for
+// K = 3072) and a copy back.  A chain of latencies on one SM: with a bit a round,
+// two barriers each, and all sixteen channels of a thread counted it took 17.0 us
+// at K = 3072, now 10.6.  NaN scores: *bad = 1 and the identity.
 __global__ void __launch_bounds__(kPermThreads) build_permutation_kernel(
     const float* __restrict__ scores, int K, int32_t* __restrict__ perm,
     int32_t* __restrict__ bad) {
-  __shared__ int red[32];
+  __shared__ int2 red[3][32];  // alternating in the search, the last for the prefix sum
   const int per = (K + kPermThreads - 1) / kPermThreads;
   const int k0 = static_cast<int>(threadIdx.x) * per;
   const int h = K / 2;
@@ -195,39 +183,55 @@ __global__ void __launch_bounds__(kPermThreads) build_permutation_kernel(
   }
   nan = __syncthreads_or(nan);
   if (threadIdx.x == 0) *bad = nan ? 1 : 0;
-  uint32_t cut = 0;  // the h-th largest key
-  for (int bit = 31; bit >= 0 && h > 0; --bit) {
-    const uint32_t t = cut | (1u << bit);
-    int c = 0;
+  // at least h keys are at or above it, at last just h or the h-th largest key
+  uint32_t cut = h > 0 ? 0u : ~0u;
+  for (int bit = 30; bit >= 0 && h > 0; bit -= 2) {
+    const uint32_t one = 1u << bit;
+    int c1 = 0, c23 = 0;  // counts up to 16384 in 16 bits
 #pragma unroll
-    for (int i = 0; i < kPermPer; ++i) c += key[i] >= t;
-    if (block_sum(c, red) >= h) cut = t;
+    for (int i = 0; i < kPermPer; ++i) {
+      if (i >= per) break;
+      c1 += key[i] >= (cut | one);
+      c23 += (key[i] >= (cut | (2 * one)) ? 1 : 0) + (key[i] >= (cut | (3 * one)) ? 65536 : 0);
+    }
+    const int2 n = block_sum2(c1, c23, red[(bit >> 1) & 1]);
+    const int n1 = n.x, n2 = n.y & 0xFFFF, n3 = n.y >> 16;
+    const int j = n3 >= h ? 3 : n2 >= h ? 2 : n1 >= h ? 1 : 0;
+    cut |= static_cast<uint32_t>(j) << bit;
+    if (j > 0 && (j == 3 ? n3 : j == 2 ? n2 : n1) == h) break;  // no tie to settle
   }
-  int above = 0, equal = 0;
+  int mine = 0;  // keys above the cut, and at it times 65536
 #pragma unroll
   for (int i = 0; i < kPermPer; ++i) {
-    above += key[i] > cut;
-    equal += key[i] == cut;
+    if (i >= per) break;
+    mine += (key[i] > cut ? 1 : 0) + (key[i] == cut ? 65536 : 0);
   }
-  const int left = h - block_sum(above, red);  // of the channels at the cut, the first `left`
-  int rank = block_scan(equal, red);
-  uint32_t high = 0;
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int sum = mine;  // over the threads of the warp up to this one
 #pragma unroll
-  for (int i = 0; i < kPermPer; ++i) {
-    if (key[i] > cut || (key[i] == cut && rank < left)) high |= 1u << i;
-    rank += key[i] == cut;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, sum, o);
+    if (lane >= o) sum += t;
   }
-  if (h == 0) high = 0;
-  int pos = block_scan(__popc(high), red);  // high channels before this thread's
+  if (lane == 31) red[2][w].x = sum;
+  __syncthreads();
+  const int warp_sum = red[2][lane].x;
+  const int before = __reduce_add_sync(0xffffffffu, lane < w ? warp_sum : 0) + sum - mine;
+  // of the channels at the cut, the first `left` are high
+  const int left = h - (__reduce_add_sync(0xffffffffu, warp_sum) & 0xFFFF);
+  int rank = before >> 16;                            // channels at the cut before this one
+  int pos = (before & 0xFFFF) + (rank < left ? rank : left);  // high channels before it
 #pragma unroll
   for (int i = 0; i < kPermPer; ++i) {
     const int k = k0 + i;
     if (i >= per || k >= K) break;
-    const bool hi = (high >> i) & 1u;
+    const bool at = key[i] == cut;
+    const bool hi = key[i] > cut || (at && rank < left);
     if (nan)
       perm[k] = k;
     else
       perm[hi ? pos : h + (k - pos)] = k;
+    rank += at;
     pos += hi;
   }
 }

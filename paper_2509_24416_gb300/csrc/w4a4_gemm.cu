@@ -156,8 +156,8 @@ __device__ __forceinline__ uint32_t e4m3_to_packed(uint32_t x, uint32_t y) {
 // written as 0 and reported.  Between E4M3 bytes and packed nibbles whole words
 // are converted, checked by the way back, and only a group that holds something
 // else goes code by code; with one byte a load and store the kernel took 24 us for
-// 9216 x 3072 codes E4M3 -> packed, 46 back (copying them 6); now 15.4 and
-// 7.3.
+// 9216 x 3072 codes E4M3 -> packed, 46 back (copying them 6); by whole words with
+// arithmetic on the magnitudes 15.4; now 11.4 and 7.3.
 __global__ void convert_codes_kernel(const uint8_t* __restrict__ src, int src_codes,
                                      uint8_t* __restrict__ dst, int dst_codes, int rows, int K,
                                      int32_t* status) {
