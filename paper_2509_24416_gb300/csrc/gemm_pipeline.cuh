@@ -43,8 +43,11 @@
 // epilogue adds 4000.  The stages matter most once operands come from further
 // away: 4608 x 12288 x 3072 took 112.6 us with four 32 KB stages, 98.3 with
 // five and 90.1 with six, which is why the staging buffers are 2 KB a warp.
-// The epilogue warps keep their column data to themselves and read their row
-// scales before the accumulator is complete: no barrier joins them.
+// The epilogue warps keep their column data to themselves, no barrier joins them,
+// and they load it and their row scales a tile ahead: at K = 1152 a tile's epilogue
+// takes about as long as its MMAs, and those loads' latency stood at its head (8192
+// x 3456 x 1152 with asymmetric activations 27.9 -> 23.6 us, symmetric in a layer,
+// where rotate-quant has just written the scales, 32.1 -> 30.8 for both kernels).
 // With `ready` counters (fused kernel), the producer waits until all rows of
 // a tile's token block have been published before loading its A tiles.
 // Every wait is bounded; on a timeout the roles drain their own copies and
@@ -365,6 +368,34 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
     const uint32_t empty0 = CG == 2 ? cluster_addr(&bars->acc_empty[0], 0) : 0;  // leader's
     uint8_t* staging = smem + C::OFF_EPI + ew * EPI_BYTES;
     float* col = reinterpret_cast<float*>(smem + C::OFF_COL) + ew * C::COL_FLOATS;
+    // A tile's column data (s_w / b, bias, zero-point sums) and row scales, loaded
+    // into registers a tile ahead.
+    constexpr int NC = NCOL / 32;
+    float sc[NC], bi[NC], wz[NC], nsx[4], nlo[4];
+    auto load_scales = [&](int t) {
+      const int mb = t / tiles_n;
+      const int m0 = mb * TM + rank * BM;
+      const int n0 = (t - mb * tiles_n) * BNT;
+#pragma unroll
+      for (int j = 0; j < NC; ++j) {
+        const int cn = n0 + part * NCOL + 32 * j + lane;
+        const bool in = t < tiles && cn < g.N;
+        sc[j] = in ? __ldg(g.s_w + cn) : 0.f;
+        bi[j] = in && g.bias != nullptr
+                    ? Num<OutT>::to_f(__ldg(static_cast<const uint16_t*>(g.bias) + cn))
+                    : 0.f;
+        if (ASYM) wz[j] = in ? __ldg(g.wsum + cn) : 0.f;
+      }
+      // a thread's fragments hold rows 8 k + lane / 4 of the warp's 32
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int row = m0 + quarter * EPI_ROWS + 8 * k + (lane >> 2);
+        const bool in = ready == nullptr && t < tiles && row < g.M;
+        nsx[k] = in ? __ldg(g.s_x + row) : 0.f;
+        if (ASYM) nlo[k] = in ? __ldg(g.lo + row) : 0.f;
+      }
+    };
+    load_scales(unit);
     int tc = 0;
     for (int t = unit; t < tiles; t += units, ++tc) {
       const int mb = t / tiles_n;
@@ -372,31 +403,21 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
       const int n0 = (t - mb * tiles_n) * BNT;
       const int buf = C::NBUF == 1 ? 0 : (tc & 1);
       const uint32_t use = C::NBUF == 1 ? tc : (tc >> 1);
-      // This warp's column data and row scales, while the tile's MMAs run.
 #pragma unroll
-      for (int j = lane; j < NCOL; j += 32) {
-        const int cn = n0 + part * NCOL + j;
-        float sc = 0.f, bi = 0.f;
-        if (cn < g.N) {
-          sc = g.s_w[cn] * g.inv_b;
-          if (g.bias != nullptr) bi = Num<OutT>::to_f(static_cast<const uint16_t*>(g.bias)[cn]);
-        }
-        col[j] = sc;
-        col[NCOL + j] = bi;
-        if (ASYM) col[2 * NCOL + j] = cn < g.N ? g.wsum[cn] * sc : 0.f;
+      for (int j = 0; j < NC; ++j) {
+        const float s = sc[j] * g.inv_b;
+        col[32 * j + lane] = s;
+        col[NCOL + 32 * j + lane] = bi[j];
+        if (ASYM) col[2 * NCOL + 32 * j + lane] = wz[j] * s;
       }
-      // Row scales: a thread's fragments hold rows 8 k + lane / 4 of the warp's
-      // 32.  Asymmetric codes: the value of code 0 is min + 2^(n-1) delta.
+      // Asymmetric codes: the value of code 0 is min + 2^(n-1) delta.
       float sx[4], zm[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const int row = m0 + quarter * EPI_ROWS + 8 * k + (lane >> 2);
-        sx[k] = zm[k] = 0.f;
-        if (ready == nullptr && row < g.M) {
-          sx[k] = __ldg(g.s_x + row);
-          if (ASYM) zm[k] = fmaf(g.zp_shift, sx[k], __ldg(g.lo + row));
-        }
+        sx[k] = nsx[k];
+        zm[k] = ASYM ? fmaf(g.zp_shift, sx[k], nlo[k]) : 0.f;
       }
+      load_scales(t + units);
       __syncwarp();
       bool ok = mbar_wait_bounded(&bars->acc_full[buf], use & 1, abort, g.status,
                                   kWaitLimitNs);
