@@ -23,8 +23,8 @@
 // __threadfence, atomicAdd), then turns into a GEMM pipeline.
 //
 // Concurrent form (fused_concurrent_kernel; E4M3 weights, K <= 9216): the
-// two run side by side.  Warps 0-5 of every CTA are the GEMM pipeline with
-// four epilogue warps and three to six stages; warps 6-14 rotate and quantize token
+// two run side by side.  Warps 0-5 of every CTA are the GEMM pipeline (of CTA
+// pairs where tiles are wide) with four epilogue warps and four to six stages; warps 6-14 rotate and quantize token
 // rows in the shared memory the GEMM leaves free, and warp 15 claims their
 // tiles, loads and publishes them (rq::run's loader mode).  The GEMM of a
 // token block starts as soon as its rows are published.
@@ -104,13 +104,19 @@ constexpr int kTeamCompute = kTeamThreads - 32;   // 288
 constexpr uint32_t kTeamBarrier = 2;  // 0: CTA, 1: GEMM epilogue, 2-3: team
 constexpr int kConcStride = 18 * 1024;
 constexpr int kConcStages = 3;
-// GEMM stages of the concurrent form: what fits beside three rotate-quant stages.
+// The concurrent form's GEMM: CTA pairs for the wide tiles, which large products
+// take (4608 x 3072 x 12288 136 -> 121 us, 16384 x 1152 x 4608 82 -> 73, 2048 x 1152 x
+// 4608 19.9 -> 19.6), single CTAs for the narrow ones, where a pair's joint start costs
+// more than its shared operands give (256 x 1152 x 1152 10.2 us, as pairs 11.2).
 template <int BNT>
-constexpr int kConcGemmStages = BNT >= 192 ? 3 : BNT == 128 ? 4 : 6;
+constexpr int kConcCG = BNT >= 192 ? 2 : 1;
+// Its stages: what fits beside three rotate-quant stages.
+template <int BNT>
+constexpr int kConcGemmStages = BNT == 192 ? 5 : BNT == 64 ? 6 : 4;
 
 template <int BNT>
 struct Conc {
-  using C = Cfg<false, false, BNT, 1, 1, 4, kConcGemmStages<BNT>>;
+  using C = Cfg<false, false, BNT, 1, 1, 4, kConcGemmStages<BNT>, 0, kConcCG<BNT>>;
   static constexpr size_t RQ_OFF = (C::BYTES + 1023) & ~static_cast<size_t>(1023);
 };
 
@@ -157,9 +163,13 @@ __global__ void __launch_bounds__(FT, 1)
   __shared__ Barriers bars;
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  setup<false, false, BNT, 1, 1, 4, kConcGemmStages<BNT>>(&bars);
+  constexpr int CG = kConcCG<BNT>;
+  setup<false, false, BNT, 1, 1, 4, kConcGemmStages<BNT>, 0, CG>(&bars);
   tc_fence_before();
-  __syncthreads();
+  if (CG == 2)
+    cluster_sync();  // the peer's barriers exist before anything arrives on them
+  else
+    __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars.tmem_slot;
 
@@ -173,12 +183,15 @@ __global__ void __launch_bounds__(FT, 1)
   } else {
     pdl_wait();  // the counters are zeroed, and Y is this kernel's to write
     const Maps maps{&mapA, &mapB, use_tma_store ? &mapY : nullptr, nullptr, nullptr};
-    pipeline<T, false, false, BNT, 1, 1, false, 4, kConcGemmStages<BNT>, F6>(maps, g, smem,
-                                                                              &bars, tmem, ready);
+    pipeline<T, false, false, BNT, 1, 1, false, 4, kConcGemmStages<BNT>, F6, 0, CG>(
+        maps, g, smem, &bars, tmem, ready);
   }
   tc_fence_before();
-  __syncthreads();
-  teardown(tmem, C::TMEM);
+  if (CG == 2)
+    cluster_sync();  // a pair leaves together
+  else
+    __syncthreads();
+  teardown<CG>(tmem, C::TMEM);
 }
 
 template <typename T, int BNT, bool F6>
@@ -192,8 +205,8 @@ cudaError_t launch_conc_t(const CUtensorMap& mapA, const CUtensorMap& mapB,
   auto k = fused_concurrent_kernel<T, BNT, F6>;
   cudaError_t e = kernel_setup(reinterpret_cast<const void*>(k), smem, FT, nullptr);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k, grid, FT, smem, st, mapA, mapB, mapY, rq, g, ready, tile_counter,
-                    use_tma_store);
+  return launch_cluster_pdl(k, grid, kConcCG<BNT>, FT, smem, st, mapA, mapB, mapY, rq, g, ready,
+                            tile_counter, use_tma_store);
 }
 
 template <typename T>

@@ -54,7 +54,9 @@ cudaError_t launch_concurrent(const RotateQuantArgs& rq_in, const uint8_t* W, in
   rq.rows_per_tile = R;
   // The narrow tiles' gain, us: 256 x 1152 x 1152 12.9 -> 10.5, 875 x 5120 x 192 32.1 ->
   // 23.7, 1024 x 1152 x 1152 13.4 -> 11.4.
-  const int bn = gemm_tile_n(g.M, g.N, g.K, BM, sms, true, true, 1100);
+  int bn = gemm_tile_n(g.M, g.N, g.K, BM, sms, true, true, 1100);
+  const int cg = bn >= 192 ? 2 : 1;  // CTA pairs (kConcCG)
+  if (cg == 2) bn = gemm_tile_n(g.M, g.N, g.K, 2 * BM, sms / 2, true, false, 1100);
   const size_t rq_bytes = rq::smem_bytes(R, kConcStride, kConcStages);
 
   const int tiles_m = (g.M + BM - 1) / BM;
@@ -62,7 +64,7 @@ cudaError_t launch_concurrent(const RotateQuantArgs& rq_in, const uint8_t* W, in
   if (e != cudaSuccess) return e;
   CUtensorMap mapA, mapB, mapY;
   if (!encode_codes_map(&mapA, rq.Q, a_codes, g.M, g.K, BM, 0) ||
-      !encode_codes_map(&mapB, W, w_codes, g.N, g.K, bn, 0))
+      !encode_codes_map(&mapB, W, w_codes, g.N, g.K, bn / cg, 0))
     return cudaErrorInvalidValue;
   const int use_tma_store = (g.N % 8 == 0) ? 1 : 0;
   if (use_tma_store) {
@@ -71,7 +73,7 @@ cudaError_t launch_concurrent(const RotateQuantArgs& rq_in, const uint8_t* W, in
     mapY = mapA;  // unused
   }
   auto* go = dtype == CLQ_F16 ? launch_conc_f16 : launch_conc_bf16;
-  return go(mapA, mapB, mapY, rq, g, bn, f6, ready, use_tma_store, rq_bytes, sms, st);
+  return go(mapA, mapB, mapY, rq, g, bn, f6, ready, use_tma_store, rq_bytes, sms / cg * cg, st);
 }
 
 }  // namespace

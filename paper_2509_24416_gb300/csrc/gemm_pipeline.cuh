@@ -111,7 +111,7 @@ struct Cfg {
   static_assert(EPI_WARPS == 4 || !UNPACK, "packed operands leave four epilogue warps");
   static_assert(EPI_NCOL % EPI_COLS == 0 && STAGE % 1024 == 0, "whole blocks, aligned staging");
   static_assert(SMAX <= MAX_STAGES, "barrier arrays hold MAX_STAGES stages");
-  static_assert(CG == 1 || (CG == 2 && !UNPACK && EW == 0), "pairs: E4M3 / E2M3 operands only");
+  static_assert(CG == 1 || (CG == 2 && !UNPACK), "pairs: E4M3 / E2M3 operands only");
   static_assert((SEP != 0) == (PA == 2 && PB == 2) && (SEP == 0 || SEP == 2 || SEP == 3),
                 "SEP: two or three accumulators, 8-bit x 8-bit codes");
   static_assert(ACC <= 512, "one buffer fits tensor memory");
@@ -252,9 +252,9 @@ __device__ __forceinline__ void pipeline(const Maps& maps, const GemmArgs& g, ui
         const int mb = t / tiles_n;
         const int m0 = mb * TM + rank * BM;
         const int n0 = (t - mb * tiles_n) * BNT + rank * (BNT / CG);
-        if (ready != nullptr && mb != ready_m) {
-          if (!wait_rows_ready(ready, mb, static_cast<uint32_t>(min(BM, g.M - m0)), abort,
-                               g.status)) {
+        if (ready != nullptr && mb != ready_m && m0 < g.M) {  // this CTA's 128 rows
+          if (!wait_rows_ready(ready, mb * CG + rank, static_cast<uint32_t>(min(BM, g.M - m0)),
+                               abort, g.status)) {
             ok = false;
             break;
           }

@@ -147,3 +147,24 @@ def test_w8a8_accumulators_at_their_limit(K, M, N):
     want = qx.double() @ qw.double().t()
     assert torch.equal(acc.double(), want)
     assert clq.device_status() == 0
+
+
+@pytest.mark.parametrize("w_codes", [None, clq.CLQ_CODES_E2M3])
+@pytest.mark.parametrize("M,N,K", [(1900, 4600, 1152), (2200, 4701, 640), (9700, 1152, 1152),
+                                   (8322, 1160, 1152)])
+def test_fused_wide_tiles_match_separate(M, N, K, w_codes):
+    """The one-kernel layer on the wide tiles that CTA pairs share, with a last pair
+    whose second CTA has no rows or few and ragged columns: the separate kernels'
+    output bit for bit, twice over one workspace."""
+    g = torch.Generator(device=DEV).manual_seed(N)
+    b = 64
+    X = torch.randn(M, K, generator=g, device=DEV).half()
+    W = (0.05 * torch.randn(N, K, generator=g, device=DEV)).half()
+    bias = torch.randn(N, generator=g, device=DEV).half()
+    perm = torch.randperm(K, generator=g, device=DEV).to(torch.int32)
+    layer = clq.PreparedLinear.from_weight(W, perm, b, bias=bias, w_codes=w_codes)
+    ws = clq.fused_workspace(M, K, DEV)
+    want = layer(X)
+    for _ in range(2):
+        assert torch.equal(layer(X, fused=True, workspace=ws), want)
+    assert clq.device_status() == 0
