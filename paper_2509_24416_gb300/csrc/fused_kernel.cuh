@@ -49,6 +49,13 @@ constexpr int FT = 512;
 // Epilogue warps of the sequential form (unpack warps leave room for four).
 template <bool BPACK>
 constexpr int kSeqEpiWarps = BPACK ? 4 : 8;
+// Its GEMM: CTA pairs unless the weights are packed (4608 x 3072 x 12288 190 -> 169 us,
+// 16384 x 1152 x 9344 392 -> 362, 64 x 1152 x 12288 44.6 -> 40.5; 3129 x 4544 x 11008,
+// where pairs need a round more, 157.5 -> 161).
+template <bool BPACK>
+constexpr int kSeqCG = BPACK ? 1 : 2;
+template <bool BPACK>
+using SeqCfg = Cfg<false, BPACK, BN, 1, 1, kSeqEpiWarps<BPACK>, MAX_STAGES, 0, kSeqCG<BPACK>>;
 
 // Adds the rows [row0, row0 + rows) to the ready counters of the 128-token
 // blocks they fall in (a tile of rows may straddle two blocks); RELEASE: each
@@ -105,8 +112,8 @@ constexpr uint32_t kTeamBarrier = 2;  // 0: CTA, 1: GEMM epilogue, 2-3: team
 constexpr int kConcStride = 18 * 1024;
 constexpr int kConcStages = 3;
 // The concurrent form's GEMM: CTA pairs for the wide tiles, which large products
-// take (4608 x 3072 x 12288 136 -> 121 us, 16384 x 1152 x 4608 82 -> 73, 2048 x 1152 x
-// 4608 19.9 -> 19.6), single CTAs for the narrow ones, where a pair's joint start costs
+// take (4608 x 12288 x 3072 136 -> 121 us, 16384 x 4608 x 1152 82 -> 73, 2048 x 4608 x
+// 1152 19.9 -> 19.6), single CTAs for the narrow ones, where a pair's joint start costs
 // more than its shared operands give (256 x 1152 x 1152 10.2 us, as pairs 11.2).
 template <int BNT>
 constexpr int kConcCG = BNT >= 192 ? 2 : 1;
@@ -132,10 +139,13 @@ __global__ void __launch_bounds__(FT, 1)
   __shared__ Barriers bars;
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  constexpr int EW = kSeqEpiWarps<BPACK>;
-  setup<false, BPACK, BNT, 1, 1, EW>(&bars);
+  constexpr int EW = kSeqEpiWarps<BPACK>, CG = kSeqCG<BPACK>;
+  setup<false, BPACK, BNT, 1, 1, EW, MAX_STAGES, 0, CG>(&bars);
   tc_fence_before();
-  __syncthreads();
+  if (CG == 2)
+    cluster_sync();
+  else
+    __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars.tmem_slot;
 
@@ -144,11 +154,14 @@ __global__ void __launch_bounds__(FT, 1)
   __syncthreads();
 
   const Maps maps{&mapA, &mapB, use_tma_store ? &mapY : nullptr};
-  pipeline<T, false, BPACK, BNT, 1, 1, false, EW, MAX_STAGES, F6>(maps, g, smem, &bars, tmem,
-                                                                  ready);
+  pipeline<T, false, BPACK, BNT, 1, 1, false, EW, MAX_STAGES, F6, 0, CG>(maps, g, smem, &bars,
+                                                                         tmem, ready);
   tc_fence_before();
-  __syncthreads();
-  teardown(tmem, Cfg<false, BPACK, BNT, 1, 1, EW>::TMEM);
+  if (CG == 2)
+    cluster_sync();
+  else
+    __syncthreads();
+  teardown<CG>(tmem, SeqCfg<BPACK>::TMEM);
 }
 
 template <typename T, int BNT, bool F6>
@@ -241,8 +254,8 @@ cudaError_t launch_t(const CUtensorMap& mapA, const CUtensorMap& mapB, const CUt
   auto k = fused_linear_kernel<T, BPACK, BNT, F6>;
   cudaError_t e = kernel_setup(reinterpret_cast<const void*>(k), smem, FT, nullptr);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k, grid, FT, smem, st, mapA, mapB, mapY, rq, g, ready, tile_counter,
-                    use_tma_store);
+  return launch_cluster_pdl(k, grid, kSeqCG<BPACK>, FT, smem, st, mapA, mapB, mapY, rq, g, ready,
+                            tile_counter, use_tma_store);
 }
 
 }  // namespace

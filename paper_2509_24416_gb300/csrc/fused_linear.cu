@@ -87,8 +87,8 @@ cudaError_t launch_fused_linear(const RotateQuantArgs& rq_in, const uint8_t* W, 
   if (!bpack && rq_in.K <= kConcStride / 2 && rq_in.K / 32 <= kTeamCompute)
     return launch_concurrent(rq_in, W, w_codes, g, logb, dtype, ready, sms, st);
   const int bn = BN;
-  const size_t gemm_bytes = bpack ? Cfg<false, true, BN, 1, 1, kSeqEpiWarps<true>>::BYTES
-                                  : Cfg<false, false, BN, 1, 1, kSeqEpiWarps<false>>::BYTES;
+  const int cg = bpack ? kSeqCG<true> : kSeqCG<false>;
+  const size_t gemm_bytes = bpack ? SeqCfg<true>::BYTES : SeqCfg<false>::BYTES;
   const size_t limit = 227u * 1024u - 2048u;  // dynamic + static shared memory
   // Rotate-quant phase: as many rows per tile as 512 threads cover and one
   // raw stage holds.
@@ -111,7 +111,7 @@ cudaError_t launch_fused_linear(const RotateQuantArgs& rq_in, const uint8_t* W, 
 
   CUtensorMap mapA, mapB, mapY;
   if (!encode_codes_map(&mapA, rq.Q, f6 ? CLQ_CODES_E2M3 : CLQ_CODES_E4M3, g.M, g.K, BM, 0) ||
-      !encode_codes_map(&mapB, W, w_codes, g.N, g.K, bn, 0))
+      !encode_codes_map(&mapB, W, w_codes, g.N, g.K, bn / cg, 0))
     return cudaErrorInvalidValue;
   const int use_tma_store = (g.N % 8 == 0) ? 1 : 0;
   if (use_tma_store) {
@@ -119,7 +119,7 @@ cudaError_t launch_fused_linear(const RotateQuantArgs& rq_in, const uint8_t* W, 
   } else {
     mapY = mapA;  // unused
   }
-  const int grid = sms;
+  const int grid = sms / cg * cg;
   if (f6)
     return dtype == CLQ_F16
                ? launch_t<__half, false, BN, true>(mapA, mapB, mapY, rq, g, ready, use_tma_store,
