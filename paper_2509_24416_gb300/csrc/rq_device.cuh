@@ -153,6 +153,15 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return r;
 }
 
+// Whether asymmetric codes of a row of span `am` take exact divisions instead of
+// a product with div * rcp_approx(am), div = 2^n - 1: subnormal spans, spans from
+// 2^126 on (bf16 inputs near their top), whose reciprocal is subnormal and flushed
+// to zero, and spans so small that the product div / am is no longer finite (am <
+// div * 2^-128; the bound leaves a factor of four).
+__device__ __forceinline__ bool asym_exact(float am, float div) {
+  return am > 0.f && (am < div * 1.17549435e-38f || am >= 8.50705917e37f);
+}
+
 __device__ __forceinline__ void mbar_inval(uint64_t* bar) {
   asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
@@ -521,10 +530,8 @@ __device__ __forceinline__ void run(const RotateQuantArgs& a, uint8_t* smem,
             constexpr float half = SPLIT ? 128.0f : 8.0f;
             const float2 mg = make_float2(12582912.0f - half, 12582912.0f - half);
             const float2 nlo = make_float2(-row_lo, -row_lo);
-            // exact divisions also where rcp(span) would be subnormal (span
-            // >= 2^126, bf16 inputs near their top), which rcp.approx.ftz
-            // flushes to zero
-            if (am > 0.f && (am < 1.17549435e-38f || am >= 8.50705917e37f)) {
+            // exact divisions for spans that asym_exact names
+            if (asym_exact(am, div)) {
 #pragma unroll
               for (int k = 0; k < 16; ++k) {
                 const float2 d = __fadd2_rn(v[k], nlo);

@@ -372,13 +372,11 @@ __device__ __forceinline__ void wide_quant_store_asym(const RotateQuantArgs& a, 
   }
   // v <- rint((v - min) * (2^n - 1) / span) + 1.5 * 2^23 - 2^(n-1) (the centered
   // code in the low mantissa bits; 8 more for split planes); a constant row gets q
-  // = 0; a subnormal span takes exact divisions.
+  // = 0; spans that asym_exact names take exact divisions.
   constexpr float mgc = CODES == 2 ? kSplitMagic - 128.0f : 12582912.0f - 8.0f;
   const float2 mg = make_float2(mgc, mgc);
   const float2 nlo = make_float2(-row_lo, -row_lo);
-  // exact divisions also where rcp(span) would be subnormal (span >= 2^126,
-  // bf16 inputs near their top), which rcp.approx.ftz flushes to zero
-  if (am > 0.f && (am < 1.17549435e-38f || am >= 8.50705917e37f)) {
+  if (asym_exact(am, div)) {
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
       const float2 d = __fadd2_rn(v[k], nlo);

@@ -112,3 +112,39 @@ def test_wide_equals_general(b, K, M, dtype):
     assert torch.equal(rot, rot_want) and torch.equal(lut[q.long()], want)
     assert clq.device_status() == 0
     assert np.isfinite(s.cpu().numpy()).all()
+
+
+def _small_rows(M, K, b, spans, seed):
+    """bf16 rows whose rotated values span about spans[i % len(spans)]."""
+    g = torch.Generator().manual_seed(seed)
+    x = torch.randn(M, K, generator=g, dtype=torch.float64)
+    s = torch.tensor(spans, dtype=torch.float64)[torch.arange(M) % len(spans)]
+    return (x * (s / (7 * b ** 0.5))[:, None]).to(torch.bfloat16).to(DEV)
+
+
+@pytest.mark.parametrize("b,K", [(32, 1152), (64, 1152), (128, 1152), (256, 1280)])
+def test_asym_small_spans(b, K):
+    """Asymmetric codes of rows whose span is normal but so small that (2^n - 1) /
+    span passes the largest float (spans below 4.4e-38 with 4 bits, 7.5e-37 with 8),
+    and of rows around that range, in both loops."""
+    X = _small_rows(64, K, b, [1.3e-38, 2e-38, 4e-38, 5e-38, 1e-37, 3e-37, 7e-37, 8e-37, 3e-36], b)
+    perm = torch.randperm(K, generator=torch.Generator().manual_seed(K)).to(torch.int32).to(DEV)
+    lut = _lut()
+    for codes, bits in ((clq.CLQ_CODES_INT4_PACKED, 4), (clq.CLQ_CODES_E4M3, 4),
+                        (clq.CLQ_CODES_E4M3_SPLIT, 8)):
+        q, d, lo, rot = clq.rotate_quant_act_asym(X, perm, b, codes=codes, with_rot=True)
+        x64 = rot.double()
+        span = x64.amax(1, keepdim=True) - x64.amin(1, keepdim=True)
+        small = (2 ** bits - 1) * 2.0 ** -128  # below: the reciprocal's product overflows
+        assert bool(((span > 2.0 ** -126) & (span < small)).any())
+        assert bool((span > small).any())
+        got = (_nibbles(q) if codes == clq.CLQ_CODES_INT4_PACKED else
+               lut[q.long()] if codes == clq.CLQ_CODES_E4M3 else _planes(q, K)).double()
+        ratio = (x64 - x64.amin(1, keepdim=True)) / span * (2 ** bits - 1)
+        # a quotient and its product with 2^n - 1: fp32 keeps ratios up to 255 within 1e-4
+        assert bool(((got + 2 ** (bits - 1) - ratio).abs() <= 0.5 + 1e-4).all())
+        assert torch.equal(lo.double(), x64.amin(1))
+        # as above: 2 ulp, or one step of the subnormal grid
+        assert bool(((d.double() * (2 ** bits - 1) - span[:, 0]).abs()
+                     <= 2.5e-7 * span[:, 0] + (2 ** bits - 1) * 2.0 ** -149).all())
+    assert clq.device_status() == 0
