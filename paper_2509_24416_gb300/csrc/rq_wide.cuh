@@ -206,16 +206,16 @@ __device__ __forceinline__ void wide_store_split(const RotateQuantArgs& a, float
   }
 }
 
-// The same for a row with a subnormal scale: values times 2^64 (exact) against
-// `rcp`, the reciprocal of the scale times 2^64.  A call of its own, on a copy of
-// the values: as a branch of the hot path it cost that path 80 bytes of spills.
+// The same for a row with a subnormal scale s: exact divisions, as in rq_device.cuh.
+// A call of its own, on a copy of the values: as a branch of the hot path it cost
+// that path 80 bytes of spills.
 template <int X>
 static __device__ __noinline__ void wide_store_split_tiny(uint8_t* qrow, int K, const float2* t,
-                                                          float rcp, uint32_t flip, int lane) {
+                                                          float s, uint32_t flip, int lane) {
 #pragma unroll 1
   for (int r = 0; r < 64; ++r) {
-    const float v = ((r & 1) ? t[r >> 1].y : t[r >> 1].x) * kTwo64;
-    const float x = fmaf(v, ((flip >> (r >> 2)) & 1u) ? -rcp : rcp, kSplitMagic);
+    const float v = __fdiv_rn((r & 1) ? t[r >> 1].y : t[r >> 1].x, s);
+    const float x = (((flip >> (r >> 2)) & 1u) ? -v : v) + kSplitMagic;
     const float q = x - kSplitMagic;
     const float h16 = 16.f * floorf((q + 8.f) * 0.0625f);
     uint16_t eh, el;
@@ -252,14 +252,15 @@ __device__ __forceinline__ void wide_quant_store(const RotateQuantArgs& a, float
     }
   }
   // v <- rint(v / s) + 1.5 * 2^23 (ties to even), v / s as v * rcp(s); a zero
-  // row gets zero codes; a subnormal s is scaled with v by 2^64 first.
+  // row gets zero codes; a subnormal s takes exact divisions with 8-bit codes, and
+  // is scaled with v by 2^64 first with 4-bit ones.
   if constexpr (CODES == 2) {
     if (s_row > 0.f && s_row < 1.17549435e-38f) {
       float2 t[32];
 #pragma unroll
       for (int k = 0; k < 32; ++k) t[k] = v[k];
-      wide_store_split_tiny<X>(a.Q + static_cast<size_t>(row) * 2 * K + block, K, t,
-                               rcp_approx(s_row * kTwo64), flip, lane);
+      wide_store_split_tiny<X>(a.Q + static_cast<size_t>(row) * 2 * K + block, K, t, s_row, flip,
+                               lane);
       return;
     }
     const float rcp = s_row > 0.f ? rcp_approx(s_row) : 0.f;

@@ -91,12 +91,8 @@ def test_wide_equals_general(b, K, M, dtype):
     v8_want = _planes(q8_want, K)
     for p in (perm, shifted):
         q8, s8 = clq.rotate_quant_act(wide[:, :K], p, b, S8)
-        # rows with a subnormal scale take exact divisions in the general loop and a
-        # scaled reciprocal in this one
-        rows = s8_want >= 1.2e-38
         assert torch.equal(s8, s8_want)
-        assert torch.equal(_planes(q8, K)[rows], v8_want[rows])
-        assert int((_planes(q8, K)[~rows] - v8_want[~rows]).abs().max() if (~rows).any() else 0) <= 1
+        assert torch.equal(_planes(q8, K), v8_want)
     qa, da, la = clq.rotate_quant_act_asym(X, perm, b, codes=S8)
     x64 = rot_want.double()
     lo, span = x64.amin(1, keepdim=True), x64.amax(1, keepdim=True) - x64.amin(1, keepdim=True)
@@ -147,4 +143,23 @@ def test_asym_small_spans(b, K):
         # as above: 2 ulp, or one step of the subnormal grid
         assert bool(((d.double() * (2 ** bits - 1) - span[:, 0]).abs()
                      <= 2.5e-7 * span[:, 0] + (2 ** bits - 1) * 2.0 ** -149).all())
+    assert clq.device_status() == 0
+
+
+@pytest.mark.parametrize("b,K", [(64, 4736), (128, 4736), (256, 1280)])
+def test_split_subnormal_scales(b, K):
+    """8-bit codes of rows with a subnormal scale (|x| up to 127 * 2^-126 = 1.5e-36):
+    the nearest integer to the fp32 quotient by that scale, in the general loop
+    (reached through a clip that never binds) and in the wide one."""
+    M = 300
+    X = _small_rows(M, K, b, [1e-38, 1e-37, 5e-37, 1e-36], K)
+    perm = torch.randperm(K, generator=torch.Generator().manual_seed(b)).to(torch.int32).to(DEV)
+    S8 = clq.CLQ_CODES_E4M3_SPLIT
+    q, s, rot = clq.rotate_quant_act(X, perm, b, S8, with_rot=True)
+    assert bool(((s > 0) & (s < 2.0 ** -126)).all())
+    want = torch.round((rot.double() / s.double()[:, None]).float()).to(torch.int32)
+    assert torch.equal(_planes(q, K), want)
+    clip = torch.full((M,), 3e38, device=DEV)
+    q, s_want = clq.prepare_weights(X, perm, b, clip=clip, codes=S8)
+    assert torch.equal(s, s_want) and torch.equal(_planes(q, K), want)
     assert clq.device_status() == 0
