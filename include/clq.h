@@ -54,11 +54,11 @@
  *    reads the swap vector `perm`, a layer constant.  So that `perm` must not
  *    be written by the kernel enqueued just before the call on the same
  *    stream: the writes of a kernel are guaranteed visible to the next one
- *    only once the latter has waited for it.  Of the calls of this library only
- *    clq_build_permutation_device writes a swap vector on the device
- *    (clq_build_permutation runs on the host); a copy or another call of this
+ *    only once the latter has waited for it.  A copy or another call of this
  *    library enqueued between the writing kernel and the call restores the
- *    usual order.  The weight-preparation calls and clq_clip_search launch
+ *    usual order.  clq_build_permutation_device, the one call of this library
+ *    that writes a swap vector on the device, orders its own writes: any call
+ *    may follow it.  The weight-preparation calls and clq_clip_search launch
  *    without the overlap, so a swap vector computed on the device just before
  *    them is safe.
  *  - The library keeps no per-call state and is safe to call from several

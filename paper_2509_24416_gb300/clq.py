@@ -343,7 +343,8 @@ def build_permutation(scores):
 
 def build_permutation_device(scores, stream=None):
     """Column-swap vector from scores [K] fp32 on the GPU, without a copy to the
-    host -> (perm int32 [K], bad int32 [1], 1 if a score is NaN), on the GPU."""
+    host -> (perm int32 [K], bad int32 [1], 1 if a score is NaN), on the GPU.  Any
+    call may follow it on the stream, those that read perm early too."""
     K = scores.numel()
     scores = scores.contiguous()
     perm = torch.empty(K, dtype=torch.int32, device=scores.device)
@@ -399,7 +400,12 @@ def rotate_quant_act(X, perm, b, codes=CLQ_CODES_INT4_PACKED, Xq=None, s_x=None,
                      with_rot=False, stream=None):
     """X [M, K] -> (Xq uint8, s_x fp32 [M][, x_rot fp32 [M, K]]); Xq is
     [M, K/2] packed (CLQ_CODES_INT4_PACKED), [M, K] E4M3 (CLQ_CODES_E4M3) or,
-    for 8-bit codes, [M, 2K] split planes (CLQ_CODES_E4M3_SPLIT)."""
+    for 8-bit codes, [M, 2K] split planes (CLQ_CODES_E4M3_SPLIT).
+
+    The kernel reads perm while the previous kernel on the stream still runs, here
+    and in rotate_quant_act_asym and a layer's call: perm must not be the output of a
+    kernel (a torch operator, say) enqueued just before, unless a copy or another
+    call of this module lies between them or that call was build_permutation_device."""
     _row_major(X, "X")
     M, K = X.shape
     dev = X.device

@@ -236,11 +236,18 @@ __global__ void __launch_bounds__(kPermThreads) build_permutation_kernel(
   }
 }
 
+// Launched plainly behind the builder, it starts once that has completed and its
+// writes are visible.  Rotate-quant and the fused kernel read the swap vector before
+// their programmatic-launch wait; they can start no earlier than this kernel ends,
+// so a vector built just before them on the stream is the one they read.
+__global__ void order_swap_vector_kernel() {}
+
 }  // namespace
 
 cudaError_t launch_build_permutation(const float* scores, int K, int32_t* perm, int32_t* bad,
                                      cudaStream_t st) {
   build_permutation_kernel<<<1, kPermThreads, 0, st>>>(scores, K, perm, bad);
+  order_swap_vector_kernel<<<1, 32, 0, st>>>();
   return cudaGetLastError();
 }
 

@@ -290,8 +290,8 @@ __device__ __forceinline__ void run(const RotateQuantArgs& a, uint8_t* smem,
   tsync();
   // Past pdl_wait, the previous kernel on the stream has completed (it may
   // still be finishing when this grid starts): X, the tile counter and every
-  // output are touched only after it, the swap vector (a layer constant that
-  // no kernel of this library writes) before it.
+  // output are touched only after it, the swap vector (a layer constant; a kernel
+  // of this library that writes one orders its writes before this grid) before it.
   if (LOADER && tid >= nthr) {
     // ---- loader warp ---------------------------------------------------------
     pdl_wait();

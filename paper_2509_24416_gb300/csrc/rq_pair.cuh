@@ -366,8 +366,8 @@ __global__ void __maxnreg__(pair_max_regs<NR>()) rotate_quant_pair_kernel(Rotate
   // keep the shuffles convergent and never reach a row maximum.
   const unsigned grp = __match_any_sync(0xffffffffu, active ? r : -1);
   const int leader = __ffs(grp) - 1;
-  // X is read only from here on (the swap vector above is a layer constant,
-  // which no kernel of this library writes).
+  // X is read only from here on (the swap vector above is a layer constant; a
+  // kernel of this library that writes one orders its writes before this grid).
   pdl_wait();
   pdl_launch_dependents();
   if (tid == 0)

@@ -82,3 +82,36 @@ def test_convert_every_byte():
     assert torch.equal(clq.convert_codes(there, 1152, P).cpu(), codes)
     assert torch.equal(there, clq.expand_weights(codes.to(DEV)))
     assert clq.device_status() == 0
+
+
+@pytest.mark.parametrize("K,b", [(1152, 128), (12288, 64), (1152, 32)])
+def test_device_permutation_feeds_the_next_call(K, b):
+    """A vector built on the device into a buffer that held another one, and read by
+    the very next call on the stream: each rotate-quant loop and the one-kernel
+    layer give what they give for the finished vector."""
+    g = torch.Generator(device=DEV).manual_seed(K)
+    X = torch.randn(300, K, generator=g, device=DEV).half()
+    W = (0.05 * torch.randn(64, K, generator=g, device=DEV)).half()
+    scores = [torch.rand(K, generator=g, device=DEV) for _ in range(4)]
+    perms = [clq.build_permutation_device(s)[0] for s in scores]
+    layers = [clq.PreparedLinear.from_weight(W, p, b) for p in perms]
+    ws = clq.fused_workspace(300, K, DEV)
+    calls = [lambda p, i, c=c: clq.rotate_quant_act(X, p, b, c)
+             for c in (P, E, clq.CLQ_CODES_E4M3_SPLIT)]
+    calls.append(lambda p, i: clq.rotate_quant_act_asym(X, p, b))
+    calls.append(lambda p, i: (clq.fused_linear(X, p, b, layers[i].We, layers[i].s_w,
+                                                workspace=ws),))
+    torch.cuda.synchronize()
+    want = [[call(perms[i], i) for i in range(4)] for call in calls]
+    torch.cuda.synchronize()
+    perm = perms[3].clone()
+    bad = torch.zeros(1, dtype=torch.int32, device=DEV)
+    st = torch.cuda.current_stream().cuda_stream
+    for j, call in enumerate(calls):
+        for n in range(20):
+            i = n % 4
+            assert clq.clq_build_permutation_device(scores[i].data_ptr(), K, perm.data_ptr(),
+                                                    bad.data_ptr(), st) == 0
+            got = call(perm, i)
+            assert all(torch.equal(a, w) for a, w in zip(got, want[j][i]))
+    assert clq.device_status() == 0
