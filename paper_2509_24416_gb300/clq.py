@@ -14,6 +14,8 @@ A prepared layer's plain call takes one native step (csrc/host_layer.cpp, module
 _clq_host): the same two C calls without the interpreter between them.
 """
 import ctypes
+import functools
+import inspect
 import os
 
 import torch
@@ -288,6 +290,46 @@ def _stream(stream):
     return _raw_stream(torch.cuda.current_device())
 
 
+def _torch_stream(stream):
+    """`stream`, or torch's name for the handle of a stream object of another kind."""
+    if isinstance(stream, torch.cuda.Stream):
+        return stream
+    h = stream.cuda_stream
+    return torch.cuda.ExternalStream(h) if h else torch.cuda.default_stream()
+
+
+def _record(tensors, stream):
+    for t in tensors:
+        if isinstance(t, torch.Tensor) and t.is_cuda:
+            t.record_stream(stream)
+
+
+def _with_stream(stream, fn, args, kw):
+    """fn(*args, **kw) with `stream` current, so that the buffers it allocates come
+    from that stream's pool: a block of the caller's stream could still be in use
+    there, or be handed out again, while kernels on `stream` work on it.  The results
+    are recorded on the caller's stream, which may read and drop them."""
+    here = torch.cuda.current_stream()
+    with torch.cuda.stream(_torch_stream(stream)):
+        out = fn(*args, **kw)
+    _record(out if isinstance(out, tuple) else (out,), here)
+    return out
+
+
+def _on_stream(fn):
+    """A call with a ``stream`` argument other than the current stream runs under
+    _with_stream."""
+    at = list(inspect.signature(fn).parameters).index("stream")
+
+    @functools.wraps(fn)
+    def call(*args, **kw):
+        stream = args[at] if len(args) > at else kw.get("stream")
+        if stream is None or stream.cuda_stream == _stream(None):
+            return fn(*args, **kw)
+        return _with_stream(stream, fn, args, kw)
+    return call
+
+
 def _check(st, where):
     if st != 0:
         raise ClqError(st, where)
@@ -313,6 +355,7 @@ def _row_major(t, name):
 OUTLIER_METRICS = {"absmax": 0, "percentile": 1, "topk_mean": 2, "range": 3, "par": 4}
 
 
+@_on_stream
 def outlier_scores(calib, metric="absmax", stream=None):
     """calib [B, T, K] fp16/bf16 on the GPU -> fp32 scores [K] under `metric`
     (one of OUTLIER_METRICS; "absmax" is the method's, Sec. 3.3)."""
@@ -341,6 +384,7 @@ def build_permutation(scores):
     return perm
 
 
+@_on_stream
 def build_permutation_device(scores, stream=None):
     """Column-swap vector from scores [K] fp32 on the GPU, without a copy to the
     host -> (perm int32 [K], bad int32 [1], 1 if a score is NaN), on the GPU.  Any
@@ -370,6 +414,7 @@ def exec_layout(K):
     return CLQ_CODES_E4M3
 
 
+@_on_stream
 def prepare_weights(W, perm, b, clip=None, with_rot=False, stream=None,
                     codes=CLQ_CODES_INT4_PACKED):
     """W [N, K] -> (Wq uint8 [N, width], s_w fp32 [N][, w_rot fp32 [N, K]]);
@@ -396,6 +441,7 @@ def prepare_weights(W, perm, b, clip=None, with_rot=False, stream=None,
     return (Wq, s_w, rot) if with_rot else (Wq, s_w)
 
 
+@_on_stream
 def rotate_quant_act(X, perm, b, codes=CLQ_CODES_INT4_PACKED, Xq=None, s_x=None,
                      with_rot=False, stream=None):
     """X [M, K] -> (Xq uint8, s_x fp32 [M][, x_rot fp32 [M, K]]); Xq is
@@ -427,6 +473,7 @@ def rotate_quant_act(X, perm, b, codes=CLQ_CODES_INT4_PACKED, Xq=None, s_x=None,
     return (Xq, s_x, rot) if with_rot else (Xq, s_x)
 
 
+@_on_stream
 def rotate_quant_act_asym(X, perm, b, codes=CLQ_CODES_E4M3, Xq=None,
                           delta=None, lo=None, with_rot=False, stream=None):
     """X [M, K] -> (Xq uint8, delta fp32 [M], lo fp32 [M][, x_rot fp32
@@ -459,6 +506,7 @@ def rotate_quant_act_asym(X, perm, b, codes=CLQ_CODES_E4M3, Xq=None,
     return (Xq, delta, lo, rot) if with_rot else (Xq, delta, lo)
 
 
+@_on_stream
 def weight_code_sums(W, K, stream=None):
     """Integer code sums of each row of a weight code array (any layout) ->
     fp32 [N]."""
@@ -469,6 +517,7 @@ def weight_code_sums(W, K, stream=None):
     return wsum
 
 
+@_on_stream
 def expand_weights(Wq, stream=None):
     """Packed codes [N, K/2] -> E4M3 execution layout [N, K] (uint8)."""
     N, Kh = Wq.shape
@@ -492,6 +541,7 @@ def codes_layout(t, K):
                      "[rows, 3K/4] E2M3 or [rows, 2K] split")
 
 
+@_on_stream
 def convert_codes(src, K, dst_codes, dst=None, stream=None):
     """A 4-bit code array in any layout -> the same codes in layout
     `dst_codes` (uint8 [rows, width])."""
@@ -506,6 +556,7 @@ def convert_codes(src, K, dst_codes, dst=None, stream=None):
     return dst
 
 
+@_on_stream
 def w4a4_linear(Xq, s_x, W, s_w, b, K, bias=None, out_dtype=torch.float16,
                 Y=None, with_acc=False, stream=None):
     """Activation codes x weight codes (each packed [rows, K/2] or E4M3
@@ -527,6 +578,7 @@ def w4a4_linear(Xq, s_x, W, s_w, b, K, bias=None, out_dtype=torch.float16,
     return (Y, acc) if with_acc else Y
 
 
+@_on_stream
 def linear(Xq, s_x, W, s_w, b, K, bias=None, out_dtype=torch.float16,
            Y=None, with_acc=False, stream=None):
     """Codes x codes at any bit setting (W4A4, W4A8, W8A8; layouts inferred
@@ -548,6 +600,7 @@ def linear(Xq, s_x, W, s_w, b, K, bias=None, out_dtype=torch.float16,
     return (Y, acc) if with_acc else Y
 
 
+@_on_stream
 def linear_asym(Xq, delta, lo, W, s_w, wsum, b, K, bias=None,
                 out_dtype=torch.float16, Y=None, with_acc=False, stream=None):
     """Asymmetric activation codes (rotate_quant_act_asym) x weight codes
@@ -572,6 +625,7 @@ def linear_asym(Xq, delta, lo, W, s_w, wsum, b, K, bias=None,
 CLIP_GRID = tuple(0.001 * i for i in range(11))  # [beta, gamma] = [0, 0.01]
 
 
+@_on_stream
 def clip_search(W, perm, b, Xcal, Yref, bias=None, grid=CLIP_GRID, stream=None):
     """Per-layer clip search (Sec. 3.4, Eq. 3): W [N, K], Xcal [M, K] (same
     dtype, on the GPU), Yref fp32 [M, N] the full-precision layer output.
@@ -605,6 +659,7 @@ def fused_workspace(M, K, device):
     return torch.empty(max(n, 256), dtype=torch.uint8, device=device)
 
 
+@_on_stream
 def fused_linear(X, perm, b, W, s_w, bias=None, Y=None, workspace=None,
                  stream=None):
     """X [M, K] -> Y [M, N] in X's dtype, rotate-quant and GEMM in one
@@ -734,15 +789,26 @@ class PreparedLinear:
         4-bit, the per-layer clip search (Eq. 3) on the B * T calibration
         tokens against their fp32 product, and finally the prepared layer.
         Returns (layer, info) with info = dict(scores, perm, clip, errors,
-        best)."""
+        best).  With a `stream` all of it runs there, behind the current stream's
+        work and in front of what that enqueues next."""
+        if stream is not None and stream.cuda_stream != _stream(None):
+            here, there = torch.cuda.current_stream(), _torch_stream(stream)
+            there.wait_stream(here)
+            try:
+                with torch.cuda.stream(there):
+                    layer, info = cls.calibrate(W, calib, b, bias=bias, metric=metric,
+                                                clip_grid=clip_grid, a_bits=a_bits,
+                                                w_bits=w_bits)
+            finally:
+                here.wait_stream(there)
+            _record((layer.We, layer.s_w, layer.perm, *info.values()), here)
+            return layer, info
         K = W.shape[1]
-        scores = outlier_scores(calib, metric=metric, stream=stream)
+        scores = outlier_scores(calib, metric=metric)
         if K > 16384 or scores.device != W.device:
             perm, bad = build_permutation(scores).to(W.device), None
         else:  # on the GPU: no copy, no sort on the host, one wait, at the end
-            perm, bad = build_permutation_device(scores, stream=stream)
-            if stream is not None:
-                torch.cuda.current_stream().wait_stream(stream)
+            perm, bad = build_permutation_device(scores)
         clip = errors = best = None
         if clip_grid is not None and w_bits == 4:
             Xcal = calib.reshape(-1, K).contiguous()
@@ -754,7 +820,7 @@ class PreparedLinear:
                 Yref = Yref + bias.double()[None, :]
             Yref = Yref.float().contiguous()
             clip, errors, best = clip_search(W.contiguous(), perm, b, Xcal, Yref, bias,
-                                             grid=clip_grid, stream=stream)
+                                             grid=clip_grid)
         layer = cls.from_weight(W, perm, b, bias=bias, clip=clip, a_bits=a_bits,
                                 w_bits=w_bits)
         if bad is not None and bad.item():  # NaN scores, as build_permutation refuses them
@@ -791,10 +857,11 @@ class PreparedLinear:
         codes / scales of the separate path (Xq [M, K] uint8 for 4-bit, [M, 2K]
         for 8-bit activations; s_x [M] fp32), may be passed in to avoid
         allocations."""
+        if stream is not None and stream.cuda_stream != _stream(None):
+            return _with_stream(stream, self, (X, fused, workspace, None, Y, Xq, s_x), {})
         if not fused and Y is None and Xq is None and s_x is None and type(X) is torch.Tensor:
             r = (_host or load_host()).layer(X, self.perm, self.We, self.s_w, self.bias, self.b,
-                                             self.K, self.act_codes,
-                                             None if stream is None else stream.cuda_stream)
+                                             self.K, self.act_codes)
             if r is not None:
                 if type(r) is int:
                     raise ClqError(r & 255, "clq_rotate_quant_act" if r < 256 else

@@ -39,12 +39,13 @@ int64_t codes_width(int64_t codes, int64_t K) {
   }
 }
 
-// layer(X, perm, We, s_w, bias | None, b, K, a_codes, stream | None) -> Y [M, N];
-// None: not the plain case; an int: status | 256 * (0 rotate-quant, 1 product).
+// layer(X, perm, We, s_w, bias | None, b, K, a_codes) -> Y [M, N] on the current
+// stream, whose pool the buffers come from; None: not the plain case; an int:
+// status | 256 * (0 rotate-quant, 1 product).
 PyObject* layer(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
   HANDLE_TH_ERRORS
-  if (nargs != 9) {
-    PyErr_SetString(PyExc_TypeError, "layer() takes 9 arguments");
+  if (nargs != 8) {
+    PyErr_SetString(PyExc_TypeError, "layer() takes 8 arguments");
     return nullptr;
   }
   for (int i = 0; i < 4; ++i)
@@ -73,13 +74,7 @@ PyObject* layer(PyObject*, PyObject* const* args, Py_ssize_t nargs) {
       (w_codes == CLQ_CODES_E4M3_SPLIT && a_codes != CLQ_CODES_E4M3_SPLIT) ||
       M > INT32_MAX || N > INT32_MAX || ld > INT32_MAX || b < 0 || b > INT32_MAX)
     Py_RETURN_NONE;
-  void* stream;
-  if (args[8] == Py_None) {
-    stream = c10::cuda::getCurrentCUDAStream().stream();
-  } else {
-    stream = PyLong_AsVoidPtr(args[8]);
-    if (stream == nullptr && PyErr_Occurred()) return nullptr;
-  }
+  void* stream = c10::cuda::getCurrentCUDAStream().stream();
   // Activation codes and, behind them, their fp32 scales: one buffer.
   const int64_t codes_bytes = (M * width + 15) / 16 * 16;
   at::Tensor codes = at::empty({codes_bytes + 4 * M}, X.options().dtype(at::kByte));

@@ -69,3 +69,50 @@ def test_empty_and_refused_calls():
         layer(torch.randn(4, 1152, device=DEV).half())
     assert e.value.status == 2 and "clq_rotate_quant_act" in str(e.value)
     assert clq.device_status() == 0
+
+
+def _pool(t):
+    """Handle of the stream whose allocator pool holds t."""
+    at = t.data_ptr()
+    for seg in torch.cuda.memory_snapshot():
+        if seg["address"] <= at < seg["address"] + seg["total_size"]:
+            return seg["stream"]
+    return None
+
+
+@pytest.mark.parametrize("kw", [{}, dict(a_bits=8), dict(w_codes=P)])
+def test_explicit_stream_owns_its_buffers(kw):
+    """layer(X, stream=side) without buffers, behind a busy side stream and in front
+    of work on the current stream that takes blocks of the same sizes."""
+    layer = _layer(N=1152, **kw)
+    X = torch.randn(2048, 1152, device=DEV).half()
+    want = layer(X)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    for fused in (False, True)[:1 if kw.get("a_bits") else 2]:
+        got = []
+        for _ in range(4):
+            with torch.cuda.stream(side):
+                torch.cuda._sleep(2000000)  # about a millisecond
+            got.append(layer(X, fused=fused, stream=side))
+            assert _pool(got[-1]) == side.cuda_stream
+            for n in (want.numel() * 2, X.numel(), 2 * X.numel(), 4 * 2048):
+                torch.full((n,), 0x7F, dtype=torch.uint8, device=DEV)
+        torch.cuda.synchronize()
+        assert all(torch.equal(y, want) for y in got)
+
+
+def test_calibrate_on_a_stream():
+    g = torch.Generator(device=DEV).manual_seed(3)
+    W = torch.randn(96, 1152, generator=g, device=DEV).half()
+    calib = torch.randn(4, 64, 1152, generator=g, device=DEV).half()
+    side = torch.cuda.Stream()
+    for grid in (None, (0.0, 0.01)):
+        want, iw = clq.PreparedLinear.calibrate(W, calib, 64, clip_grid=grid)
+        torch.cuda._sleep(2000000)  # the inputs may still be in the making
+        c2 = calib * 1
+        got, ig = clq.PreparedLinear.calibrate(W * 1, c2, 64, clip_grid=grid, stream=side)
+        assert torch.equal(got.We, want.We) and torch.equal(got.s_w, want.s_w)
+        assert torch.equal(ig["perm"], iw["perm"]) and torch.equal(ig["scores"], iw["scores"])
+        assert _pool(got.We) == side.cuda_stream
+    assert clq.device_status() == 0
