@@ -11,12 +11,15 @@ Two layers:
 Every step of the computation runs in the CUDA kernels of libclq.so; there is
 no CPU or PyTorch fallback.  If the library is missing, the first call raises.
 A prepared layer's plain call takes one native step (csrc/host_layer.cpp, module
-_clq_host): the same two C calls without the interpreter between them.
+_clq_host): the same two C calls without the interpreter between them.  Where that
+module is missing or does not import, the call takes them from Python, with a
+warning.
 """
 import ctypes
 import functools
 import inspect
 import os
+import warnings
 
 import torch
 
@@ -112,16 +115,28 @@ def load():
     return _lib
 
 
-_host = None
+_host = None  # the module, or False where it cannot be imported
 
 
 def load_host():
     """The native form of a layer's call (built in-tree beside libclq.so)."""
     global _host
-    if _host is None:
+    if not _host:
         load()
         from . import _clq_host
         _host = _clq_host
+    return _host
+
+
+def _find_host():
+    """load_host(), or False, with one warning, where the module cannot be imported."""
+    global _host
+    if _host is None:
+        try:
+            load_host()
+        except ImportError as e:
+            _host = False
+            warnings.warn("layer calls go through Python (about 20 us of host time more): %s" % e)
     return _host
 
 
@@ -859,9 +874,10 @@ class PreparedLinear:
         allocations."""
         if stream is not None and stream.cuda_stream != _stream(None):
             return _with_stream(stream, self, (X, fused, workspace, None, Y, Xq, s_x), {})
-        if not fused and Y is None and Xq is None and s_x is None and type(X) is torch.Tensor:
-            r = (_host or load_host()).layer(X, self.perm, self.We, self.s_w, self.bias, self.b,
-                                             self.K, self.act_codes)
+        if (not fused and Y is None and Xq is None and s_x is None and type(X) is torch.Tensor
+                and (_host or _find_host())):
+            r = _host.layer(X, self.perm, self.We, self.s_w, self.bias, self.b, self.K,
+                            self.act_codes)
             if r is not None:
                 if type(r) is int:
                     raise ClqError(r & 255, "clq_rotate_quant_act" if r < 256 else

@@ -297,3 +297,31 @@ def test_binding_rejects_mis_sized_output_buffers():
     s = torch.empty(8, dtype=torch.float32)
     with pytest.raises(ValueError):
         clq.linear(Xq, s[:4], W, s, 32, 64, Y=torch.empty((4, 7), dtype=torch.float16))
+
+
+def test_layer_call_without_the_host_module(monkeypatch):
+    """libclq.so alone serves a layer's call: where the native module does not import,
+    the two C calls come from Python, with one warning."""
+    import sys
+    import warnings
+
+    import paper_2509_24416_gb300 as package
+    monkeypatch.setattr(clq, "_host", None)
+    monkeypatch.delattr(package, "_clq_host", raising=False)
+    monkeypatch.setitem(sys.modules, package.__name__ + "._clq_host", None)
+    monkeypatch.setattr(clq, "_raw_stream", lambda device: 0)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    calls = []
+    for name in ("clq_rotate_quant_act", "clq_w4a4_linear"):
+        monkeypatch.setattr(clq, name, lambda *a, name=name: calls.append(name) or 0)
+    layer = clq.PreparedLinear(None, torch.zeros(8), torch.arange(128, dtype=torch.int32), 32,
+                               We=torch.zeros(8, 128, dtype=torch.uint8))
+    with warnings.catch_warnings(record=True) as seen:
+        warnings.simplefilter("always")
+        for _ in range(2):
+            Y = layer(torch.zeros(4, 128, dtype=torch.float16))
+            assert Y.shape == (4, 8) and Y.dtype == torch.float16
+    assert len(seen) == 1 and "layer calls go through Python" in str(seen[0].message)
+    assert calls == ["clq_rotate_quant_act", "clq_w4a4_linear"] * 2
+    with pytest.raises(ImportError):
+        clq.load_host()
