@@ -9,6 +9,7 @@ import glob
 import os
 import shutil
 import subprocess
+import sys
 import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -49,9 +50,20 @@ def _compile(src, obj, extra):
 
 
 def _host_object():
-    """Object of the host module, named by the torch it was compiled against."""
+    """Object of the host module, named by the torch and the Python it was compiled
+    against."""
     import torch
-    return os.path.join(BUILD, "host_layer-%s.o" % torch.__version__)
+    return os.path.join(BUILD, "host_layer-%s-%s.o" % (torch.__version__,
+                                                       sys.implementation.cache_tag))
+
+
+def _linked_host():
+    """Name of the object that _clq_host.so was linked from, or None."""
+    try:
+        with open(os.path.join(BUILD, "host_layer.linked")) as f:
+            return f.read()
+    except OSError:
+        return None
 
 
 def _compile_host(obj):
@@ -78,6 +90,8 @@ def _link_host(obj):
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("link failed:\n%s%s" % (r.stdout, r.stderr))
+    with open(os.path.join(BUILD, "host_layer.linked"), "w") as f:
+        f.write(os.path.basename(obj))
 
 
 def build(verbose=False, force=False, extra_flags=()):
@@ -111,7 +125,8 @@ def build(verbose=False, force=False, extra_flags=()):
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("link failed:\n%s%s" % (r.stdout, r.stderr))
-    if host_new or not os.path.exists(HOST) or os.path.getmtime(HOST) < os.path.getmtime(host_obj):
+    if (host_new or not os.path.exists(HOST) or _linked_host() != os.path.basename(host_obj)
+            or os.path.getmtime(HOST) < os.path.getmtime(host_obj)):
         _link_host(host_obj)
     return LIB
 

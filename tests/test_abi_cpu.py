@@ -325,3 +325,41 @@ def test_layer_call_without_the_host_module(monkeypatch):
     assert calls == ["clq_rotate_quant_act", "clq_w4a4_linear"] * 2
     with pytest.raises(ImportError):
         clq.load_host()
+
+
+def test_host_module_follows_torch_and_python(monkeypatch, tmp_path):
+    """The host module is linked again whenever the torch or the Python in use is not
+    the one it was linked for, also on the way back to an object already there."""
+    import sys
+    import types
+    src = tmp_path / "csrc"
+    src.mkdir()
+    (tmp_path / "include").mkdir()
+    for f in (src / "host_layer.cpp", tmp_path / "include" / "clq.h", tmp_path / "libclq.so"):
+        f.write_text("")
+    for name, path in dict(ROOT=tmp_path, CSRC=src, BUILD=tmp_path / "_build",
+                           LIB=tmp_path / "libclq.so", HOST=tmp_path / "_clq_host.so",
+                           HOST_SRC=src / "host_layer.cpp").items():
+        monkeypatch.setattr(build, name, str(path))
+    compiled, linked = [], []
+
+    def run(cmd, **kw):  # g++ -c .. -o object, or g++ -shared -o module object ..
+        out = cmd[cmd.index("-o") + 1]
+        (linked if "-shared" in cmd else compiled).append(out)
+        if "-shared" in cmd:
+            linked[-1] = os.path.basename(cmd[cmd.index("-o") + 2])
+        open(out, "w").write("x")
+        return types.SimpleNamespace(returncode=0, stdout="", stderr="")
+
+    monkeypatch.setattr(build.subprocess, "run", run)
+    want = []
+    for version, tag in (("2.9", "a"), ("2.9", "a"), ("2.11", "a"), ("2.9", "a"), ("2.9", "b"),
+                         ("2.9", "a"), ("2.9", "a")):
+        monkeypatch.setattr(torch, "__version__", version)
+        monkeypatch.setattr(sys.implementation, "cache_tag", tag)
+        now = "host_layer-%s-%s.o" % (version, tag)
+        if not want or want[-1] != now:
+            want.append(now)
+        build.build()
+        assert linked == want
+    assert len(compiled) == 3
