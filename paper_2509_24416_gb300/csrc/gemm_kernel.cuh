@@ -89,13 +89,15 @@ cudaError_t launch_gemm_t(const MapSet& m, const GemmArgs& g, int use_tma_store,
                             use_tma_store);
 }
 
-// CTA pairs for operands in an execution layout, single CTAs for packed ones
-// (whose unpack warps work on a whole tile's operands).
+// CTA pairs for operands in an execution layout, single CTAs for packed ones (whose
+// unpack warps work on a whole tile's operands) and for the widest tile where
+// single_cta_wins.
 #define CLQ_GO(...) return launch_gemm_t<OutT, __VA_ARGS__>(m, g, use_tma_store, grid, st)
 
 template <typename OutT>
 cudaError_t launch_gemm_e4m3(const MapSet& m, const GemmArgs& g, int, int, TileShape t,
                              int use_tma_store, int grid, cudaStream_t st) {
+  if (t.cg == 1) CLQ_GO(false, false, 256, 1);
   switch (t.bn) {
     case 64: CLQ_GO(false, false, 64, 2);
     case 128: CLQ_GO(false, false, 128, 2);
@@ -107,6 +109,7 @@ cudaError_t launch_gemm_e4m3(const MapSet& m, const GemmArgs& g, int, int, TileS
 template <typename OutT>
 cudaError_t launch_gemm_e2m3(const MapSet& m, const GemmArgs& g, int, int, TileShape t,
                              int use_tma_store, int grid, cudaStream_t st) {
+  if (t.cg == 1) CLQ_GO(false, false, 256, 1, 1, 1, false, true);
   switch (t.bn) {
     case 64: CLQ_GO(false, false, 64, 2, 1, 1, false, true);
     case 128: CLQ_GO(false, false, 128, 2, 1, 1, false, true);
@@ -119,6 +122,17 @@ template <typename OutT>
 cudaError_t launch_gemm_bits(const MapSet& m, const GemmArgs& g, int x_codes, int w_codes,
                              TileShape t, int use_tma_store, int grid, cudaStream_t st) {
   const bool a8 = x_codes == CLQ_CODES_E4M3_SPLIT, w8 = w_codes == CLQ_CODES_E4M3_SPLIT;
+  if (t.cg == 1) {
+    if (g.lo != nullptr) {
+      if (a8 && w8 && g.K > kSep2MaxK) CLQ_GO(false, false, 128, 1, 2, 2, true, false, 3);
+      if (a8 && w8) CLQ_GO(false, false, 128, 1, 2, 2, true, false, 2);
+      if (a8) CLQ_GO(false, false, 256, 1, 2, 1, true);
+      CLQ_GO(false, false, 256, 1, 1, 1, true);
+    }
+    if (w8 && g.K > kSep2MaxK) CLQ_GO(false, false, 128, 1, 2, 2, false, false, 3);
+    if (w8) CLQ_GO(false, false, 128, 1, 2, 2, false, false, 2);
+    CLQ_GO(false, false, 256, 1, 2, 1);
+  }
   if (g.lo != nullptr) {  // asymmetric activations
     if (a8 && w8 && g.K > kSep2MaxK) CLQ_GO(false, false, 128, 2, 2, 2, true, false, 3);
     if (a8 && w8) CLQ_GO(false, false, 128, 2, 2, 2, true, false, 2);

@@ -369,6 +369,27 @@ bool encode_codes_map(CUtensorMap* map, const uint8_t* base, int codes, int rows
                                CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
+namespace {
+
+// Clocks a K step of a pair's tile of bn columns takes with 1, 2 or 4 products of
+// code planes (a single CTA: 740 and 1200 at 256 columns, 1300 at 128 with four),
+// fitted to 434 measured products.
+double pair_step(int products, int bn) {
+  if (products == 4) return bn == 64 ? 766 : 1146;
+  if (products == 2) return bn == 64 ? 520 : bn == 128 ? 630 : 1128;
+  return bn == 64 ? 300 : bn == 128 ? 390 : bn == 192 ? 458 : 587;
+}
+
+// Clocks of a product by the model of gemm_tile_n.
+double tiles_cost(int M, int N, int K, int rows, int units, int bn, double step, int epi) {
+  const long tiles = static_cast<long>((M + rows - 1) / rows) * ((N + bn - 1) / bn);
+  const long rounds = (tiles + units - 1) / units;
+  const double drain = epi * bn / 64.0;
+  return rounds * std::max((K + BK - 1) / BK * step, drain + 500) + drain;
+}
+
+}  // namespace
+
 // Tile width of execution-layout operands, `units` CTAs or CTA pairs walking tiles
 // of `rows` rows.  The units go ceil(tiles / units) rounds; a tile takes its K
 // steps (clocks a step of a pair's main loop, measured alone: 587 / 458 / 390 for
@@ -384,23 +405,41 @@ bool encode_codes_map(CUtensorMap* map, const uint8_t* base, int codes, int rows
 // the best of them on 15 such shapes in each layout).  `narrow`: 64 and 128 are
 // built for these operands; `mid`: 192 is.
 int gemm_tile_n(int M, int N, int K, int rows, int units, bool mid, bool narrow, int epi) {
-  const long mt = (M + rows - 1) / rows;
-  const double nk = (K + BK - 1) / BK;
   const int width[4] = {256, 192, 128, 64};
-  const double step[4] = {587, 458, 390, 300};
   int best = BN;
   double best_cost = 1e300;
   for (int i = 0; i < 4; ++i) {
     if ((width[i] == 192 && !mid) || (width[i] < 192 && !narrow)) continue;
-    const long rounds = (mt * ((N + width[i] - 1) / width[i]) + units - 1) / units;
-    const double drain = epi * width[i] / 64.0;
-    const double cost = rounds * std::max(nk * step[i], drain + 500) + drain;
+    const double cost = tiles_cost(M, N, K, rows, units, width[i], pair_step(1, width[i]), epi);
     if (cost < best_cost) {
       best_cost = cost;
       best = width[i];
     }
   }
   return best;
+}
+
+// Whether the widest tile of a single CTA beats the pairs' tile of `pair_bn` columns;
+// `products`: products of code planes a K step (1, 2 for W4A8, 4 for W8A8).  Pairs win
+// large products, but with twice the rows a tile their rounds come out coarser: 3129
+// rows x 12288 -> 3072, W4A8, takes three rounds of 256 x 256 (161 us) or two of 128 x
+// 256 (123); 375 x 5376 -> 4960, W8A8, 50.5 us or 30.0; 300 x 3072 -> 12288 14.8 or
+// 12.4, W4A8 24.7 or 17.7.  And activation codes of less than 128 KB starve pairs more
+// than single CTAs (3072 -> 12288: 12.6 us with 16 to 32 rows, 9.7 with 48; as single
+// CTAs 11.5 to 11.9 and 11.4), by about 10 clocks a step for each pair that reads
+// them: 4 x 896 -> 11479, W4A8, 14.0 or 9.1; 1 x 8512 -> 10112 36.7 or 26.1.  The
+// margin of 10 % covers what the model leaves open: of 678 products of 1 .. 16384
+// rows, at random, the rule moves 26, all of them to a tile at least as fast.
+bool single_cta_wins(int M, int N, int K, int products, int pair_bn, int sms, int epi) {
+  const double codes = static_cast<double>(M) * K * (products == 1 ? 1 : 2);
+  const int readers = std::min((N + pair_bn - 1) / pair_bn, sms / 2);
+  const double starved = codes < 131072 ? 10.0 * readers : 0.0;
+  const double pair = tiles_cost(M, N, K, 2 * BM, sms / 2, pair_bn,
+                                 pair_step(products, pair_bn) + starved, epi);
+  const double one =
+      products == 4 ? tiles_cost(M, N, K, BM, sms, 128, 1300, epi)
+                    : tiles_cost(M, N, K, BM, sms, BN, products == 2 ? 1200 : 740, epi);
+  return 1.1 * one < pair;
 }
 
 cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, int w_codes,
@@ -427,6 +466,8 @@ cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, i
   }
   else if (!apack && !bpack && !(split && g.lo != nullptr))
     t.bn = gemm_tile_n(g.M, g.N, g.K, t.cg * BM, sms / t.cg, !split && g.lo == nullptr, true);
+  if (t.cg == 2 && single_cta_wins(g.M, g.N, g.K, w8a8 ? 4 : split ? 2 : 1, t.bn, sms))
+    t = {1, w8a8 ? 128 : BN};
   MapSet m;
   const int brows = t.bn / t.cg;  // each CTA of a pair loads half of B
   if (!encode_codes_map(&m.A, Xq, x_codes, g.M, g.K, BM, 0) ||

@@ -168,3 +168,53 @@ def test_fused_wide_tiles_match_separate(M, N, K, w_codes):
     for _ in range(2):
         assert torch.equal(layer(X, fused=True, workspace=ws), want)
     assert clq.device_status() == 0
+
+
+@pytest.mark.parametrize("setting", sorted(SETTINGS) + ["asym", "asym_w4a8", "asym_w8a8"])
+@pytest.mark.parametrize("M,N,K", [(300, 10241, 4608), (300, 10008, 8064), (12, 11013, 2304)])
+def test_single_cta_tiles(setting, M, N, K):
+    """Shapes whose rounds of 256-row tiles would come out so coarse, or whose rows are
+    so few, that the launcher takes single CTAs, on both sides of the K up to which
+    W8A8 has two accumulators: products exact, outputs as in test_tile_widths."""
+    a_bits, w_bits, w_codes = SETTINGS.get(setting.replace("asym_", ""), (4, 4, None))
+    asym = setting.startswith("asym")
+    g = torch.Generator(device=DEV).manual_seed(M + N)
+    b = 128
+    X = torch.randn(M, K, generator=g, device=DEV).bfloat16()
+    W = (0.05 * torch.randn(N, K, generator=g, device=DEV)).bfloat16()
+    bias = torch.randn(N, generator=g, device=DEV).bfloat16()
+    perm = torch.randperm(K, generator=g, device=DEV).to(torch.int32)
+    layer = clq.PreparedLinear.from_weight(W, perm, b, bias=bias, a_bits=a_bits, w_bits=w_bits,
+                                           w_codes=w_codes)
+    kw = dict(out_dtype=torch.bfloat16, with_acc=True,
+              Y=torch.full((M + 1, N), 7.0, dtype=torch.bfloat16, device=DEV)[:M])
+    guard = kw["Y"].as_strided((N,), (1,), M * N)  # the row behind Y
+    if asym:
+        codes = clq.CLQ_CODES_E4M3 if a_bits == 4 else clq.CLQ_CODES_E4M3_SPLIT
+        Xq, s_x, lo = clq.rotate_quant_act_asym(X, perm, b, codes)
+        wsum = clq.weight_code_sums(layer.We, K)
+        Y, acc = clq.linear_asym(Xq, s_x, lo, layer.We, layer.s_w, wsum, b, K, bias, **kw)
+    else:
+        Xq, s_x = clq.rotate_quant_act(X, perm, b, layer.act_codes)
+        Y, acc = clq.linear(Xq, s_x, layer.We, layer.s_w, b, K, bias, **kw)
+    assert clq.device_status() == 0 and bool((guard == 7.0).all())
+
+    def codes64(t):
+        if w_codes is not None:
+            t = clq.convert_codes(t, K, clq.CLQ_CODES_E4M3)
+        return torch.from_numpy(_values(t, clq.codes_layout(t, K), K)).to(DEV).double()
+
+    qx, qw = codes64(Xq), codes64(layer.We)
+    want = qx @ qw.t()
+    assert torch.equal(acc.double(), want)
+    scale = layer.s_w.double()[None, :] / b
+    y64 = want * s_x.double()[:, None] * scale
+    size = y64.abs()
+    if asym:
+        zp = (lo.double() + (8 if a_bits == 4 else 128) * s_x.double())[:, None] \
+            * qw.sum(1)[None, :] * scale
+        y64, size = y64 + zp, size + zp.abs()
+    y64 = y64 + bias.double()[None, :]
+    size = size + bias.double().abs()[None, :]
+    # half an ulp of bf16, three fp32 roundings of the terms
+    assert bool(((Y.double() - y64).abs() <= 2.0 ** -8 * y64.abs() + 1e-6 * size + 2.0 ** -126).all())
