@@ -71,7 +71,8 @@ int gemm_tile_n(int M, int N, int K, int rows, int units, bool mid, bool narrow,
                 int epi = 1000);
 // Whether single CTAs (256 columns, 128 with four products of code planes) take the
 // product in less time than pairs with pair_bn columns.
-bool single_cta_wins(int M, int N, int K, int products, int pair_bn, int sms, int epi = 1000);
+bool single_cta_wins(int M, int N, int K, int products, int pair_bn, int sms,
+                     bool few_starve = true);
 cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, int w_codes,
                              const GemmArgs& g, int out_dtype, cudaStream_t st);
 

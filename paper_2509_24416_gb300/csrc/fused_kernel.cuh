@@ -49,13 +49,12 @@ constexpr int FT = 512;
 // Epilogue warps of the sequential form (unpack warps leave room for four).
 template <bool BPACK>
 constexpr int kSeqEpiWarps = BPACK ? 4 : 8;
-// Its GEMM: CTA pairs unless the weights are packed (4608 x 3072 x 12288 190 -> 169 us,
-// 16384 x 1152 x 9344 392 -> 362, 64 x 1152 x 12288 44.6 -> 40.5; 3129 x 4544 x 11008,
-// where pairs need a round more, 157.5 -> 161).
-template <bool BPACK>
-constexpr int kSeqCG = BPACK ? 1 : 2;
-template <bool BPACK>
-using SeqCfg = Cfg<false, BPACK, BN, 1, 1, kSeqEpiWarps<BPACK>, MAX_STAGES, 0, kSeqCG<BPACK>>;
+// Its GEMM: CTA pairs (CG 2; 4608 x 3072 x 12288 190 -> 169 us, 16384 x 1152 x 9344
+// 392 -> 362, 64 x 1152 x 12288 44.6 -> 40.5), single CTAs for packed weights and where
+// pairs need a round more (single_cta_wins: 3129 x 12288 -> 3072 137.6 us before pairs,
+// 142.5 on them, 130.2 on single CTAs; 300 x 9344 -> 10240 50.0, 60.6, 46.2).
+template <bool BPACK, int CG>
+using SeqCfg = Cfg<false, BPACK, BN, 1, 1, kSeqEpiWarps<BPACK>, MAX_STAGES, 0, CG>;
 
 // Adds the rows [row0, row0 + rows) to the ready counters of the 128-token
 // blocks they fall in (a tile of rows may straddle two blocks); RELEASE: each
@@ -129,7 +128,7 @@ struct Conc {
 
 // F6 (both forms): the workspace codes and the weights are E2M3, loaded by
 // 16U6 tensor maps (gemm::pipeline's F6 mode).
-template <typename T, bool BPACK, int BNT, bool F6>
+template <typename T, bool BPACK, int BNT, bool F6, int CG>
 __global__ void __launch_bounds__(FT, 1)
     fused_linear_kernel(const __grid_constant__ CUtensorMap mapA,
                         const __grid_constant__ CUtensorMap mapB,
@@ -139,7 +138,7 @@ __global__ void __launch_bounds__(FT, 1)
   __shared__ Barriers bars;
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  constexpr int EW = kSeqEpiWarps<BPACK>, CG = kSeqCG<BPACK>;
+  constexpr int EW = kSeqEpiWarps<BPACK>;
   setup<false, BPACK, BNT, 1, 1, EW, MAX_STAGES, 0, CG>(&bars);
   tc_fence_before();
   if (CG == 2)
@@ -161,7 +160,7 @@ __global__ void __launch_bounds__(FT, 1)
     cluster_sync();
   else
     __syncthreads();
-  teardown<CG>(tmem, SeqCfg<BPACK>::TMEM);
+  teardown<CG>(tmem, SeqCfg<BPACK, CG>::TMEM);
 }
 
 template <typename T, int BNT, bool F6>
@@ -246,16 +245,16 @@ cudaError_t launch_conc(const CUtensorMap& mapA, const CUtensorMap& mapB, const 
 #undef CLQ_GO
 }
 
-template <typename T, bool BPACK, int BNT, bool F6>
+template <typename T, bool BPACK, int BNT, bool F6, int CG>
 cudaError_t launch_t(const CUtensorMap& mapA, const CUtensorMap& mapB, const CUtensorMap& mapY,
                      const RotateQuantArgs& rq, const GemmArgs& g, uint32_t* ready,
                      int use_tma_store, size_t smem, int grid, cudaStream_t st) {
   uint32_t* tile_counter = ready + (g.M + BM - 1) / BM;
-  auto k = fused_linear_kernel<T, BPACK, BNT, F6>;
+  auto k = fused_linear_kernel<T, BPACK, BNT, F6, CG>;
   cudaError_t e = kernel_setup(reinterpret_cast<const void*>(k), smem, FT, nullptr);
   if (e != cudaSuccess) return e;
-  return launch_cluster_pdl(k, grid, kSeqCG<BPACK>, FT, smem, st, mapA, mapB, mapY, rq, g, ready,
-                            tile_counter, use_tma_store);
+  return launch_cluster_pdl(k, grid, CG, FT, smem, st, mapA, mapB, mapY, rq, g, ready, tile_counter,
+                            use_tma_store);
 }
 
 }  // namespace

@@ -87,8 +87,10 @@ cudaError_t launch_fused_linear(const RotateQuantArgs& rq_in, const uint8_t* W, 
   if (!bpack && rq_in.K <= kConcStride / 2 && rq_in.K / 32 <= kTeamCompute)
     return launch_concurrent(rq_in, W, w_codes, g, logb, dtype, ready, sms, st);
   const int bn = BN;
-  const int cg = bpack ? kSeqCG<true> : kSeqCG<false>;
-  const size_t gemm_bytes = bpack ? SeqCfg<true>::BYTES : SeqCfg<false>::BYTES;
+  const int cg = bpack || single_cta_wins(g.M, g.N, g.K, 1, bn, sms, false) ? 1 : 2;
+  const size_t gemm_bytes = bpack     ? SeqCfg<true, 1>::BYTES
+                            : cg == 1 ? SeqCfg<false, 1>::BYTES
+                                      : SeqCfg<false, 2>::BYTES;
   const size_t limit = 227u * 1024u - 2048u;  // dynamic + static shared memory
   // Rotate-quant phase: as many rows per tile as 512 threads cover and one
   // raw stage holds.
@@ -120,21 +122,18 @@ cudaError_t launch_fused_linear(const RotateQuantArgs& rq_in, const uint8_t* W, 
     mapY = mapA;  // unused
   }
   const int grid = sms / cg * cg;
-  if (f6)
-    return dtype == CLQ_F16
-               ? launch_t<__half, false, BN, true>(mapA, mapB, mapY, rq, g, ready, use_tma_store,
-                                                   smem, grid, st)
-               : launch_t<__nv_bfloat16, false, BN, true>(mapA, mapB, mapY, rq, g, ready,
-                                                          use_tma_store, smem, grid, st);
-  if (dtype == CLQ_F16)
-    return bpack ? launch_t<__half, true, BN, false>(mapA, mapB, mapY, rq, g, ready,
-                                                     use_tma_store, smem, grid, st)
-                 : launch_t<__half, false, BN, false>(mapA, mapB, mapY, rq, g, ready,
-                                                      use_tma_store, smem, grid, st);
-  return bpack ? launch_t<__nv_bfloat16, true, BN, false>(mapA, mapB, mapY, rq, g, ready,
+#define CLQ_GO(BPACK, F6, CG)                                                                    \
+  return dtype == CLQ_F16                                                                        \
+             ? launch_t<__half, BPACK, BN, F6, CG>(mapA, mapB, mapY, rq, g, ready,               \
+                                                   use_tma_store, smem, grid, st)                \
+             : launch_t<__nv_bfloat16, BPACK, BN, F6, CG>(mapA, mapB, mapY, rq, g, ready,        \
                                                           use_tma_store, smem, grid, st)
-               : launch_t<__nv_bfloat16, false, BN, false>(mapA, mapB, mapY, rq, g, ready,
-                                                           use_tma_store, smem, grid, st);
+  if (bpack) CLQ_GO(true, false, 1);
+  if (f6 && cg == 1) CLQ_GO(false, true, 1);
+  if (f6) CLQ_GO(false, true, 2);
+  if (cg == 1) CLQ_GO(false, false, 1);
+  CLQ_GO(false, false, 2);
+#undef CLQ_GO
 }
 
 }  // namespace clq

@@ -427,13 +427,15 @@ int gemm_tile_n(int M, int N, int K, int rows, int units, bool mid, bool narrow,
 // 12.4, W4A8 24.7 or 17.7.  And activation codes of less than 128 KB starve pairs more
 // than single CTAs (3072 -> 12288: 12.6 us with 16 to 32 rows, 9.7 with 48; as single
 // CTAs 11.5 to 11.9 and 11.4), by about 10 clocks a step for each pair that reads
-// them: 4 x 896 -> 11479, W4A8, 14.0 or 9.1; 1 x 8512 -> 10112 36.7 or 26.1.  The
+// them: 4 x 896 -> 11479, W4A8, 14.0 or 9.1; 1 x 8512 -> 10112 36.7 or 26.1
+// (`few_starve`; not in the fused kernel: 2 x 10816 -> 11616 47.7, single 62.5).  The
 // margin of 10 % covers what the model leaves open: of 678 products of 1 .. 16384
 // rows, at random, the rule moves 26, all of them to a tile at least as fast.
-bool single_cta_wins(int M, int N, int K, int products, int pair_bn, int sms, int epi) {
+bool single_cta_wins(int M, int N, int K, int products, int pair_bn, int sms, bool few_starve) {
   const double codes = static_cast<double>(M) * K * (products == 1 ? 1 : 2);
   const int readers = std::min((N + pair_bn - 1) / pair_bn, sms / 2);
-  const double starved = codes < 131072 ? 10.0 * readers : 0.0;
+  const double starved = few_starve && codes < 131072 ? 10.0 * readers : 0.0;
+  const int epi = 1000;
   const double pair = tiles_cost(M, N, K, 2 * BM, sms / 2, pair_bn,
                                  pair_step(products, pair_bn) + starved, epi);
   const double one =

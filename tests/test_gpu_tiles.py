@@ -151,11 +151,13 @@ def test_w8a8_accumulators_at_their_limit(K, M, N):
 
 @pytest.mark.parametrize("w_codes", [None, clq.CLQ_CODES_E2M3])
 @pytest.mark.parametrize("M,N,K", [(1900, 4600, 1152), (2200, 4701, 640), (9700, 1152, 1152),
-                                   (8322, 1160, 1152), (700, 1400, 9344)])
+                                   (8322, 1160, 1152), (700, 1400, 9344), (300, 10241, 9344),
+                                   (300, 10240, 9344)])
 def test_fused_wide_tiles_match_separate(M, N, K, w_codes):
     """The one-kernel layer on the wide tiles that CTA pairs share, with a last pair
     whose second CTA has no rows or few and ragged columns: the separate kernels'
-    output bit for bit, twice over one workspace."""
+    output bit for bit, twice over one workspace.  At K = 9344 the sequential form, on
+    pairs and, where those take a round more, on single CTAs."""
     g = torch.Generator(device=DEV).manual_seed(N)
     b = 64
     X = torch.randn(M, K, generator=g, device=DEV).half()
