@@ -167,10 +167,19 @@ cudaError_t launch_rotate_quant(const RotateQuantArgs& a, int dtype, int logb,
   // 128 / 256: 16384 rows x 1152 / 1280 16.3 / 18.4 against 18.8 / 25.8, 4608 x
   // 12288 42 / 42 against 53 / 62 (E2M3 42 / 49 against 57 / 64; asymmetric 46 / 46
   // against 67 / 72; 8-bit codes at b = 64 / 128 against the general one:
-  // 8192 x 1152 10.4 / 11.7 against 14.4 / 15.3, 4608 x 12288 49 / 55 against 79 / 83);
-  // at 256 rows, a launch of about 2.7 us, it is up to 0.2 us slower.
+  // 8192 x 1152 10.4 / 11.7 against 14.4 / 15.3, 4608 x 12288 49 / 55 against 79 / 83).
+  // Few elements of short rows go to the general loop: with a tile or two a CTA a
+  // launch is one chain of latencies, which 64 positions a thread make longer (b =
+  // 128, general against wide, 256 x 1152: E4M3 2.50 us against 2.57, 8-bit 2.63
+  // against 2.75, asymmetric 2.69 against 2.96, 8-bit asymmetric 2.82 against 3.33;
+  // 640 x 1152 3.10 / 3.22 / 3.26 / 3.47 against 2.84 / 3.08 / 3.27 / 3.56; 64 x 4608
+  // 2.43 / 2.63 / 2.60 / 2.86 against 2.24 / 2.44 / 2.53 / 2.87; b = 64, 8-bit
+  // asymmetric, 256 x 1152 2.75 against 2.86).
   const bool hot = a.clip == nullptr && a.e4m3 != 0;  // not packed, not clipped
-  if (hot && logb >= 6) {  // b divides K, so K % 64 == 0
+  const bool a8 = a.e4m3 == 2, asym = a.lo != nullptr;
+  const long few = logb >= 7 ? ((a8 || asym) ? 4096 : 2048) : (a8 && asym) ? 2048 : 0;
+  const bool chain = a.K <= 4096 && static_cast<long>(a.M) * a.K <= few * sms;
+  if (hot && logb >= 6 && !chain) {  // b divides K, so K % 64 == 0
     int stage = 0;
     rotate_quant_wide_config(a.M, a.K, sms, &args.rows_per_tile, &threads, &smem, &stage);
     const bool e2 = a.e4m3 == 3;
@@ -184,7 +193,7 @@ cudaError_t launch_rotate_quant(const RotateQuantArgs& a, int dtype, int logb,
     return e2 ? launch_rotate_quant_wide_bf16_e2m3(args, logb, stage, threads, smem, sms, st)
               : launch_rotate_quant_wide_bf16_e4m3(args, logb, stage, threads, smem, sms, st);
   }
-  if (hot && a.lo == nullptr && a.e4m3 != 2 && logb == 5) {
+  if (hot && !asym && !a8 && logb == 5) {
     int half = 0;
     rotate_quant_pair_config(a.M, a.K, sms, &args.rows_per_tile, &threads, &smem, &half);
     const bool e2 = a.e4m3 == 3;

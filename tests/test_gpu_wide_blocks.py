@@ -163,3 +163,12 @@ def test_split_subnormal_scales(b, K):
     q, s_want = clq.prepare_weights(X, perm, b, clip=clip, codes=S8)
     assert torch.equal(s, s_want) and torch.equal(_planes(q, K), want)
     assert clq.device_status() == 0
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+@pytest.mark.parametrize("b,K,M", [(64, 1152, 700), (128, 128, 5000), (128, 1152, 700),
+                                   (256, 256, 2500), (256, 1280, 700)])
+def test_wide_equals_general_many_rows(b, K, M, dtype):
+    """Short rows, which the wide loop takes from some 600 thousand elements on in every
+    layout (fewer go to the general loop)."""
+    test_wide_equals_general(b, K, M, dtype)
