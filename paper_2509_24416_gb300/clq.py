@@ -16,8 +16,6 @@ module is missing or does not import, the call takes them from Python, with a
 warning.
 """
 import ctypes
-import functools
-import inspect
 import os
 import warnings
 
@@ -319,30 +317,20 @@ def _record(tensors, stream):
             t.record_stream(stream)
 
 
-def _with_stream(stream, fn, args, kw):
-    """fn(*args, **kw) with `stream` current, so that the buffers it allocates come
-    from that stream's pool: a block of the caller's stream could still be in use
-    there, or be handed out again, while kernels on `stream` work on it.  The results
-    are recorded on the caller's stream, which may read and drop them."""
+def _elsewhere(stream):
+    return stream.cuda_stream != _stream(None)
+
+
+def _with_stream(stream, fn, *args):
+    """fn(*args) with `stream` current, so that the buffers it allocates come from that
+    stream's pool: a block of the caller's stream could still be in use there, or be
+    handed out again, while kernels on `stream` work on it.  The results are recorded
+    on the caller's stream, which may read and drop them."""
     here = torch.cuda.current_stream()
     with torch.cuda.stream(_torch_stream(stream)):
-        out = fn(*args, **kw)
+        out = fn(*args)
     _record(out if isinstance(out, tuple) else (out,), here)
     return out
-
-
-def _on_stream(fn):
-    """A call with a ``stream`` argument other than the current stream runs under
-    _with_stream."""
-    at = list(inspect.signature(fn).parameters).index("stream")
-
-    @functools.wraps(fn)
-    def call(*args, **kw):
-        stream = args[at] if len(args) > at else kw.get("stream")
-        if stream is None or stream.cuda_stream == _stream(None):
-            return fn(*args, **kw)
-        return _with_stream(stream, fn, args, kw)
-    return call
 
 
 def _check(st, where):
@@ -370,10 +358,11 @@ def _row_major(t, name):
 OUTLIER_METRICS = {"absmax": 0, "percentile": 1, "topk_mean": 2, "range": 3, "par": 4}
 
 
-@_on_stream
 def outlier_scores(calib, metric="absmax", stream=None):
     """calib [B, T, K] fp16/bf16 on the GPU -> fp32 scores [K] under `metric`
     (one of OUTLIER_METRICS; "absmax" is the method's, Sec. 3.3)."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, outlier_scores, calib, metric)
     calib = calib.contiguous()
     B, T, K = calib.shape
     scores = torch.empty(K, dtype=torch.float32, device=calib.device)
@@ -399,11 +388,12 @@ def build_permutation(scores):
     return perm
 
 
-@_on_stream
 def build_permutation_device(scores, stream=None):
     """Column-swap vector from scores [K] fp32 on the GPU, without a copy to the
     host -> (perm int32 [K], bad int32 [1], 1 if a score is NaN), on the GPU.  Any
     call may follow it on the stream, those that read perm early too."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, build_permutation_device, scores)
     K = scores.numel()
     scores = scores.contiguous()
     perm = torch.empty(K, dtype=torch.int32, device=scores.device)
@@ -429,12 +419,14 @@ def exec_layout(K):
     return CLQ_CODES_E4M3
 
 
-@_on_stream
 def prepare_weights(W, perm, b, clip=None, with_rot=False, stream=None,
                     codes=CLQ_CODES_INT4_PACKED):
     """W [N, K] -> (Wq uint8 [N, width], s_w fp32 [N][, w_rot fp32 [N, K]]);
     4-bit codes packed ([N, K/2], the default) or E4M3 ([N, K]), or 8-bit
     codes as split planes ([N, 2K], CLQ_CODES_E4M3_SPLIT)."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, prepare_weights, W, perm, b, clip, with_rot, None,
+                            codes)
     _row_major(W, "W")
     N, K = W.shape
     dev = W.device
@@ -456,7 +448,6 @@ def prepare_weights(W, perm, b, clip=None, with_rot=False, stream=None,
     return (Wq, s_w, rot) if with_rot else (Wq, s_w)
 
 
-@_on_stream
 def rotate_quant_act(X, perm, b, codes=CLQ_CODES_INT4_PACKED, Xq=None, s_x=None,
                      with_rot=False, stream=None):
     """X [M, K] -> (Xq uint8, s_x fp32 [M][, x_rot fp32 [M, K]]); Xq is
@@ -467,6 +458,8 @@ def rotate_quant_act(X, perm, b, codes=CLQ_CODES_INT4_PACKED, Xq=None, s_x=None,
     and in rotate_quant_act_asym and a layer's call: perm must not be the output of a
     kernel (a torch operator, say) enqueued just before, unless a copy or another
     call of this module lies between them or that call was build_permutation_device."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, rotate_quant_act, X, perm, b, codes, Xq, s_x, with_rot)
     _row_major(X, "X")
     M, K = X.shape
     dev = X.device
@@ -488,13 +481,15 @@ def rotate_quant_act(X, perm, b, codes=CLQ_CODES_INT4_PACKED, Xq=None, s_x=None,
     return (Xq, s_x, rot) if with_rot else (Xq, s_x)
 
 
-@_on_stream
 def rotate_quant_act_asym(X, perm, b, codes=CLQ_CODES_E4M3, Xq=None,
                           delta=None, lo=None, with_rot=False, stream=None):
     """X [M, K] -> (Xq uint8, delta fp32 [M], lo fp32 [M][, x_rot fp32
     [M, K]]): asymmetric codes (Eq. 1, dynamic min / max) stored centered,
     4-bit in CLQ_CODES_E4M3 / CLQ_CODES_INT4_PACKED, 8-bit in
     CLQ_CODES_E4M3_SPLIT."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, rotate_quant_act_asym, X, perm, b, codes, Xq, delta,
+                            lo, with_rot)
     _row_major(X, "X")
     M, K = X.shape
     dev = X.device
@@ -521,10 +516,11 @@ def rotate_quant_act_asym(X, perm, b, codes=CLQ_CODES_E4M3, Xq=None,
     return (Xq, delta, lo, rot) if with_rot else (Xq, delta, lo)
 
 
-@_on_stream
 def weight_code_sums(W, K, stream=None):
     """Integer code sums of each row of a weight code array (any layout) ->
     fp32 [N]."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, weight_code_sums, W, K)
     N = W.shape[0]
     wsum = torch.empty(N, dtype=torch.float32, device=W.device)
     _check(clq_weight_code_sums(_ptr(W), codes_layout(W, K), N, K, _ptr(wsum),
@@ -532,9 +528,10 @@ def weight_code_sums(W, K, stream=None):
     return wsum
 
 
-@_on_stream
 def expand_weights(Wq, stream=None):
     """Packed codes [N, K/2] -> E4M3 execution layout [N, K] (uint8)."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, expand_weights, Wq)
     N, Kh = Wq.shape
     We = torch.empty((N, 2 * Kh), dtype=torch.uint8, device=Wq.device)
     _check(clq_expand_weights(_ptr(Wq), N, 2 * Kh, _ptr(We), _stream(stream)),
@@ -556,10 +553,11 @@ def codes_layout(t, K):
                      "[rows, 3K/4] E2M3 or [rows, 2K] split")
 
 
-@_on_stream
 def convert_codes(src, K, dst_codes, dst=None, stream=None):
     """A 4-bit code array in any layout -> the same codes in layout
     `dst_codes` (uint8 [rows, width])."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, convert_codes, src, K, dst_codes, dst)
     rows = src.shape[0]
     width = codes_width(dst_codes, K)
     if dst is None:
@@ -571,11 +569,13 @@ def convert_codes(src, K, dst_codes, dst=None, stream=None):
     return dst
 
 
-@_on_stream
 def w4a4_linear(Xq, s_x, W, s_w, b, K, bias=None, out_dtype=torch.float16,
                 Y=None, with_acc=False, stream=None):
     """Activation codes x weight codes (each packed [rows, K/2] or E4M3
     [rows, K]) -> Y [M, N] (out_dtype)[, acc int32 [M, N]]."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, w4a4_linear, Xq, s_x, W, s_w, b, K, bias, out_dtype,
+                            Y, with_acc)
     M = Xq.shape[0]
     N = W.shape[0]
     if Y is None:
@@ -593,11 +593,13 @@ def w4a4_linear(Xq, s_x, W, s_w, b, K, bias=None, out_dtype=torch.float16,
     return (Y, acc) if with_acc else Y
 
 
-@_on_stream
 def linear(Xq, s_x, W, s_w, b, K, bias=None, out_dtype=torch.float16,
            Y=None, with_acc=False, stream=None):
     """Codes x codes at any bit setting (W4A4, W4A8, W8A8; layouts inferred
     from the widths) -> Y [M, N] (out_dtype)[, acc int32 [M, N]]."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, linear, Xq, s_x, W, s_w, b, K, bias, out_dtype, Y,
+                            with_acc)
     M = Xq.shape[0]
     N = W.shape[0]
     if Y is None:
@@ -615,11 +617,13 @@ def linear(Xq, s_x, W, s_w, b, K, bias=None, out_dtype=torch.float16,
     return (Y, acc) if with_acc else Y
 
 
-@_on_stream
 def linear_asym(Xq, delta, lo, W, s_w, wsum, b, K, bias=None,
                 out_dtype=torch.float16, Y=None, with_acc=False, stream=None):
     """Asymmetric activation codes (rotate_quant_act_asym) x weight codes
     with the zero-point epilogue -> Y [M, N][, acc int32 [M, N]]."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, linear_asym, Xq, delta, lo, W, s_w, wsum, b, K, bias,
+                            out_dtype, Y, with_acc)
     M = Xq.shape[0]
     N = W.shape[0]
     if Y is None:
@@ -640,12 +644,13 @@ def linear_asym(Xq, delta, lo, W, s_w, wsum, b, K, bias=None,
 CLIP_GRID = tuple(0.001 * i for i in range(11))  # [beta, gamma] = [0, 0.01]
 
 
-@_on_stream
 def clip_search(W, perm, b, Xcal, Yref, bias=None, grid=CLIP_GRID, stream=None):
     """Per-layer clip search (Sec. 3.4, Eq. 3): W [N, K], Xcal [M, K] (same
     dtype, on the GPU), Yref fp32 [M, N] the full-precision layer output.
     Returns (clip fp32 [N] of the best percentile, errors fp64 [G] (host),
     best index).  Synchronizes the stream."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, clip_search, W, perm, b, Xcal, Yref, bias, grid)
     _row_major(W, "W")
     _row_major(Xcal, "Xcal")
     N, K = W.shape
@@ -674,11 +679,12 @@ def fused_workspace(M, K, device):
     return torch.empty(max(n, 256), dtype=torch.uint8, device=device)
 
 
-@_on_stream
 def fused_linear(X, perm, b, W, s_w, bias=None, Y=None, workspace=None,
                  stream=None):
     """X [M, K] -> Y [M, N] in X's dtype, rotate-quant and GEMM in one
     kernel.  W is packed [N, K/2], E4M3 [N, K] or E2M3 [N, 3K/4]."""
+    if stream is not None and _elsewhere(stream):
+        return _with_stream(stream, fused_linear, X, perm, b, W, s_w, bias, Y, workspace)
     _row_major(X, "X")
     M, K = X.shape
     N = W.shape[0]
@@ -806,7 +812,7 @@ class PreparedLinear:
         Returns (layer, info) with info = dict(scores, perm, clip, errors,
         best).  With a `stream` all of it runs there, behind the current stream's
         work and in front of what that enqueues next."""
-        if stream is not None and stream.cuda_stream != _stream(None):
+        if stream is not None and _elsewhere(stream):
             here, there = torch.cuda.current_stream(), _torch_stream(stream)
             there.wait_stream(here)
             try:
@@ -872,8 +878,8 @@ class PreparedLinear:
         codes / scales of the separate path (Xq [M, K] uint8 for 4-bit, [M, 2K]
         for 8-bit activations; s_x [M] fp32), may be passed in to avoid
         allocations."""
-        if stream is not None and stream.cuda_stream != _stream(None):
-            return _with_stream(stream, self, (X, fused, workspace, None, Y, Xq, s_x), {})
+        if stream is not None and _elsewhere(stream):
+            return _with_stream(stream, self, X, fused, workspace, None, Y, Xq, s_x)
         if (not fused and Y is None and Xq is None and s_x is None and type(X) is torch.Tensor
                 and (_host or _find_host())):
             r = _host.layer(X, self.perm, self.We, self.s_w, self.bias, self.b, self.K,
