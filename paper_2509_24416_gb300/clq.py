@@ -931,6 +931,13 @@ class HostPipeline:
         self.s_in = torch.cuda.Stream(device=dev)
         self.s_comp = torch.cuda.Stream(device=dev)
         self.s_out = torch.cuda.Stream(device=dev)
+        # The buffers are the current stream's: its earlier work on their blocks comes
+        # first, and the blocks go back to it only behind the three streams' work.
+        here = torch.cuda.current_stream(dev)
+        for s, used in ((self.s_in, self.xd), (self.s_out, self.yd),
+                        (self.s_comp, self.xd + self.yd + self.xq + self.sx + self.ws)):
+            s.wait_stream(here)
+            _record(used, s)
         n = len(layers)
         self.in_done = [torch.cuda.Event() for _ in range(n)]
         self.comp_done = [torch.cuda.Event() for _ in range(n)]

@@ -65,6 +65,25 @@ def _layer():
     return clq.PreparedLinear(None, SW, PERM, b, We=WE)
 
 
+def test_host_pipeline_buffers(fake, monkeypatch):
+    made, recorded = [], []
+    monkeypatch.setattr(torch.cuda, "Event", lambda *a, **k: None)
+    monkeypatch.setattr(torch.cuda, "Stream", lambda device: made.append(
+        FakeStream(20 + len(made), fake.log)) or made[-1])
+    monkeypatch.setattr(clq, "_record", lambda ts, s: recorded.extend(
+        (t.data_ptr(), s.cuda_stream) for t in ts if t is not None), raising=False)
+    p = clq.HostPipeline([(_layer(), M, K, N)], torch.float16, "cpu", fused=True)
+    # behind the current stream's work on the blocks the buffers are made of
+    last = max(i for i, e in enumerate(fake.log) if e[0] == "empty")
+    assert {("wait", s.cuda_stream, HERE) for s in made} <= set(fake.log[last + 1:])
+    assert len(made) == 3
+    # and the blocks go back only behind the streams that use them
+    want = [(t, s) for t in p.xd for s in (p.s_in, p.s_comp)]
+    want += [(t, s) for t in p.yd for s in (p.s_comp, p.s_out)]
+    want += [(t, p.s_comp) for t in p.xq + p.sx + p.ws]
+    assert {(t.data_ptr(), s.cuda_stream) for t, s in want} <= set(recorded)
+
+
 CALLS = {
     "outlier_scores": lambda s: clq.outlier_scores(X[None], stream=s),
     "outlier_scores_range": lambda s: clq.outlier_scores(X[None], "range", s),
