@@ -60,10 +60,6 @@ struct GemmArgs {
   float zp_shift;
 };
 
-// A = activation codes, B = weight codes, each in layout CLQ_CODES_INT4_PACKED
-// ([rows][K/2]), CLQ_CODES_E4M3 ([rows][K]) or, for 8-bit codes,
-// CLQ_CODES_E4M3_SPLIT ([rows][2][K]; A split with B E4M3 or split); TMA maps
-// are built here.
 // Output-channel tile width (256, 192, 128 or 64) of the product of
 // execution-layout operands, tiles of `rows` rows dealt to `units` CTAs or pairs;
 // mid: 192 is built for them, narrow: 128 and 64 are.
@@ -73,6 +69,10 @@ int gemm_tile_n(int M, int N, int K, int rows, int units, bool mid, bool narrow,
 // product in less time than pairs with pair_bn columns.
 bool single_cta_wins(int M, int N, int K, int products, int pair_bn, int sms,
                      bool few_starve = true);
+// A = activation codes, B = weight codes, each in layout CLQ_CODES_INT4_PACKED
+// ([rows][K/2]), CLQ_CODES_E4M3 ([rows][K]), CLQ_CODES_E2M3 ([rows][3K/4], both or
+// neither) or, for 8-bit codes, CLQ_CODES_E4M3_SPLIT ([rows][2][K]; A split with B
+// E4M3 or split); TMA maps are built here.
 cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, int w_codes,
                              const GemmArgs& g, int out_dtype, cudaStream_t st);
 

@@ -107,7 +107,7 @@ constexpr int kRqStages = 4;
 constexpr int kTeamFirst = (WARP_MMA + 1) * 32;  // 192
 constexpr int kTeamThreads = FT - kTeamFirst;     // 320
 constexpr int kTeamCompute = kTeamThreads - 32;   // 288
-constexpr uint32_t kTeamBarrier = 2;  // 0: CTA, 1: GEMM epilogue, 2-3: team
+constexpr uint32_t kTeamBarrier = 2;  // 0: CTA, 2-3: team
 constexpr int kConcStride = 18 * 1024;
 constexpr int kConcStages = 3;
 // The concurrent form's GEMM: CTA pairs for the wide tiles, which large products

@@ -13,13 +13,10 @@ constexpr int BN = 256;           // rows of B (output channels) per tile (wides
 constexpr int BK = 128;           // codes per K step = one 128-byte swizzle row
 constexpr int BKP = BK / 2;       // packed bytes per row per K step
 constexpr int A_U = BM * BK;      // 16 KB unpacked A stage
-constexpr int B_U = BN * BK;      // 32 KB unpacked B stage
 constexpr int A_P = BM * BKP;     // 8 KB packed A stage
-constexpr int B_P = BN * BKP;     // 16 KB packed B stage
 constexpr int EPI_COLS = 32;      // output columns per epilogue store
 constexpr int EPI_ROWS = 32;      // rows per store: one warp's TMEM lanes
 constexpr int EPI_BYTES = EPI_ROWS * EPI_COLS * 2;  // 2 KB staging buffer, one a warp
-constexpr int TMEM_COLS = 512;    // two 128 x 256 fp32 accumulators
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t c) {
   uint32_t d;

@@ -68,7 +68,7 @@ constexpr int WARP_UNPACK0 = 6;
 constexpr int MIN_THREADS = (WARP_UNPACK0 + NUM_UNPACK / 32) * 32;  // 448
 constexpr int MAX_STAGES = 8;
 
-// Tile BM x BNT (BNT = 256, or 192 for E4M3 operands where N splits better).
+// Tile BM x BNT a CTA (BNT 256, 192, 128 or 64; gemm_tile_n picks it).
 // PA / PB: E4M3 planes per operand, 1 for 4-bit codes, 2 for 8-bit codes
 // split as q = 16 h + l (plane 0 holds 16 h, plane 1 holds l; both E4M3
 // values, so the MMAs of the two planes add up to q in one accumulator).

@@ -70,10 +70,10 @@ cudaError_t launch_b(const RotateQuantArgs& a, int threads, size_t smem, int sms
 }
 
 // Paired-row kernel (rq_pair.cuh): a.rows_per_tile = rows of one half.
-template <typename T, int LOGB, int CODES, int HALF, bool ROT>
+template <typename T, int CODES, int HALF, bool ROT>
 cudaError_t launch_pair_geom(const RotateQuantArgs& a, int threads, size_t smem, int sms,
                              cudaStream_t st) {
-  auto kern = rotate_quant_pair_kernel<T, LOGB, CODES, HALF, kPairStages, ROT>;
+  auto kern = rotate_quant_pair_kernel<T, CODES, HALF, kPairStages, ROT>;
   int per_sm = 0;
   cudaError_t e = kernel_setup(reinterpret_cast<const void*>(kern), smem, threads, &per_sm);
   if (e != cudaSuccess) return e;
@@ -89,8 +89,8 @@ template <typename T, int CODES, bool ROT>
 cudaError_t launch_pair_h(const RotateQuantArgs& a, int half, int threads, size_t smem, int sms,
                           cudaStream_t st) {
   return half == kPairHalfSmall
-             ? launch_pair_geom<T, 5, CODES, kPairHalfSmall, ROT>(a, threads, smem, sms, st)
-             : launch_pair_geom<T, 5, CODES, kPairHalfLarge, ROT>(a, threads, smem, sms, st);
+             ? launch_pair_geom<T, CODES, kPairHalfSmall, ROT>(a, threads, smem, sms, st)
+             : launch_pair_geom<T, CODES, kPairHalfLarge, ROT>(a, threads, smem, sms, st);
 }
 
 template <typename T, int CODES>

@@ -1,5 +1,5 @@
 // Paired-row rotate-quantize: the hot-path variant of the tile loop in
-// rq_device.cuh, for symmetric 4-bit codes (launched at b = 32, no clip):
+// rq_device.cuh, for symmetric 4-bit codes at b = 32 (no clip):
 // the OBS transform of arxiv 2509.24416 Sec. 3.3 (column gather by the swap
 // vector, block Sylvester Hadamard H_b) followed by per-token symmetric
 // quantization with a dynamic fp32 scale (Sec. 3.1, Eq. 1 with l = -r).
@@ -23,10 +23,9 @@
 //     perm[32 seg + (k ^ m)] (m: the XOR order of rq_device.cuh, which only
 //     flips signs that the store restores) with the first butterfly stage on
 //     the way in;
-//  2. the remaining stages (in registers up to stride 16, across lanes above),
-//     |x| maxima, warp reductions, shared atomicMax per row;
-//  3. one CTA barrier, then scales, codes and 16-byte (E4M3, packed) or
-//     8-byte (E2M3) stores for both rows.
+//  2. the remaining stages, |x| maxima, warp reductions, shared atomicMax per row;
+//  3. one CTA barrier, then scales, codes and 16-byte (E4M3) or 8-byte (E2M3)
+//     stores for both rows.
 #pragma once
 
 #include "rq_device.cuh"
@@ -87,39 +86,19 @@ __device__ __forceinline__ float seg_absmax(const float2 (&v)[16]) {
   return max3(max3(a, b, c), m[9], m[10]);
 }
 
-// Butterfly stages of one row's segment: strides 2 .. min(b, 32) / 2 in
-// registers (v[k] holds positions 2k, 2k + 1, stride 1 already done), then
-// strides 32 .. b / 2 across lanes.
-template <int LOGB>
-__device__ __forceinline__ void seg_butterflies(float2 (&v)[16], int lane) {
+// Butterfly stages of one row's segment, strides 2 .. 16 (v[k] holds positions
+// 2k, 2k + 1, stride 1 already done).
+__device__ __forceinline__ void seg_butterflies(float2 (&v)[16]) {
   const float2 neg1 = make_float2(-1.f, -1.f);
 #pragma unroll
-  for (int hp = 1; hp < 16; hp <<= 1) {
-    if (2 * hp < (1 << LOGB)) {
+  for (int hp = 1; hp < 16; hp <<= 1)
 #pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        if ((k & hp) == 0) {
-          const float2 x0 = v[k], x1 = v[k + hp];
-          v[k] = __fadd2_rn(x0, x1);
-          v[k + hp] = __ffma2_rn(x1, neg1, x0);
-        }
+    for (int k = 0; k < 16; ++k)
+      if ((k & hp) == 0) {
+        const float2 x0 = v[k], x1 = v[k + hp];
+        v[k] = __fadd2_rn(x0, x1);
+        v[k + hp] = __ffma2_rn(x1, neg1, x0);
       }
-    }
-  }
-#pragma unroll
-  for (int hl = 1; hl < 8; hl <<= 1) {
-    if (LOGB > 5 && hl < (1 << (LOGB > 5 ? LOGB - 5 : 0))) {
-      const float sg = (lane & hl) ? -1.f : 1.f;
-      const float2 sg2 = make_float2(sg, sg);
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        float2 p;
-        p.x = __shfl_xor_sync(0xffffffffu, v[k].x, hl);
-        p.y = __shfl_xor_sync(0xffffffffu, v[k].y, hl);
-        v[k] = __ffma2_rn(v[k], sg2, p);  // lower lane: x + p, upper lane: p - x
-      }
-    }
-  }
 }
 
 // Scale, codes and stores of one row's segment; `am` is the row's |x| maximum.
@@ -177,7 +156,7 @@ __device__ __forceinline__ void seg_quant_store(const RotateQuantArgs& a, float2
     uint4* qrow = reinterpret_cast<uint4*>(a.Q + static_cast<size_t>(row) * K + seg * 32);
     qrow[0] = make_uint4(w[0], w[1], w[2], w[3]);
     qrow[1] = make_uint4(w[4], w[5], w[6], w[7]);
-  } else if constexpr (CODES == 3) {
+  } else {
     // E2M3, 16 codes in 12 bytes (the packing of rq_device.cuh)
     uint32_t g[8];
 #pragma unroll
@@ -200,20 +179,6 @@ __device__ __forceinline__ void seg_quant_store(const RotateQuantArgs& a, float2
     qrow[0] = make_uint2(g[0] | (g[1] << 24), (g[1] >> 8) | (g[2] << 16));
     qrow[1] = make_uint2((g[2] >> 16) | (g[3] << 8), g[4] | (g[5] << 24));
     qrow[2] = make_uint2((g[5] >> 8) | (g[6] << 16), (g[6] >> 16) | (g[7] << 8));
-  } else {
-    // packed nibbles: the low four bits of v are the code's two's complement
-    // (no XOR order on this path: flip_words is 0)
-    uint32_t by[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k)
-      by[k] = (__float_as_uint(v[k].x) & 0xFu) | ((__float_as_uint(v[k].y) << 4) & 0xF0u);
-    uint32_t w[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      w[q] = prmt_b32(prmt_b32(by[4 * q], by[4 * q + 1], 0x0040u),
-                      prmt_b32(by[4 * q + 2], by[4 * q + 3], 0x0040u), 0x5410u);
-    *reinterpret_cast<uint4*>(a.Q + static_cast<size_t>(row) * (K >> 1) + seg * 16) =
-        make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
@@ -283,12 +248,12 @@ constexpr int pair_max_regs() {
   return NR == 2 ? kPairMaxRegs : 96;
 }
 
-template <typename T, int LOGB, int CODES, int HALF, int STAGES, bool ROT, int NR = 2>
+template <typename T, int CODES, int HALF, int STAGES, bool ROT, int NR = 2>
 __global__ void __maxnreg__(pair_max_regs<NR>()) rotate_quant_pair_kernel(RotateQuantArgs a) {
   extern __shared__ __align__(16) uint8_t smem[];
   constexpr int STRIDE = NR * HALF;
   static_assert(NR == 1 || NR == 2, "one or two rows a thread");
-  static_assert(LOGB >= 4 && LOGB <= 8, "paired loop: 16 <= b <= 256");
+  static_assert(CODES == 1 || CODES == 3, "paired loop: E4M3 or E2M3 codes");
   const int K = a.K;
   const int segs = K >> 5;
   const int RH = a.rows_per_tile;
@@ -323,12 +288,9 @@ __global__ void __maxnreg__(pair_max_regs<NR>()) rotate_quant_pair_kernel(Rotate
   const int r = active ? tid / segs : 0;
   const int seg = active ? tid - r * segs : 0;
   // XOR order of the gather (see rq_device.cuh): m a multiple of 8 that
-  // differs between neighbouring lane groups; not for packed codes, whose
-  // sign restore would cost a negation per code.
-  const bool xor_order = CODES != 0 && (reinterpret_cast<uintptr_t>(a.perm) & 15u) == 0;
-  const int xm = xor_order ? ((8 * (lane >> (LOGB > 5 ? LOGB - 5 : 0))) &
-                              ((1 << (LOGB < 5 ? LOGB : 5)) - 8))
-                           : 0;
+  // differs between neighbouring lanes.
+  const bool xor_order = (reinterpret_cast<uintptr_t>(a.perm) & 15u) == 0;
+  const int xm = xor_order ? ((8 * lane) & 24) : 0;
   uint32_t flip_words = 0;
 #pragma unroll
   for (int q = 0; q < 8; ++q)
@@ -414,8 +376,8 @@ __global__ void __maxnreg__(pair_max_regs<NR>()) rotate_quant_pair_kernel(Rotate
         }
       }
       // ---- 2. remaining stages, row maxima -----------------------------------
-      seg_butterflies<LOGB>(va, lane);
-      if constexpr (NR == 2) seg_butterflies<LOGB>(vb, lane);
+      seg_butterflies(va);
+      if constexpr (NR == 2) seg_butterflies(vb);
       const unsigned ka = __reduce_max_sync(grp, __float_as_uint(seg_absmax(va)));
       unsigned kb = 0;
       if constexpr (NR == 2) kb = __reduce_max_sync(grp, __float_as_uint(seg_absmax(vb)));
