@@ -129,40 +129,57 @@ __device__ __forceinline__ int staged_chunk(int r, int q) {
   return r * 64 + ((q ^ ((r >> 1) & 3)) << 4);
 }
 
+__device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
+}
+
 // A staged block (rows row0 .. row0 + 31, columns col0 .. col0 + 31) straight to
 // Y when N % 8 != 0 rules the tensor store out: half a warp takes consecutive
 // column pairs of one row, four-byte aligned whatever N's parity (in a row that
 // starts at an odd element, pairs 1-2, 3-4, .., and the last lane takes columns
-// 31 and 0).  All pairs are read before the first is stored: with loads and
+// 31 and 0).  Eight pairs are read before the first is stored: with loads and
 // stores alternating, which may alias as far as the compiler knows, a block took
-// about 4700 clocks.
-__device__ __forceinline__ void store_block_direct(const uint8_t* staging, int lane, int row0,
-                                                   int M, int col0, int N, uint16_t* Y) {
+// about 4700 clocks.  What is left is instructions, so the swizzled rows' addresses
+// are four registers and immediates, one load serves a pair (the next lane's comes
+// by shuffle) and rows past M are skipped by halves: with addresses formed per load,
+// two loads a pair and a divergent exit, a product of packed operands with 24 rows and
+// 111 columns took 9.4 us, 1357 x 1184 -> 1003 8.5 and 8192 x 1152 -> 3455 51.1; now
+// 6.9, 7.0 and 34.7 (stores by elements before that: 7.8 and 31.7).
+__device__ __forceinline__ void store_block_direct(uint32_t staging, int lane, int row0, int M,
+                                                   int col0, int N, uint16_t* Y) {
   const int ncol = min(EPI_COLS, N - col0);
-  const int p = lane & 15, q = (p + 1) & 15;  // this lane's pair and the next
-  const int r0 = row0 + (lane >> 4);
-  uint16_t* y = Y + static_cast<size_t>(r0) * N + col0;
+  const int rows = min(EPI_ROWS, M - row0);      // warp-uniform
+  const int p = lane & 15, h = lane >> 4;        // this lane's pair, of rows h, h + 2, ..
+  const int next = (lane & 16) | ((p + 1) & 15);  // the lane of the next pair
+  uint16_t* y = Y + static_cast<size_t>(row0 + h) * N + col0;
   const uint32_t odd0 = static_cast<uint32_t>(reinterpret_cast<uintptr_t>(y) >> 1) & 1u;
-  uint32_t w[EPI_ROWS / 2];
+  // row 2 i + h: its chunk c lies at (c ^ (i & 3)) << 4 (staged_chunk)
+  uint32_t at[4];
 #pragma unroll
-  for (int i = 0; i < EPI_ROWS / 2; ++i) {  // rows r0 + 2 i: the same parity for all i
-    const int r = 2 * i + (lane >> 4);
-    const uint32_t a =
-        *reinterpret_cast<const uint32_t*>(staging + staged_chunk(r, p >> 2) + (p & 3) * 4);
-    const uint32_t b =
-        *reinterpret_cast<const uint32_t*>(staging + staged_chunk(r, q >> 2) + (q & 3) * 4);
-    w[i] = __funnelshift_r(a, b, 16u * odd0);
-  }
+  for (int k = 0; k < 4; ++k) at[k] = staging + h * 64 + (((p >> 2) ^ k) << 4) + (p & 3) * 4;
   const int j = 2 * p + static_cast<int>(odd0);  // column of the low half
-  const bool both = j + 1 < ncol, low = j < ncol, first = odd0 != 0 && p == 15;
+  // rows 2 i + h < M whose pair is stored whole, in its low half, or in its high half
+  // (column 0 of a row that starts at an odd element)
+  const int both = j + 1 < ncol ? rows - h : 0;
+  const int low = j + 1 == ncol ? rows - h : 0;
+  const int first = odd0 != 0 && p == 15 ? rows - h : 0;
 #pragma unroll
-  for (int i = 0; i < EPI_ROWS / 2; ++i, y += 2 * static_cast<size_t>(N)) {
-    if (r0 + 2 * i >= M) break;
-    if (both)
-      *reinterpret_cast<uint32_t*>(y + j) = w[i];
-    else if (low)
-      y[j] = static_cast<uint16_t>(w[i]);
-    if (first) y[0] = static_cast<uint16_t>(w[i] >> 16);
+  for (int i0 = 0; i0 < EPI_ROWS / 2; i0 += 8) {  // rows 2 i + h: the same parity for all i
+    if (2 * i0 >= rows) break;
+    uint32_t w[8];
+#pragma unroll
+    for (int i = i0; i < i0 + 8; ++i) {
+      const uint32_t a = lds_u32(at[i & 3] + 128 * i);
+      w[i - i0] = __funnelshift_r(a, __shfl_sync(0xffffffffu, a, next), 16u * odd0);
+    }
+#pragma unroll
+    for (int i = i0; i < i0 + 8; ++i, y += 2 * static_cast<size_t>(N)) {
+      if (2 * i < both) *reinterpret_cast<uint32_t*>(y + j) = w[i - i0];
+      if (2 * i < low) y[j] = static_cast<uint16_t>(w[i - i0]);
+      if (2 * i < first) y[0] = static_cast<uint16_t>(w[i - i0] >> 16);
+    }
   }
 }
 
@@ -281,7 +298,7 @@ __device__ __forceinline__ void epilogue_part(uint32_t tmem_acc, int quarter, in
       }
     } else {
       __syncwarp();
-      store_block_direct(staging, lane, row0, M, n0 + c, N, static_cast<uint16_t*>(Y));
+      store_block_direct(stage_addr, lane, row0, M, n0 + c, N, static_cast<uint16_t*>(Y));
       __syncwarp();
     }
   }
