@@ -11,12 +11,12 @@
 // 8-bit codes (W4A8, W8A8) arrive as two E4M3 planes, 16 h and l with
 // q = 16 h + l.  W4A8 multiplies both activation planes into one
 // accumulator: every partial sum stays below 2^24 for K <= 16384 (at most
-// (128 + 8) * 7 per code pair), so it is exact too.  W8A8 keeps three
+// (128 + 8) * 7 per code pair), so it is exact too.  W8A8 keeps two or three
 // accumulators (SEP below) that are each exact and are added as integers.
 // E2M3 operands (F6) take the same MMA with 6-bit formats.
 //
-// Persistent: one CTA per SM walks 128 (M) x 256 (N) tiles, or a pair of CTAs
-// (CG 2, one cluster, tcgen05 cta_group::2) walks 256 x 256 tiles, in a static
+// Persistent: one CTA per SM walks 128 (M) x BNT (N) tiles, or a pair of CTAs
+// (CG 2, one cluster, tcgen05 cta_group::2) walks 256 x BNT tiles, in a static
 // round-robin order, K step 128 codes.  Each operand arrives either as E4M3
 // bytes, which TMA writes straight into the MMA operand buffer with the
 // 128-byte swizzle, or as packed nibbles (APACK / BPACK), which TMA stages and

@@ -10,8 +10,8 @@
 // Unclipped codes in an execution layout run the specialized loops where those
 // reach: rq_wide.cuh at b >= 64 (E4M3, E2M3, split planes, asymmetric codes),
 // rq_pair.cuh at b = 32 (symmetric E4M3 and E2M3).  This general loop serves every
-// other setting (packed codes, smaller blocks, clipped weights) and the fused
-// kernel.
+// other setting (packed codes, smaller blocks, clipped weights, few elements of short
+// rows) and the fused kernel.
 //
 // Every thread of the CTA takes part.  The CTA walks tiles of R rows.  Raw
 // rows stream into a ring of STAGES shared-memory buffers (STRIDE bytes

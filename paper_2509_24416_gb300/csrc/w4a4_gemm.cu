@@ -452,8 +452,8 @@ cudaError_t launch_w4a4_gemm(const uint8_t* Xq, int x_codes, const uint8_t* W, i
   const bool bpack = w_codes == CLQ_CODES_INT4_PACKED;
   const bool split = x_codes == CLQ_CODES_E4M3_SPLIT || w_codes == CLQ_CODES_E4M3_SPLIT;
   const bool w8a8 = x_codes == CLQ_CODES_E4M3_SPLIT && w_codes == CLQ_CODES_E4M3_SPLIT;
-  // Operands in an execution layout run on CTA pairs (tcgen05 cta_group::2): each
-  // CTA loads its 128 rows of A and half of B's rows, so a K step brings 32 KB
+  // Operands in an execution layout run on CTA pairs (tcgen05 cta_group::2) unless
+  // single_cta_wins: each CTA loads its 128 rows of A and half of B's rows, so a K step brings 32 KB
   // into an SM instead of 48, six stages fit instead of four, and the L2 reads
   // and power of a product fall with them (measured against single CTAs with
   // the same epilogue: 8192 x 3456 x 1152 26.8 -> 23.5 us, 4608 x 3072 x 12288
