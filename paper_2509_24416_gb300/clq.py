@@ -324,12 +324,13 @@ def _elsewhere(stream):
 def _with_stream(stream, fn, *args):
     """fn(*args) with `stream` current, so that the buffers it allocates come from that
     stream's pool: a block of the caller's stream could still be in use there, or be
-    handed out again, while kernels on `stream` work on it.  The results are recorded
+    handed out again, while kernels on `stream` work on it.  New results are recorded
     on the caller's stream, which may read and drop them."""
     here = torch.cuda.current_stream()
     with torch.cuda.stream(_torch_stream(stream)):
         out = fn(*args)
-    _record(out if isinstance(out, tuple) else (out,), here)
+    _record([t for t in (out if isinstance(out, tuple) else (out,))
+             if not any(t is a for a in args)], here)
     return out
 
 

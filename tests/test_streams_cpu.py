@@ -109,6 +109,17 @@ CALLS = {
 }
 
 
+def test_only_new_results_are_recorded(fake, monkeypatch):
+    recorded = []
+    monkeypatch.setattr(clq, "_record", lambda ts, s: recorded.extend((t, s.cuda_stream)
+                                                                      for t in ts))
+    Y = torch.zeros(M, N, dtype=torch.float16)
+    out, acc = clq.linear(Q, S, WE, SW, b, K, Y=Y, with_acc=True, stream=fake.side)
+    assert out is Y and len(recorded) == 1
+    assert recorded[0][0] is acc and recorded[0][1] == HERE
+    assert _layer()(X, stream=fake.side, Y=Y) is Y and len(recorded) == 1
+
+
 @pytest.mark.parametrize("name", sorted(CALLS))
 def test_buffers_belong_to_the_calls_stream(fake, name):
     CALLS[name](fake.side)
