@@ -15,9 +15,9 @@ struct MapSet {
   CUtensorMap A, B, Y, A2, B2;
 };
 
-// Tile shape of a launch: cg * 128 rows (a CTA or a CTA pair) x bn columns (256,
-// 192, 128 or 64 for execution-layout operands, 256 for packed ones, 128 or 64
-// for W8A8).
+// Tile shape of a launch: cg * 128 rows (a CTA or a CTA pair) x bn columns (pairs, for
+// execution-layout operands: 256, 192, 128 or 64, W8A8 128 or 64; single CTAs, for
+// those too and for packed ones: 256, W8A8 128).
 struct TileShape {
   int cg, bn;
 };

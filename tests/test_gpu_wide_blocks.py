@@ -3,7 +3,8 @@ asymmetric E4M3 codes, 8-bit split planes) against the general loop on the same
 rows, which writes packed nibbles (and, given clip bounds that never bind, 8-bit
 codes): both form every output by the same sums in the same order, so codes,
 scales, bounds and rotated rows agree bit for bit (a zero code may be written as
-either zero)."""
+either zero).  Few elements of short rows go to the general loop on both sides; the
+last test has enough of them."""
 import numpy as np
 import pytest
 import torch
